@@ -537,8 +537,7 @@ int run_device(sc_ctx* c, const float* cube, const int64_t* dims, const sc_kerne
   const bool share_on = !(flags & (SC_FLAG_NO_SHARE | SC_FLAG_GENERIC));
   bool share_cnt_clear = false;
   int p_owner = -1;  // pair whose spatial sums sh_P holds
-  for (int k = first_identity ? 1 : 0; k < nk; ++k) {
-    CK(cudaMemsetAsync(c->hist, 0, sizeof(unsigned long long) * kNumBins, s));
+  for (int k = first_identity ? 1 : 0; k < nk; ++k) {  // the histogram is clear: the last plan left it so
     SmoothArgs a = base_args(c, cube, dims, h16);
     a.pd = pds[k];
     a.pair = k;

@@ -287,7 +287,8 @@ cudaError_t launch_hist(const float* x, long long n, DevState* st, unsigned long
 // Histogram (and max) of a 16-bit cube, decoding it into out (if non-null).
 cudaError_t launch_hist16(const Half16& h, long long plane, long long n, DevState* st, unsigned long long* hist,
                           int win, int want_maxabs, float* out, int sms, cudaStream_t s);
-cudaError_t launch_plan(DevState* st, const unsigned long long* hist, int win, const float* src, long long n_total,
+// The plan of a measurement from the histogram, which it clears.
+cudaError_t launch_plan(DevState* st, unsigned long long* hist, int win, const float* src, long long n_total,
                         Lists L, float threshold, int clip, int std_mode, unsigned int force_flags, cudaStream_t s);
 cudaError_t launch_pass2(const float* src, long long n, uint32_t* mbits, DevState* st, Lists L, int sms,
                          cudaStream_t s);

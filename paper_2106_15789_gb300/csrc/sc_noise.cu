@@ -23,6 +23,8 @@
 // When a candidate set would exceed its buffer, the plan switches that part
 // to full passes over S (k_sel_* on the whole array, k_clip_full); results are
 // identical, only slower.
+#include <cooperative_groups.h>
+
 #include <atomic>
 #include <cfloat>
 #include <cstdio>
@@ -238,13 +240,13 @@ __device__ __forceinline__ unsigned int cell_class(unsigned int cell, const Nois
   return k;
 }
 
-// All threads of the block write the 64 KiB class table (one byte per cell).
-__device__ void fill_class_table(const NoisePlan& p, BinCfg cfg, unsigned char* cls) {
-  const bool live = !(p.flags & (PLAN_EMPTY | PLAN_STD));
-  const bool med = live && !(p.flags & PLAN_MED_FULL);
-  const bool mad = live && !(p.flags & PLAN_MAD_FULL);
-  const bool amb = live && (p.flags & PLAN_CLIP) && !(p.flags & PLAN_CLIP_FULL);
-  for (int i = threadIdx.x; i < kClsCells / 16; i += blockDim.x) {
+// Thread t of nt writes its share of the 64 KiB class table (one byte per cell).
+__device__ void fill_class_table(const NoisePlan& p, BinCfg cfg, unsigned char* cls, int t, int nt) {
+  if (p.flags & (PLAN_EMPTY | PLAN_STD)) return;  // the candidate pass returns before it reads the table
+  const bool med = !(p.flags & PLAN_MED_FULL);
+  const bool mad = !(p.flags & PLAN_MAD_FULL);
+  const bool amb = (p.flags & PLAN_CLIP) && !(p.flags & PLAN_CLIP_FULL);
+  for (int i = t; i < kClsCells / 16; i += nt) {
     unsigned int w[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -257,68 +259,11 @@ __device__ void fill_class_table(const NoisePlan& p, BinCfg cfg, unsigned char* 
   }
 }
 
-__device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long* cum, int win, const float* src,
-                                          long long n_total, Lists L, float threshold, int clip, int std_mode,
-                                          unsigned int force_flags);
-
-__global__ void __launch_bounds__(1024) k_plan(DevState* st, const unsigned long long* __restrict__ hist, int win,
-                                               const float* src, long long n_total, Lists L, float threshold,
-                                               int clip, int std_mode, unsigned int force_flags) {
-  extern __shared__ unsigned long long cum[];  // kNumBins + 1
-  __shared__ unsigned long long wsum[32];
-  const int tid = threadIdx.x;
-  constexpr int kPer = (kNumBins + 1023) / 1024;
-  unsigned long long loc[kPer];
-  unsigned long long s = 0;
-#pragma unroll
-  for (int j = 0; j < kPer; ++j) {
-    int b = tid * kPer + j;
-    loc[j] = b < kNumBins ? hist[b] : 0ull;
-    s += loc[j];
-  }
-  // block exclusive scan of s
-  unsigned long long incl = s;
-  for (int o = 1; o < 32; o <<= 1) {
-    unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
-    if ((tid & 31) >= o) incl += t;
-  }
-  if ((tid & 31) == 31) wsum[tid >> 5] = incl;
-  __syncthreads();
-  if (tid < 32) {
-    unsigned long long w = wsum[tid], wi = w;
-    for (int o = 1; o < 32; o <<= 1) {
-      unsigned long long t = __shfl_up_sync(0xffffffffu, wi, o);
-      if (tid >= o) wi += t;
-    }
-    wsum[tid] = wi - w;
-  }
-  __syncthreads();
-  unsigned long long run = wsum[tid >> 5] + incl - s;
-#pragma unroll
-  for (int j = 0; j < kPer; ++j) {
-    int b = tid * kPer + j;
-    if (b < kNumBins) cum[b] = run;
-    run += loc[j];
-  }
-  if (tid == 1023) cum[kNumBins] = run;
-  // reset counters and selection state
-  for (int i = tid; i < 3 * kSelBins; i += blockDim.x) {
-    (&st->sel_med.hist[0][0])[i] = 0ull;
-    (&st->sel_mad.hist[0][0])[i] = 0ull;
-  }
-  __syncthreads();
-  __shared__ NoisePlan s_plan;
-  if (tid == 0) s_plan = plan_of(st, cum, win, src, n_total, L, threshold, clip, std_mode, force_flags);
-  __syncthreads();
-  if (L.cls != nullptr) {
-    BinCfg cfg = kFullRange;
-    if (win) cfg = st->win;
-    fill_class_table(s_plan, cfg, L.cls);
-  }
-}
-
-// The plan proper (one thread). Returns the plan it stored in st->plan.
-__device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long* cum, int win, const float* src,
+// The plan proper (one thread): the median bins and the float bits of the
+// MAD's bracket (0xffffffff: no such bound) are given. Returns the plan it
+// stored in st->plan.
+__device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long* cum, BinCfg cfg, int b_med_lo,
+                                          int b_med_hi, unsigned int T1_bits, unsigned int T2_bits, const float* src,
                                           long long n_total, Lists L, float threshold, int clip, int std_mode,
                                           unsigned int force_flags) {
   NoisePlan p;
@@ -364,37 +309,19 @@ __device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long
   }
   p.k_lo = (n - 1ull) / 2ull;
   p.k_hi = n / 2ull;
-  // bins of the two middle order statistics
-  int lo = 0, hi = kNumBins - 1;
-  while (lo < hi) {  // first bin b with cum[b + 1] > k_lo
-    int mid = (lo + hi) >> 1;
-    if (cum[mid + 1] > p.k_lo) hi = mid; else lo = mid + 1;
-  }
-  p.b_med_lo = lo;
-  hi = kNumBins - 1;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (cum[mid + 1] > p.k_hi) hi = mid; else lo = mid + 1;
-  }
-  p.b_med_hi = lo;
+  p.b_med_lo = b_med_lo;
+  p.b_med_hi = b_med_hi;
   p.below_med = cum[p.b_med_lo];
   p.bound_med = cum[p.b_med_hi + 1] - cum[p.b_med_lo];
   if (p.bound_med > L.cap.med) p.flags |= PLAN_MED_FULL;
 
   if (!std_mode) {
-    const BinCfg cfg = win ? st->win : kFullRange;
-    PlanCtx P{cum, cfg, bin_lo_value(p.b_med_lo, cfg), bin_hi_value(p.b_med_hi, cfg)};
+    const PlanCtx P{cum, cfg, bin_lo_value(p.b_med_lo, cfg), bin_hi_value(p.b_med_hi, cfg)};
     if (!(isfinite(P.m_min) && isfinite(P.m_max))) {
       p.flags |= PLAN_MAD_FULL | PLAN_CLIP_FULL;
     } else {
-      // T1: largest T with possibly-within count <= k_lo (then MAD > T1)
-      if (f_possible(P, 0.0f) <= p.k_lo) {
-        unsigned int a = 0u, b = 0x7f800000u;
-        while (b - a > 1u) {
-          unsigned int mid = a + ((b - a) >> 1);
-          if (f_possible(P, __uint_as_float(mid)) <= p.k_lo) a = mid; else b = mid;
-        }
-        p.T1 = __uint_as_float(a);
+      if (T1_bits != 0xffffffffu) {
+        p.T1 = __uint_as_float(T1_bits);
         p.has_B = 1;
         p.B_lo = f_up(P.m_max - (double)p.T1);
         p.B_hi = f_down(P.m_min + (double)p.T1);
@@ -405,15 +332,8 @@ __device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long
           p.bB_hi = bin_of(p.B_hi, cfg) - 1;
         }
       }
-      // T2: smallest T with surely-within count >= k_hi + 1 (then MAD < T2)
-      const unsigned int fmax_bits = 0x7f7fffffu;
-      if (f_sure(P, __uint_as_float(fmax_bits)) >= p.k_hi + 1ull) {
-        unsigned int a = 0u, b = fmax_bits;
-        while (b - a > 1u) {
-          unsigned int mid = a + ((b - a) >> 1);
-          if (f_sure(P, __uint_as_float(mid)) >= p.k_hi + 1ull) b = mid; else a = mid;
-        }
-        p.T2 = __uint_as_float(b);
+      if (T2_bits != 0xffffffffu) {
+        p.T2 = __uint_as_float(T2_bits);
         p.A_lo = f_down(P.m_min - (double)p.T2);
         p.A_hi = f_up(P.m_max + (double)p.T2);
       }
@@ -456,11 +376,141 @@ __device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long
   return p;
 }
 
-cudaError_t launch_plan(DevState* st, const unsigned long long* hist, int win, const float* src, long long n_total,
+// Largest float-bit pattern a in [lo, hi) with pred(a), for a predicate that
+// holds at lo, fails at hi and changes once in between: a warp tests 32
+// patterns at a time (7 rounds over the 2^31 patterns of the non-negative
+// floats). All 32 lanes call it.
+template <class Pred>
+__device__ __forceinline__ unsigned int last_true(unsigned int lo, unsigned int hi, Pred pred) {
+  const unsigned int lane = threadIdx.x & 31u;
+  while (hi - lo > 1u) {
+    const unsigned int step = (hi - lo + 32u) / 33u;
+    const unsigned int off = step * (lane + 1u);
+    const bool in = off < hi - lo;
+    const unsigned int t = __ballot_sync(0xffffffffu, in && pred(lo + off));
+    const unsigned int k = (unsigned int)__popc(t);  // the first k patterns pass
+    hi = k < 32u ? min(hi, lo + step * (k + 1u)) : hi;
+    lo += step * k;
+  }
+  return lo;
+}
+
+// One cluster of kPlanCluster blocks. The first block scans the histogram (and
+// clears it for the next measurement), finds the median bins and the bracket
+// of the MAD and writes the plan; then all blocks write their share of the
+// class table and clear the selection's histograms.
+//
+// Latency-bound: one block with the plan proper on one thread took 40 us a
+// measurement whatever the cube's size (two bisections of 31 dependent steps
+// in float64, and 64 table cells a thread); with the bisections as 33-ary
+// searches by two warps and the table spread over eight SMs it takes 15 us.
+constexpr int kPlanCluster = 8;
+constexpr int kPlanThreads = 1024;
+__global__ void __cluster_dims__(kPlanCluster, 1, 1) __launch_bounds__(kPlanThreads)
+    k_plan(DevState* st, unsigned long long* __restrict__ hist, int win, const float* src, long long n_total, Lists L,
+           float threshold, int clip, int std_mode, unsigned int force_flags) {
+  namespace cg = cooperative_groups;
+  extern __shared__ unsigned long long cum[];  // kNumBins + 1
+  __shared__ unsigned long long wsum[32];
+  __shared__ NoisePlan s_plan;
+  __shared__ int s_bins[2];
+  __shared__ unsigned int s_T[2];
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank();
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const BinCfg cfg = win ? st->win : kFullRange;
+  if (rank == 0) {
+    for (int b = tid; b < kNumBins; b += kPlanThreads) {
+      cum[b] = hist[b];
+      hist[b] = 0ull;
+    }
+    if (tid == 0) {
+      s_bins[0] = s_bins[1] = 0;
+      s_T[0] = s_T[1] = 0xffffffffu;
+    }
+    __syncthreads();
+    constexpr int kPer = (kNumBins + kPlanThreads - 1) / kPlanThreads;
+    unsigned long long loc[kPer];
+    unsigned long long s = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      const int b = tid * kPer + j;
+      loc[j] = b < kNumBins ? cum[b] : 0ull;
+      s += loc[j];
+    }
+    // block exclusive scan of s
+    unsigned long long incl = s;
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
+      if ((tid & 31) >= o) incl += t;
+    }
+    if ((tid & 31) == 31) wsum[warp] = incl;
+    __syncthreads();
+    if (tid < 32) {
+      const unsigned long long w = wsum[tid];
+      unsigned long long wi = w;
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xffffffffu, wi, o);
+        if (tid >= o) wi += t;
+      }
+      wsum[tid] = wi - w;
+      if (tid == 31) cum[kNumBins] = wi;
+    }
+    __syncthreads();
+    const unsigned long long n = cum[kNumBins];
+    const unsigned long long k_lo = n ? (n - 1ull) / 2ull : 0ull, k_hi = n / 2ull;
+    unsigned long long run = wsum[warp] + incl - s;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      const int b = tid * kPer + j;
+      if (b < kNumBins) {
+        cum[b] = run;
+        // bins of the two middle order statistics
+        if (k_lo >= run && k_lo < run + loc[j]) s_bins[0] = b;
+        if (k_hi >= run && k_hi < run + loc[j]) s_bins[1] = b;
+      }
+      run += loc[j];
+    }
+    __syncthreads();
+    if (warp < 2 && n > 0ull && !std_mode) {
+      // MAD bracket: warp 0 T1, warp 1 T2 (0xffffffff: none)
+      const PlanCtx P{cum, cfg, bin_lo_value(s_bins[0], cfg), bin_hi_value(s_bins[1], cfg)};
+      if (isfinite(P.m_min) && isfinite(P.m_max)) {
+        unsigned int T = 0xffffffffu;
+        if (warp == 0) {
+          // T1: largest T with possibly-within count <= k_lo (then MAD > T1)
+          if (f_possible(P, 0.0f) <= k_lo)
+            T = last_true(0u, 0x7f800000u, [&](unsigned int b) { return f_possible(P, __uint_as_float(b)) <= k_lo; });
+        } else {
+          // T2: smallest T with surely-within count >= k_hi + 1 (then MAD < T2)
+          const unsigned int fmax_bits = 0x7f7fffffu;
+          if (f_sure(P, __uint_as_float(fmax_bits)) >= k_hi + 1ull)
+            T = 1u + last_true(0u, fmax_bits, [&](unsigned int b) { return f_sure(P, __uint_as_float(b)) < k_hi + 1ull; });
+        }
+        if ((tid & 31) == 0) s_T[warp] = T;
+      }
+    }
+    __syncthreads();
+    if (tid == 0)
+      s_plan = plan_of(st, cum, cfg, s_bins[0], s_bins[1], s_T[0], s_T[1], src, n_total, L, threshold, clip, std_mode,
+                       force_flags);
+  }
+  cl.sync();
+  if (rank != 0 && tid == 0) s_plan = *cl.map_shared_rank(&s_plan, 0);
+  cl.sync();  // every copy is taken (a block's shared memory stays until its readers are done)
+  const int t = rank * kPlanThreads + tid, nt = kPlanCluster * kPlanThreads;
+  for (int i = t; i < 3 * kSelBins; i += nt) {
+    (&st->sel_med.hist[0][0])[i] = 0ull;
+    (&st->sel_mad.hist[0][0])[i] = 0ull;
+  }
+  if (L.cls != nullptr) fill_class_table(s_plan, cfg, L.cls, t, nt);
+}
+
+cudaError_t launch_plan(DevState* st, unsigned long long* hist, int win, const float* src, long long n_total,
                         Lists L, float threshold, int clip, int std_mode, unsigned int force_flags,
                         cudaStream_t s) {
   const size_t smem = (kNumBins + 1) * sizeof(unsigned long long);
-  k_plan<<<1, 1024, smem, s>>>(st, hist, win, src, n_total, L, threshold, clip, std_mode, force_flags);
+  k_plan<<<kPlanCluster, kPlanThreads, smem, s>>>(st, hist, win, src, n_total, L, threshold, clip, std_mode, force_flags);
   return cudaGetLastError();
 }
 
@@ -1046,8 +1096,8 @@ __device__ void fx_setup(DevState* st, double repl_d, const PairWeights& W, int 
   if (mx == 0.0f) ex = 0;
   // f depends on the spatial kernel (through wf) but not on a spectral width up
   // to kShareMaxWz, so pairs with one spatial kernel quantise alike and can
-  // share their stored spatial sums.
-  for (int k = 0; k < n_pairs; ++k) {
+  // share their stored spatial sums. A thread per pair.
+  for (int k = threadIdx.x; k < n_pairs; k += blockDim.x) {
     const long long w = W.w[k];
     const int bits = 64 - __clzll((unsigned long long)(W.wf[k] - 1));  // bit length of wf - 1
     int f = 62 - ex - bits;
@@ -1061,15 +1111,15 @@ __device__ void fx_setup(DevState* st, double repl_d, const PairWeights& W, int 
 }
 
 __global__ void k_fx_setup(DevState* st, float repl_value, PairWeights W, int n_pairs) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
+  if (threadIdx.x == 0) {
     st->repl_d = (double)repl_value;
     st->repl = repl_value;
-    fx_setup(st, (double)repl_value, W, n_pairs);
   }
+  fx_setup(st, (double)repl_value, W, n_pairs);
 }
 
 cudaError_t launch_fx_setup(DevState* st, float repl_value, const PairWeights& W, int n_pairs, cudaStream_t s) {
-  k_fx_setup<<<1, 1, 0, s>>>(st, repl_value, W, n_pairs);
+  k_fx_setup<<<1, SC_MAX_KERNELS, 0, s>>>(st, repl_value, W, n_pairs);
   return cudaGetLastError();
 }
 
@@ -1161,19 +1211,21 @@ cudaError_t launch_window_from_sample(const float* x, const Half16* h16, long lo
 }
 
 __global__ void k_sigma0_done(DevState* st, float replacement, PairWeights W, int n_pairs) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const float s0 = st->sigma_cur;
-  st->sigma0 = s0;
-  st->repl_d = (replacement > 0.0f) ? (double)replacement * st->sigma_cur_d : 0.0;
-  st->repl = __double2float_rn(st->repl_d);
-  st->win = window_cfg(s0);
-  const float mx = fmaxf(__uint_as_float(st->maxabs_bits), st->repl);
-  if (s0 > 0.0f && mx > s0 * 1048576.0f) st->warn |= SC_WARN_RANGE;
-  fx_setup(st, st->repl_d, W, n_pairs);
+  const double repl_d = (replacement > 0.0f) ? (double)replacement * st->sigma_cur_d : 0.0;
+  if (threadIdx.x == 0) {
+    st->sigma0 = s0;
+    st->repl_d = repl_d;
+    st->repl = __double2float_rn(repl_d);
+    st->win = window_cfg(s0);
+    const float mx = fmaxf(__uint_as_float(st->maxabs_bits), st->repl);
+    if (s0 > 0.0f && mx > s0 * 1048576.0f) st->warn |= SC_WARN_RANGE;
+  }
+  fx_setup(st, repl_d, W, n_pairs);
 }
 
 cudaError_t launch_sigma0_done(DevState* st, float replacement, const PairWeights& W, int n_pairs, cudaStream_t s) {
-  k_sigma0_done<<<1, 1, 0, s>>>(st, replacement, W, n_pairs);
+  k_sigma0_done<<<1, SC_MAX_KERNELS, 0, s>>>(st, replacement, W, n_pairs);
   return cudaGetLastError();
 }
 
