@@ -268,9 +268,14 @@ int measure(sc_ctx* c, const float* src, long long n, int win, float t, int clip
       c->stats.launches += 3;
     } else {
       CK(launch_pass2(src, n, c->mbits, c->st, c->L, c->sms, s));
-      CK(launch_select(c->st, 0, -1, c->sms, s));
-      CK(launch_select(c->st, 1, pair, c->sms, s));
-      c->stats.launches += 11;
+      int launched = 0;
+      CK(launch_select_lists(c->st, src, n, c->L, pair, c->sms, s, &launched));
+      c->stats.launches += 1 + launched;
+      if (n > kSelectAllMax) {
+        CK(launch_select_full(c->st, 0, -1, c->sms, s));
+        CK(launch_select_full(c->st, 1, pair, c->sms, s));
+        c->stats.launches += 8;
+      }
     }
   }
   if (gauss) {
@@ -284,11 +289,7 @@ int measure(sc_ctx* c, const float* src, long long n, int win, float t, int clip
   }
   if (clip) {
     Phase ph(c, s, EV_CLIP);
-    if (!std_mode && !gauss) {
-      CK(launch_resolve(src, c->mbits, c->st, c->L, c->sms, s));
-      c->stats.launches += 1;
-    }
-    CK(launch_clip_full(src, n, c->mbits, c->st, c->sms, s));
+    CK(launch_clip(src, n, c->mbits, c->st, c->L, c->sms, s));
     c->stats.launches += 1;
   }
   return SC_OK;
@@ -483,7 +484,7 @@ int run_device(sc_ctx* c, const float* cube, const int64_t* dims, const sc_kerne
     W.w[k] = pds[k].W;
     W.wf[k] = pds[k].Wf;
   }
-  CK(cudaMemsetAsync(c->st, 0, sizeof(DevState), s));
+  CK(cudaMemsetAsync(c->st, 0, kDevStateHead, s));
   const long long nwords = (n + 31) / 32;
   const long long plane = dims[0] * dims[1];
   const bool direct = h16 && (flags & SC_FLAG_HALF_DIRECT);
@@ -647,7 +648,7 @@ int run_device(sc_ctx* c, const float* cube, const int64_t* dims, const sc_kerne
 
 int finish(sc_ctx* c, int nk, double* sigma_host, double* sigma0_host, cudaStream_t s, bool force_sync) {
   if (!sigma_host && !sigma0_host && !force_sync) return SC_OK;
-  CK(cudaMemcpyAsync(c->st_host, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(c->st_host, c->st, kDevStateHead, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   const DevState& h = *c->st_host;
   c->stats.warnings = h.warn;
@@ -1212,7 +1213,7 @@ int sc_autotune(sc_ctx* c, const int64_t* dims, const sc_kernel* kernels, int n_
     PairWeights W{};
     W.w[0] = pd.W;
     W.wf[0] = pd.Wf;
-    if (cudaMemsetAsync(c->st, 0, sizeof(DevState), s) != cudaSuccess ||
+    if (cudaMemsetAsync(c->st, 0, kDevStateHead, s) != cudaSuccess ||
         launch_maxabs(c->stage_cube, n, c->st, c->sms, s) != cudaSuccess ||
         launch_fx_setup(c->st, 1.0f, W, 1, s) != cudaSuccess) {
       out = cuda_fail(cudaGetLastError(), "autotune setup", __LINE__);
@@ -1450,7 +1451,7 @@ int sc_smooth(sc_ctx* c, const float* cube_dev, const int64_t* dims, sc_kernel k
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   c->last = s;
-  CK(cudaMemsetAsync(c->st, 0, sizeof(DevState), s));
+  CK(cudaMemsetAsync(c->st, 0, kDevStateHead, s));
   if (mask_dev) {
     CK(launch_pack(mask_dev, cube_dev, n, c->mbits, s));
     c->stats.launches += 1;
@@ -1531,13 +1532,13 @@ int sc_noise(sc_ctx* c, const float* data_dev, int64_t n, int noise_mode, double
   cudaStream_t s = (cudaStream_t)cuda_stream;
   c->last = s;
   const unsigned int force = (flags & SC_FLAG_NO_FAST_SELECT) ? (PLAN_MED_FULL | PLAN_MAD_FULL) : 0u;
-  CK(cudaMemsetAsync(c->st, 0, sizeof(DevState), s));
+  CK(cudaMemsetAsync(c->st, 0, kDevStateHead, s));
   CK(cudaMemsetAsync(c->hist, 0, sizeof(unsigned long long) * kNumBins, s));
   CK(launch_hist(data_dev, n, c->st, c->hist, 0, 0, c->sms, s));
   c->stats.launches += 1;
   int rc = measure(c, data_dev, n, 0, 1.0f, 0, noise_mode, SC_MAX_KERNELS, force, s);
   if (rc) return rc;
-  CK(cudaMemcpyAsync(c->st_host, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(c->st_host, c->st, kDevStateHead, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   rc = status_to_code(*c->st_host);
   *sigma_host = rc == SC_OK ? (double)c->st_host->sigma_cur : 0.0;

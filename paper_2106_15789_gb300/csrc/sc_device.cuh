@@ -35,6 +35,11 @@ __host__ __device__ __forceinline__ BinCfg window_cfg(float sigma0) {
   return BinCfg{e, kWindowE, kWindowMB};
 }
 
+// sigma from the MAD, rounded once to float. Monotone in mad, so the plan's
+// bounds on the MAD give bounds on sigma through the same function.
+constexpr double kMadToSigma = 1.4826;
+__device__ __forceinline__ float sigma_of_mad(double mad) { return __double2float_rn(kMadToSigma * mad); }
+
 // Histogram bin of a non-NaN float (monotone in the value): the magnitude's
 // top 9 + MB bits (exponent and MB mantissa bits), offset by the window base
 // and clamped to the underflow / overflow bins.

@@ -27,7 +27,6 @@ constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
 constexpr int kBins = 2048;
 constexpr unsigned kNone = 0xffffffffu;
-constexpr double kMadToSigma = 1.4826;
 
 struct Scratch {
   unsigned hist[kBins];

@@ -54,6 +54,7 @@ struct SelJob {
   unsigned long long c_le;        // elements with key <= key_lo
   unsigned int min_gt;            // smallest key > key_lo
   unsigned int key_lo;
+  unsigned int done;              // blocks through the successor pass
 };
 
 // ---------------------------------------------------------------------------
@@ -72,6 +73,7 @@ struct NoisePlan {
   unsigned long long k_lo, k_hi;  // median / MAD order statistics (0-based)
   unsigned long long below_med;   // values in bins below the median bins
   int b_med_lo, b_med_hi;         // bins holding the two middle values
+  BinCfg cfg;                     // bin layout of the histogram
   int flags;
   int has_B;
   float B_lo, B_hi;  // s in [B_lo, B_hi]  =>  |s - m| <= T1 < MAD for sure
@@ -83,6 +85,13 @@ struct NoisePlan {
   int bA_lo, bA_hi;        // bins that may hold MAD candidates
   int bB_lo, bB_hi;        // bins surely inside the MAD band (empty if bB_lo > bB_hi)
   unsigned long long n_B;  // values in those bins
+};
+
+// |s - m| in float32 for a median m: -m = h + l exactly, or m itself (wide).
+struct AbsDev {
+  double m;
+  float h, l;
+  int wide;
 };
 
 // Device-resident state of one sc_run (one context owns one).
@@ -103,14 +112,23 @@ struct DevState {
   // counters filled by the candidate pass
   unsigned long long n_cand_med, n_cand_mad, n_amb, n_below;
   NoisePlan plan;
-  SelJob sel_med, sel_mad;
+  AbsDev dev;  // of the current measurement's median
+  // the MAD's first round over a long list: keys under its range, the values
+  // of the picked digit (in the median's list when mad_short), their key range,
+  // the rank among them and the smallest key above them
+  unsigned int mad_below, n_mad_short, mad_rank, mad_klo, mad_khi, mad_next;
+  int mad_short;
   // fixed-point smoothing scale of every pair
   int fx_shift[SC_MAX_KERNELS];      // f: X_q = rint(X * 2^f)
   float fx_scale[SC_MAX_KERNELS];    // 2^f
   float fx_inv[SC_MAX_KERNELS];      // 2^-f / W (W = integer weight total of the pair)
   long long fx_qrepl[SC_MAX_KERNELS];  // rint(repl_d * 2^f): replaced voxels in fixed point
   float sigma[SC_MAX_KERNELS + 1];   // per pair; [SC_MAX_KERNELS] = scratch for sc_noise
+  alignas(16) unsigned int mad_digits[kSelBins];  // counts of that round
+  // selection by full passes (each plan sets both up)
+  SelJob sel_med, sel_mad;
 };
+constexpr size_t kDevStateHead = offsetof(DevState, mad_digits);  // what a run clears at its start and the host reads back
 
 enum StatusBits : unsigned int {
   SC_ST_ALLNAN = 1u,
@@ -292,11 +310,19 @@ cudaError_t launch_plan(DevState* st, unsigned long long* hist, int win, const f
                         Lists L, float threshold, int clip, int std_mode, unsigned int force_flags, cudaStream_t s);
 cudaError_t launch_pass2(const float* src, long long n, uint32_t* mbits, DevState* st, Lists L, int sms,
                          cudaStream_t s);
-// which: 0 median (result in DevState::m), 1 MAD (DevState::mad, sigma_cur, sigma[pair] if pair >= 0)
-cudaError_t launch_select(DevState* st, int which, int pair, int sms, cudaStream_t s);
-cudaError_t launch_resolve(const float* src, uint32_t* mbits, DevState* st, Lists L, int sms, cudaStream_t s);
-cudaError_t launch_clip_full(const float* src, long long n, uint32_t* mbits, DevState* st, int sms,
-                             cudaStream_t s);
+// Median and MAD (DevState::m, mad, sigma_cur, sigma[pair] if pair >= 0) from
+// the candidate lists (*launches: kernels launched). Arrays of more than
+// kSelectAllMax values whose plan asks for full passes are left to
+// launch_select_full (which does nothing otherwise; which: 0 median, 1 MAD).
+constexpr long long kSelectAllMax = 1LL << 21;
+constexpr long long kSelectGridMin = 1LL << 26;
+cudaError_t launch_select_lists(DevState* st, const float* src, long long n, Lists L, int pair, int sms,
+                                cudaStream_t s, int* launches);
+void init_select_attrs();
+cudaError_t launch_select_full(DevState* st, int which, int pair, int sms, cudaStream_t s);
+// The clip of the voxels that the candidate pass left undecided, or of all by a full pass.
+cudaError_t launch_clip(const float* src, long long n, uint32_t* mbits, DevState* st, Lists L, int sms,
+                        cudaStream_t s);
 cudaError_t launch_std(const float* src, long long n, DevState* st, int sms, cudaStream_t s);
 cudaError_t launch_std_final(DevState* st, int pair, cudaStream_t s);
 // Gaussian-fit noise (after the MAD measurement of the same array): the

@@ -17,12 +17,12 @@
 //               sets the mask bits that are certain whatever sigma is inside
 //               its bounds, and lists the few voxels whose clip is not yet
 //               decided.
-//   k_sel_*     exact radix selection (11+11+10 bits) of the wanted order
-//               statistics inside the candidate lists, then of |s - m|.
-//   k_resolve   decides the listed voxels with the exact sigma.
+//   k_select    (sc_select.cu) exact selection of the wanted order statistics
+//               inside the candidate lists, then of |s - m|.
+//   k_clip_full decides the listed voxels with the exact sigma.
 // When a candidate set would exceed its buffer, the plan switches that part
-// to full passes over S (k_sel_* on the whole array, k_clip_full); results are
-// identical, only slower.
+// to full passes over S (k_sel_*: radix selection of 11 + 11 + 10 bits on the
+// whole array; k_clip_full); results are identical, only slower.
 #include <cooperative_groups.h>
 
 #include <atomic>
@@ -33,12 +33,6 @@
 #include "sc_internal.h"
 
 namespace sc {
-
-constexpr double kMadToSigma = 1.4826;
-
-// sigma from the MAD, rounded once to float. Monotone in mad, so the plan's
-// bounds on the MAD give bounds on sigma through the same function.
-__device__ __forceinline__ float sigma_of_mad(double mad) { return __double2float_rn(kMadToSigma * mad); }
 
 // ---------------------------------------------------------------------------
 // Histogram (and max |x|) of the finite values of an array.
@@ -202,17 +196,18 @@ __device__ __forceinline__ unsigned long long cum_range(const PlanCtx& P, int b1
 __device__ __forceinline__ float f_down(double v) { return nextafterf(__double2float_rd(v), -INFINITY); }
 __device__ __forceinline__ float f_up(double v) { return nextafterf(__double2float_ru(v), INFINITY); }
 
-// Values that can possibly lie within T of some m in [m_min, m_max].
-__device__ unsigned long long f_possible(const PlanCtx& P, float T) {
-  float lo = f_down(P.m_min - (double)T), hi = f_up(P.m_max + (double)T);
-  return cum_range(P, bin_of(lo, P.cfg), bin_of(hi, P.cfg));
-}
-// Values that surely lie within T of every m in [m_min, m_max] (whole bins
-// strictly inside [m_max - T, m_min + T]).
-__device__ unsigned long long f_sure(const PlanCtx& P, float T) {
-  float lo = f_up(P.m_max - (double)T), hi = f_down(P.m_min + (double)T);
-  if (!(lo <= hi)) return 0ull;
-  return cum_range(P, bin_of(lo, P.cfg) + 1, bin_of(hi, P.cfg) - 1);
+// Number of values that can possibly lie within T of some m in [m_min, m_max],
+// or (sure) that surely lie within T of every one (whole bins strictly inside
+// [m_max - T, m_min + T]).
+__device__ __noinline__ unsigned long long within(const PlanCtx& P, float T, bool sure) {
+  // one float up for a sure count's lower end and a possible count's upper
+  // end, one down for the others
+  const double x = P.m_max + (sure ? -(double)T : (double)T), y = P.m_min + (sure ? (double)T : -(double)T);
+  const float up = f_up(x), down = f_down(y);
+  const float lo = sure ? up : down, hi = sure ? down : up;
+  if (sure && !(lo <= hi)) return 0ull;
+  const int e = sure ? 1 : 0;
+  return cum_range(P, bin_of(lo, P.cfg) + e, bin_of(hi, P.cfg) - e);
 }
 
 // Class of a 16-bit cell of the float encoding (sign, 8 exponent bits, top
@@ -246,16 +241,14 @@ __device__ void fill_class_table(const NoisePlan& p, BinCfg cfg, unsigned char* 
   const bool med = !(p.flags & PLAN_MED_FULL);
   const bool mad = !(p.flags & PLAN_MAD_FULL);
   const bool amb = (p.flags & PLAN_CLIP) && !(p.flags & PLAN_CLIP_FULL);
-  for (int i = t; i < kClsCells / 16; i += nt) {
-    unsigned int w[4];
+  // (four cells a step: every launch fetches this code once, and unrolled
+  // further it costs more to fetch than to run)
+#pragma unroll 1
+  for (int i = t; i < kClsCells / 4; i += nt) {
+    unsigned int x = 0u;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      unsigned int x = 0u;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) x |= cell_class((unsigned)(i * 16 + j * 4 + b), p, cfg, med, mad, amb) << (8 * b);
-      w[j] = x;
-    }
-    reinterpret_cast<uint4*>(cls)[i] = make_uint4(w[0], w[1], w[2], w[3]);
+    for (int b = 0; b < 4; ++b) x |= cell_class((unsigned)(i * 4 + b), p, cfg, med, mad, amb) << (8 * b);
+    reinterpret_cast<unsigned int*>(cls)[i] = x;
   }
 }
 
@@ -267,6 +260,7 @@ __device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long
                                           long long n_total, Lists L, float threshold, int clip, int std_mode,
                                           unsigned int force_flags) {
   NoisePlan p;
+  p.cfg = cfg;
   p.flags = (int)force_flags;
   p.threshold = threshold;
   p.has_B = 0;
@@ -296,6 +290,7 @@ __device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long
     J[w]->c_le = 0ull;
     J[w]->min_gt = 0xffffffffu;
     J[w]->key_lo = 0u;
+    J[w]->done = 0u;
     J[w]->count_fixed = 0ull;
     J[w]->count_ptr = nullptr;
     J[w]->list = src;
@@ -398,7 +393,8 @@ __device__ __forceinline__ unsigned int last_true(unsigned int lo, unsigned int 
 // One cluster of kPlanCluster blocks. The first block scans the histogram (and
 // clears it for the next measurement), finds the median bins and the bracket
 // of the MAD and writes the plan; then all blocks write their share of the
-// class table and clear the selection's histograms.
+// class table (and clear the histograms of full selection passes, where those
+// will run).
 //
 // Latency-bound: one block with the plan proper on one thread took 40 us a
 // measurement whatever the cube's size (two bisections of 31 dependent steps
@@ -476,17 +472,16 @@ __global__ void __cluster_dims__(kPlanCluster, 1, 1) __launch_bounds__(kPlanThre
       // MAD bracket: warp 0 T1, warp 1 T2 (0xffffffff: none)
       const PlanCtx P{cum, cfg, bin_lo_value(s_bins[0], cfg), bin_hi_value(s_bins[1], cfg)};
       if (isfinite(P.m_min) && isfinite(P.m_max)) {
+        // T1 (warp 0): the largest T with possibly-within count <= k_lo (then
+        // MAD > T1); T2 (warp 1): the smallest with surely-within count >=
+        // k_hi + 1 (then MAD < T2), one above the largest without
+        const bool t2 = warp == 1;
+        const unsigned int top = t2 ? 0x7f7fffffu : 0x7f800000u;
+        const auto under = [&](unsigned int b) {
+          return within(P, __uint_as_float(b), t2) <= (t2 ? k_hi : k_lo);
+        };
         unsigned int T = 0xffffffffu;
-        if (warp == 0) {
-          // T1: largest T with possibly-within count <= k_lo (then MAD > T1)
-          if (f_possible(P, 0.0f) <= k_lo)
-            T = last_true(0u, 0x7f800000u, [&](unsigned int b) { return f_possible(P, __uint_as_float(b)) <= k_lo; });
-        } else {
-          // T2: smallest T with surely-within count >= k_hi + 1 (then MAD < T2)
-          const unsigned int fmax_bits = 0x7f7fffffu;
-          if (f_sure(P, __uint_as_float(fmax_bits)) >= k_hi + 1ull)
-            T = 1u + last_true(0u, fmax_bits, [&](unsigned int b) { return f_sure(P, __uint_as_float(b)) < k_hi + 1ull; });
-        }
+        if (t2 ? !under(top) : under(0u)) T = last_true(0u, top, under) + (t2 ? 1u : 0u);
         if ((tid & 31) == 0) s_T[warp] = T;
       }
     }
@@ -499,9 +494,11 @@ __global__ void __cluster_dims__(kPlanCluster, 1, 1) __launch_bounds__(kPlanThre
   if (rank != 0 && tid == 0) s_plan = *cl.map_shared_rank(&s_plan, 0);
   cl.sync();  // every copy is taken (a block's shared memory stays until its readers are done)
   const int t = rank * kPlanThreads + tid, nt = kPlanCluster * kPlanThreads;
-  for (int i = t; i < 3 * kSelBins; i += nt) {
-    (&st->sel_med.hist[0][0])[i] = 0ull;
-    (&st->sel_mad.hist[0][0])[i] = 0ull;
+  if (s_plan.flags & (PLAN_MED_FULL | PLAN_MAD_FULL)) {
+    for (int i = t; i < 3 * kSelBins; i += nt) {
+      (&st->sel_med.hist[0][0])[i] = 0ull;
+      (&st->sel_mad.hist[0][0])[i] = 0ull;
+    }
   }
   if (L.cls != nullptr) fill_class_table(s_plan, cfg, L.cls, t, nt);
 }
@@ -781,11 +778,19 @@ __device__ __forceinline__ unsigned long long sel_rank0(const DevState* st, cons
   return r;
 }
 
+// The full passes serve measurements with a candidate set above capacity; the
+// others have been selected from their lists by k_select.
+__device__ __forceinline__ bool sel_by_full_passes(const NoisePlan& p) {
+  return !(p.flags & (PLAN_EMPTY | PLAN_STD)) && (p.flags & (PLAN_MED_FULL | PLAN_MAD_FULL));
+}
+
+__device__ void sel_result(DevState* st, SelJob* J, int which, int pair);
+
 __global__ void __launch_bounds__(256) k_sel_round(DevState* st, int which, int r) {
   __shared__ unsigned int sh[kSelBins];
   SelJob* J = which ? &st->sel_mad : &st->sel_med;
   const NoisePlan& p = st->plan;
-  if (p.flags & (PLAN_EMPTY | PLAN_STD)) return;
+  if (!sel_by_full_passes(p)) return;
   unsigned int prefix = 0u;
   unsigned long long rank = sel_rank0(st, J, which);
   const unsigned long long count = sel_count(*J);
@@ -843,14 +848,14 @@ __global__ void __launch_bounds__(256) k_sel_round(DevState* st, int which, int 
     if (sh[i]) atomicAdd(&J->hist[r][i], (unsigned long long)sh[i]);
 }
 
-__global__ void __launch_bounds__(256) k_sel_succ(DevState* st, int which) {
+__global__ void __launch_bounds__(256) k_sel_succ(DevState* st, int which, int pair) {
   __shared__ unsigned long long s_c[8];
   __shared__ unsigned int s_m[8];
   SelJob* J = which ? &st->sel_mad : &st->sel_med;
   const NoisePlan& p = st->plan;
-  if (p.flags & (PLAN_EMPTY | PLAN_STD)) return;
+  if (!sel_by_full_passes(p)) return;
   const unsigned long long count = sel_count(*J);
-  if (sel_rank0(st, J, which) >= count) return;
+  if (sel_rank0(st, J, which) >= count) return;  // (the first round has set the error)
   unsigned int prefix = J->prefix[2];
   unsigned long long rank = J->rank_in[2];
   sel_pick(J, 3, &prefix, &rank, &st->status);
@@ -884,24 +889,24 @@ __global__ void __launch_bounds__(256) k_sel_succ(DevState* st, int which) {
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { ct += s_c[w]; mt = min(mt, s_m[w]); }
     if (ct) atomicAdd(&J->c_le, ct);
     if (mt != 0xffffffffu) atomicMin(&J->min_gt, mt);
+    __threadfence();
+    // the last block to finish forms the result
+    if (atomicAdd(&J->done, 1u) == gridDim.x - 1u) {
+      __threadfence();
+      sel_result(st, J, which, pair);
+    }
   }
 }
 
-__global__ void k_sel_final(DevState* st, int which, int pair) {
-  SelJob* J = which ? &st->sel_mad : &st->sel_med;
+// (one thread, after every block's counts)
+__device__ void sel_result(DevState* st, SelJob* J, int which, int pair) {
   const NoisePlan& p = st->plan;
-  if (p.flags & (PLAN_EMPTY | PLAN_STD)) return;
-  const unsigned long long count = sel_count(*J);
-  const unsigned long long r_lo = sel_rank0(st, J, which);
-  if (r_lo >= count) {
-    atomicOr(&st->status, (unsigned int)SC_ST_INTERNAL);
-    return;
-  }
-  const unsigned long long r_hi = r_lo + (p.k_hi - p.k_lo);
-  const unsigned int k_lo = J->key_lo;
+  const unsigned long long r_hi = sel_rank0(st, J, which) + (p.k_hi - p.k_lo);
+  const unsigned long long c_le = *(volatile unsigned long long*)&J->c_le;
+  const unsigned int k_lo = *(volatile unsigned int*)&J->key_lo;
   unsigned int k_hi = k_lo;
-  if (r_hi >= J->c_le) {
-    k_hi = J->min_gt;
+  if (r_hi >= c_le) {
+    k_hi = *(volatile unsigned int*)&J->min_gt;
     if (k_hi == 0xffffffffu) {
       atomicOr(&st->status, (unsigned int)SC_ST_INTERNAL);
       k_hi = k_lo;
@@ -921,15 +926,14 @@ __global__ void k_sel_final(DevState* st, int which, int pair) {
   }
 }
 
-cudaError_t launch_select(DevState* st, int which, int pair, int sms, cudaStream_t s) {
+cudaError_t launch_select_full(DevState* st, int which, int pair, int sms, cudaStream_t s) {
   const int grid = 2 * sms;
   for (int r = 0; r < 3; ++r) {
     k_sel_round<<<grid, 256, 0, s>>>(st, which, r);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  k_sel_succ<<<grid, 256, 0, s>>>(st, which);
-  k_sel_final<<<1, 1, 0, s>>>(st, which, pair);
+  k_sel_succ<<<grid, 256, 0, s>>>(st, which, pair);
   return cudaGetLastError();
 }
 
@@ -998,24 +1002,16 @@ cudaError_t launch_std_final(DevState* st, int pair, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------------------
-// Clip: the undecided voxels, or a full pass when the plan asked for one.
-__global__ void k_resolve(const float* __restrict__ src, uint32_t* mbits, DevState* st, Lists L) {
-  const NoisePlan& p = st->plan;
-  if (!(p.flags & PLAN_CLIP) || (p.flags & (PLAN_CLIP_FULL | PLAN_EMPTY))) return;
-  const float sg = st->sigma_cur;
-  if (!(sg > 0.0f)) return;
-  const float thr = __fmul_rn(p.threshold, sg);
+// Clip: the voxels that the candidate pass left undecided, or all of them when
+// the plan asked for a full pass.
+__device__ void clip_listed(const float* __restrict__ src, uint32_t* mbits, const DevState* st, const Lists& L,
+                            float thr) {
   const unsigned long long na = min(st->n_amb, L.cap.amb);
   for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < na;
        i += (unsigned long long)gridDim.x * blockDim.x) {
     const unsigned long long v = L.amb[i];
     if (fabsf(__ldg(src + v)) > thr) atomicOr(mbits + (v >> 5), 1u << (v & 31ull));
   }
-}
-
-cudaError_t launch_resolve(const float* src, uint32_t* mbits, DevState* st, Lists L, int sms, cudaStream_t s) {
-  k_resolve<<<sms, 256, 0, s>>>(src, mbits, st, L);
-  return cudaGetLastError();
 }
 
 // resident k_clip_full blocks per SM (init_noise_attrs, which every context
@@ -1050,12 +1046,16 @@ __device__ __forceinline__ void clip_store(uint32_t* mbits, long long ch, int la
 }
 
 __global__ void __launch_bounds__(256) k_clip_full(const float* __restrict__ src, long long n, uint32_t* mbits,
-                                                   DevState* st) {
+                                                   DevState* st, Lists L) {
   const NoisePlan& p = st->plan;
-  if (!(p.flags & PLAN_CLIP) || !(p.flags & PLAN_CLIP_FULL) || (p.flags & PLAN_EMPTY)) return;
+  if (!(p.flags & PLAN_CLIP) || (p.flags & PLAN_EMPTY)) return;
   const float sg = st->sigma_cur;
   if (!(sg > 0.0f)) return;
   const float thr = __fmul_rn(p.threshold, sg);
+  if (!(p.flags & PLAN_CLIP_FULL)) {
+    clip_listed(src, mbits, st, L, thr);
+    return;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long nchunks = (n + 127) / 128;
   const long long stride = (long long)gridDim.x * 8;
@@ -1070,15 +1070,15 @@ __global__ void __launch_bounds__(256) k_clip_full(const float* __restrict__ src
   }
 }
 
-cudaError_t launch_clip_full(const float* src, long long n, uint32_t* mbits, DevState* st, int sms,
-                             cudaStream_t s) {
+cudaError_t launch_clip(const float* src, long long n, uint32_t* mbits, DevState* st, Lists L, int sms,
+                        cudaStream_t s) {
   // one wave: as many blocks as are resident at once (a second, partial wave
   // would run on a fraction of the SMs)
   const int per_sm = g_clip_blocks_per_sm.load(std::memory_order_relaxed);
   const long long cap = (long long)(per_sm > 0 ? per_sm : 4) * sms;
   long long want = (n + 1023) / 1024;
   int grid = (int)(want < 1 ? 1 : (want > cap ? cap : want));
-  k_clip_full<<<grid, 256, 0, s>>>(src, n, mbits, st);
+  k_clip_full<<<grid, 256, 0, s>>>(src, n, mbits, st, L);
   return cudaGetLastError();
 }
 

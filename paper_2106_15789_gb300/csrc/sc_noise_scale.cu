@@ -30,7 +30,6 @@ constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
 constexpr int kBins = 2048;              // radix digits: 11, 11 and 10 bits
 constexpr unsigned kNone = 0xffffffffu;  // key of a non-finite voxel: above every finite key
-constexpr double kMadToSigma = 1.4826;
 constexpr int kCandCap = 6144;  // keys of one round-0 bin copied aside for the later rounds
 
 struct Geo {

@@ -371,6 +371,7 @@ void init_kernel_attrs() {
   init_z_attrs();
   init_share_attrs();
   init_noise_attrs();
+  init_select_attrs();
   init_noise_scale_attrs();
 }
 

@@ -94,7 +94,7 @@ extern "C" int sc_noise_static(const float* data_dev, int64_t n, int noise_mode,
   L.cap = Caps{kStaticCapMed, kStaticCapMad, 0ull};
   const int std_mode = (noise_mode == SC_NOISE_STD);
   // the previous call's contents stay in the array: clear state and histogram
-  CKS(cudaMemsetAsync(st, 0, sizeof(DevState), s));
+  CKS(cudaMemsetAsync(st, 0, kDevStateHead, s));
   CKS(cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * kNumBins, s));
   CKS(launch_hist(data_dev, n, st, hist, 0, 0, sms, s));
   CKS(launch_plan(st, hist, 0, data_dev, n, L, 1.0f, 0, std_mode, 0u, s));
@@ -103,8 +103,12 @@ extern "C" int sc_noise_static(const float* data_dev, int64_t n, int noise_mode,
     CKS(launch_std_final(st, SC_MAX_KERNELS, s));
   } else {
     CKS(launch_pass2(data_dev, n, nullptr, st, L, sms, s));
-    CKS(launch_select(st, 0, -1, sms, s));
-    CKS(launch_select(st, 1, SC_MAX_KERNELS, sms, s));
+    int launched = 0;
+    CKS(launch_select_lists(st, data_dev, n, L, SC_MAX_KERNELS, sms, s, &launched));
+    if (n > kSelectAllMax) {
+      CKS(launch_select_full(st, 0, -1, sms, s));
+      CKS(launch_select_full(st, 1, SC_MAX_KERNELS, sms, s));
+    }
   }
   if (noise_mode == SC_NOISE_GAUSS) {
     unsigned long long* ghist = reinterpret_cast<unsigned long long*>(base + kOffGHist);
