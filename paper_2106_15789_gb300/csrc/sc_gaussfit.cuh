@@ -142,6 +142,22 @@ __device__ double fit_tau(const double (&hh)[PER], const double (&x2)[PER], cons
   return tau;
 }
 
+// The fit of a 256-bin histogram by one warp (four folded bins a lane). A
+// function of its own, so that its float64 registers stay out of the callers.
+static __device__ __noinline__ double fit_tau_warp(const unsigned* counts) {
+  const int lane = threadIdx.x & 31;
+  double hh[4], x2[4];
+  bool use[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int t = lane + 32 * j;
+    hh[j] = (double)counts[kHalf + t] + (double)counts[kHalf - 1 - t];
+    x2[j] = xi2_of(t);
+    use[j] = true;
+  }
+  return fit_tau(hh, x2, use, WarpSum6{});
+}
+
 // The noise from tau and the scale k.
 __device__ __forceinline__ double noise_of(double tau, float k) { return tau * (double)kHalf / (double)k; }
 

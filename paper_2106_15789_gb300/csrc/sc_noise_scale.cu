@@ -2,21 +2,36 @@
 // channels in the speed test of Sect. 5): the cube is divided by the noise
 // level measured in a window around each voxel's cell.
 //
-//   k_noise_window  one block per cell (persistent over cells): the finite
-//                   voxels of the cell's window, clipped to the cube, go into
-//                   shared memory as order-preserving keys; the noise of the
-//                   chosen mode comes from them: MAD by two exact radix
-//                   selections in shared memory (the median, then the median
-//                   of the float32 keys |x - m|, rounded correctly for an odd
-//                   count and faithfully for an even one), STD by two passes
-//                   of compensated float32 sums combined in double. Writes
-//                   the cell's noise (double) and the float32 reciprocal used
-//                   below.
+//   k_noise_window  one block per cell (persistent over cells): the noise of
+//                   the chosen mode over the finite voxels of the cell's
+//                   window, clipped to the cube, which is streamed from
+//                   memory: MAD by two exact selections (the median, then the
+//                   median of the float32 values |x - m|, rounded correctly
+//                   for an odd count and faithfully for an even one), STD by
+//                   two passes of compensated float32 sums combined in double.
+//                   Writes the cell's noise (double) and the float32
+//                   reciprocal used below.
 //   k_noise_apply   out = in * (1 / sigma) per voxel (NaN where the input is
 //                   not finite or the cell has no positive noise).
 //
 // Cells are gx x gy x gz voxels (the last one along an axis may be shorter);
 // a cell's window is centred on voxel start + (extent - 1) / 2 of each axis.
+//
+// A selection takes one pass over the window: a sample of it (every 8th voxel
+// of a row, kept in shared memory) brackets the wanted rank, the pass counts
+// the values under the bracket and copies those inside it, and the rank is
+// found among the copies by one histogram of 2048 equal steps of the bracket
+// and a direct ranking inside one step. A bracket that misses its rank, or
+// holds more values than the copies' room, costs radix passes over the window
+// instead, so the result is exact whatever the data.
+//
+// What bounds it: instruction issue of the two passes; the 7 windows that share a voxel read it from L2. Blocks of
+// 256 threads, four to an SM, hide each other's barriers and loads. On 360 x
+// 360 x 1464 voxels (48,668 windows of 31^3) the earlier form, one block of
+// 1,024 threads per SM with the window in shared memory, warp-aggregated
+// (match_any) histograms and up to 40 barriers a window on nothing else, took
+// 16.9 ms; this one 6.4 ms.
+#include <cfloat>
 #include <cstdint>
 
 #include "sc_device.cuh"
@@ -26,11 +41,16 @@
 namespace sc {
 namespace nscale {
 
-constexpr int kThreads = 1024;
+constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kBins = 2048;              // radix digits: 11, 11 and 10 bits
-constexpr unsigned kNone = 0xffffffffu;  // key of a non-finite voxel: above every finite key
-constexpr int kCandCap = 6144;  // keys of one round-0 bin copied aside for the later rounds
+constexpr int kBlocksPerSm = 4;
+constexpr int kBins = 2048;              // steps of a bracket; radix digits of 11, 11 and 10 bits
+constexpr unsigned kNone = 0xffffffffu;  // above the key of every finite value
+constexpr int kSegCap = 640;             // copies each warp keeps of the values in a bracket
+constexpr int kCandCap = kSegCap * kWarps;
+constexpr int kSampleCap = 4096;
+constexpr int kUnroll = 8;               // loads in flight per thread
+constexpr int kFewCap = 256;             // copies ranked directly
 
 struct Geo {
   long long nx, ny, nz;
@@ -49,238 +69,290 @@ __device__ __forceinline__ void window_range(int c, int g, int w, long long n, l
   *hi = min(centre + r + 1, n);
 }
 
-// Inclusive block scan of one value per thread; returns the block total in
-// *total. Uses part[kWarps] of shared scratch (two barriers).
-__device__ __forceinline__ unsigned block_scan_incl(unsigned v, unsigned* part, unsigned* total) {
+struct Scratch {
+  float cand[kCandCap];       // per warp kSegCap copies
+  float sample[kSampleCap];   // NaN: no finite voxel
+  alignas(16) unsigned hist[kBins];
+  float few[kFewCap];
+  unsigned part[kWarps];
+  unsigned seg[kWarps];       // copies each warp wanted to make (may exceed kSegCap)
+  unsigned digit[2], rank[2], n_few, next, finite, below, n_sample;
+  float v1;
+  double dpart[kWarps + 1];
+};
+
+// A window: voxel (x, y, z) at base + z plane + y nx + x. A row goes to a
+// group of 2^lw lanes (the smallest power of two that covers it, up to 32), a
+// plane's rows to 2^wy of the block's warps, in turns, and its planes to the
+// 8 / 2^wy sets of warps that leaves.
+struct Win {
+  const float* base;
+  long long plane, nx;
+  int lx, ly, lz, lw, wy;
+  __device__ __forceinline__ void split() {
+    lw = lx > 16 ? 5 : (lx > 8 ? 4 : (lx > 4 ? 3 : 2));
+    const int need = (ly + (32 >> lw) - 1) >> (5 - lw);
+    wy = need > 4 ? 3 : (need > 2 ? 2 : (need > 1 ? 1 : 0));
+  }
+  __device__ __forceinline__ int step() const { return 1 << (wy + 5 - lw); }  // rows of a turn
+  __device__ __forceinline__ int turns() const { return (ly + step() - 1) / step(); }
+  __device__ __forceinline__ int sets() const { return kWarps >> wy; }
+  // Most voxels one warp takes.
+  __device__ __forceinline__ int share() const { return turns() * (32 >> lw) * ((lz + sets() - 1) / sets()) * lx; }
+};
+
+// f(v) for every voxel v of the window, NaN in the lanes left over; all lanes
+// of a warp call f together, kUnroll loads ahead. The turn and the plane are
+// the same for all lanes, so a lane adds its own fixed offset to an address
+// that a warp shares.
+template <class F>
+__device__ __forceinline__ void for_window(const Win& w, F f) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned x = v;
+  const int group = 1 << w.lw, step = w.step(), turns = w.turns(), sets = w.sets();
+  const int y0 = ((warp & ((1 << w.wy) - 1)) << (5 - w.lw)) + (lane >> w.lw), z0 = warp >> w.wy;
+  const int total = z0 < w.lz ? turns * ((w.lz - z0 + sets - 1) / sets) : 0;
+  const long long turn = step * w.nx, wrap = sets * w.plane - turns * turn;
+  for (int x0 = 0; x0 < w.lx; x0 += group) {
+    const int dx = x0 + (lane & (group - 1));
+    const int rows = dx < w.lx ? w.ly - y0 : 0;  // rows left from the lane's first one on
+    const float* const mine = w.base + z0 * w.plane + y0 * w.nx + dx;
+    long long at = 0;
+    int k = 0;
+    for (int t0 = 0; t0 < total; t0 += kUnroll) {
+      float v[kUnroll];
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        v[u] = __int_as_float(0x7fc00000);
+        if (k * step < rows && t0 + u < total) v[u] = __ldg(mine + at);
+        at += turn;
+        if (++k == turns) {
+          k = 0;
+          at += wrap;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) f(v[u]);
+    }
+  }
+}
+
+// Clears the histogram (a barrier follows before it is counted into).
+__device__ __forceinline__ void clear_hist(Scratch* S) {
+  uint4* h = reinterpret_cast<uint4*>(S->hist);
+  h[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
+  h[threadIdx.x + kThreads] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// The digits whose cumulative ranges in S->hist hold ranks ra and rb, and the
+// ranks within them (S->digit, S->rank). Barriers before and after.
+__device__ __forceinline__ void find_digits(Scratch* S, unsigned ra, unsigned rb) {
+  static_assert(kBins == 8 * kThreads, "eight digits per thread");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __syncthreads();
+  unsigned c[8], sum = 0u;
+  const uint4 h0 = reinterpret_cast<const uint4*>(S->hist)[2 * tid], h1 = reinterpret_cast<const uint4*>(S->hist)[2 * tid + 1];
+  c[0] = h0.x, c[1] = h0.y, c[2] = h0.z, c[3] = h0.w, c[4] = h1.x, c[5] = h1.y, c[6] = h1.z, c[7] = h1.w;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) sum += c[j];
+  unsigned x = sum;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned t = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += t;
   }
-  if (lane == 31) part[warp] = x;
+  if (lane == 31) S->part[warp] = x;
   __syncthreads();
-  if (warp == 0) {
-    unsigned w = part[lane], wi = w;
+  unsigned run = x - sum;
+  for (int k = 0; k < warp; ++k) run += S->part[k];
+  if (ra < run + sum && rb >= run) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned t = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += t;
+    for (int j = 0; j < 8; ++j) {
+      if (ra >= run && ra < run + c[j]) {
+        S->digit[0] = 8u * tid + j;
+        S->rank[0] = ra - run;
+      }
+      if (rb >= run && rb < run + c[j]) {
+        S->digit[1] = 8u * tid + j;
+        S->rank[1] = rb - run;
+      }
+      run += c[j];
     }
-    part[lane] = wi - w;  // exclusive prefix of the warps
-    if (lane == 31) part[32] = wi;
   }
   __syncthreads();
-  *total = part[32];
-  return part[warp] + x;
 }
 
-struct SelScratch {
-  unsigned hist[kBins];
-  unsigned part[kWarps + 1];
-  unsigned digit, rank, next, count, below;
+// The MAD value of x: the float of |x - m| with m = (a + b) / 2 (a == b for an
+// odd count: one correctly rounded subtraction). For an even count, x - a/2
+// and then - b/2 are taken exactly as sums of two floats and added back, which
+// rounds the exact difference faithfully (within one unit in the last place)
+// in single precision, without the slow FP64 pipe.
+__device__ __forceinline__ float two_diff(float x, float b, float* err) {
+  const float s = __fsub_rn(x, b);
+  const float bb = __fsub_rn(s, x);
+  *err = __fadd_rn(__fsub_rn(x, __fsub_rn(s, bb)), __fsub_rn(-b, bb));
+  return s;
+}
+struct AbsDev {
+  float a, b;
+  bool even;
+  __device__ __forceinline__ float operator()(float x) const {
+    if (!even) return fabsf(__fsub_rn(x, a));
+    float e1, e2;
+    const float t = two_diff(x, 0.5f * a, &e1);
+    const float u = two_diff(t, 0.5f * b, &e2);
+    return fabsf(__fadd_rn(u, __fadd_rn(e1, e2)));
+  }
+};
+struct Value {
+  __device__ __forceinline__ float operator()(float x) const { return x; }
 };
 
-// Adds this lane's digit to a histogram; lanes of the warp with the same digit
-// add once. bin == kBins: nothing to add. All 32 lanes must call it.
-__device__ __forceinline__ void hist_add_warp(unsigned* hist, unsigned bin) {
-  const unsigned peers = __match_any_sync(0xffffffffu, bin);
-  if ((threadIdx.x & 31) == __ffs(peers) - 1 && bin < (unsigned)kBins) atomicAdd(&hist[bin], __popc(peers));
-}
-
-// Appends k to out[] (at most cap entries) where `take`; the counter ends as
-// the number of takers, which may exceed cap. All 32 lanes must call it.
-__device__ __forceinline__ void append_warp(bool take, unsigned k, unsigned* out, unsigned cap, unsigned* counter) {
-  const unsigned ball = __ballot_sync(0xffffffffu, take);
-  if (ball) {
-    const int lane = threadIdx.x & 31;
-    unsigned off = 0u;
-    if (lane == 0) off = atomicAdd(counter, (unsigned)__popc(ball));
-    off = __shfl_sync(0xffffffffu, off, 0);
-    const unsigned pos = off + (unsigned)__popc(ball & ((1u << lane) - 1u));
-    if (take && pos < cap) out[pos] = k;
-  }
-}
-
-// The digit whose cumulative range in S->hist holds `rank`, and the rank
-// within it (S->digit, S->rank; the histogram is left intact).
-__device__ __forceinline__ void find_digit(SelScratch* S, unsigned rank) {
+// Order statistics r and (want_next) r + 1 of of(x) over the finite voxels x of
+// the window, by radix passes over it (digits of 11, 11 and 10 bits).
+template <class Of>
+__device__ __noinline__ void select_window(const Win& w, Of of, unsigned r, bool want_next, Scratch* S, float* v1,
+                                           float* v2) {
   const int tid = threadIdx.x;
-  const unsigned a = S->hist[2 * tid], b = S->hist[2 * tid + 1];
-  unsigned total;
-  const unsigned incl = block_scan_incl(a + b, S->part, &total);
-  const unsigned excl = incl - a - b;
-  if (rank >= excl && rank < excl + a) {
-    S->digit = 2u * tid;
-    S->rank = rank - excl;
-  } else if (rank >= excl + a && rank < incl) {
-    S->digit = 2u * tid + 1u;
-    S->rank = rank - excl - a;
-  }
-  __syncthreads();
-}
-
-// Exact radix selection (digits of 11, 11 and 10 bits, counted in a shared
-// histogram with warp-aggregated additions) of order statistic `rank` among
-// the m keys of src (all below kNone). With want_next, *next is the key of
-// order statistic rank + 1 of src, or kNone when rank is its last. All
-// threads of the block call it.
-__device__ unsigned select_keys(const unsigned* src, int m, unsigned rank, SelScratch* S, bool want_next,
-                                unsigned* next) {
-  const int tid = threadIdx.x, lane = tid & 31;
   unsigned prefix = 0u, pmask = 0u;
   for (int round = 0; round < 3; ++round) {
     const int shift = round == 0 ? 21 : (round == 1 ? 10 : 0);
     const unsigned dmask = round == 2 ? 0x3ffu : 0x7ffu;
-    for (int i = tid; i < kBins; i += kThreads) S->hist[i] = 0u;
     __syncthreads();
-    for (int base = tid - lane; base < m; base += kThreads) {
-      const int e = base + lane;
-      const unsigned k = e < m ? src[e] : kNone;
-      hist_add_warp(S->hist, (e < m && (k & pmask) == prefix) ? (k >> shift) & dmask : (unsigned)kBins);
-    }
+    clear_hist(S);
     __syncthreads();
-    find_digit(S, rank);
-    const unsigned d = S->digit;
-    rank = S->rank;
+    for_window(w, [&](float v) {
+      const unsigned k = isfinite(v) ? fkey(of(v)) : kNone;
+      const bool in = k != kNone && (k & pmask) == prefix;
+      const unsigned d = in ? (k >> shift) & dmask : kNone;
+      const unsigned d0 = __shfl_sync(0xffffffffu, d, 0);  // ties are added at once
+      if (__all_sync(0xffffffffu, d == d0)) {
+        if ((threadIdx.x & 31) == 0 && d != kNone) atomicAdd(&S->hist[d], 32u);
+      } else if (d != kNone) {
+        atomicAdd(&S->hist[d], 1u);
+      }
+    });
+    find_digits(S, r, r);
+    r = S->rank[0];
+    const unsigned d = S->digit[0];
     prefix |= d << shift;
     pmask |= dmask << shift;
-    if (round == 2 && want_next) {
-      // the successor: the same key if it occurs again, else the next
-      // non-empty bin of this round, else the smallest larger key of src
-      if (tid == 0) S->next = (rank + 1u < S->hist[d]) ? prefix : kNone;
-      __syncthreads();
-      if (S->next == kNone) {
-        for (int i = (int)d + 1 + tid; i < 1024; i += kThreads)
-          if (S->hist[i] != 0u) atomicMin(&S->next, (prefix & ~dmask) | (unsigned)i);
-        __syncthreads();
-        if (S->next == kNone) {
-          for (int e = tid; e < m; e += kThreads) {
-            const unsigned k = src[e];
-            if (k > prefix) atomicMin(&S->next, k);
-          }
-          __syncthreads();
-        }
-      }
-      *next = S->next;
-    }
-    __syncthreads();
-  }
-  return prefix;
-}
-
-constexpr int kSampleStride = 8;  // every 8th voxel of the window is sampled for the bracket
-
-// Order statistics r and (with want_next) r + 1 of key_of(k) over the finite
-// keys k of keys[0 .. n) (nf of them). A sample of the window brackets the
-// rank: the keys inside the bracket are copied into cand in one counting
-// pass and selected there; when the bracket misses (or overflows cand), or
-// the window is small, the selection runs over all keys. When `rewrite`, the
-// keys are replaced by key_of(k) if the full selection is needed (the caller
-// needs them no more).
-template <class KeyOf>
-__device__ bool select_order(unsigned* keys, int n, unsigned nf, unsigned r, bool want_next, KeyOf key_of,
-                             bool rewrite, unsigned* cand, SelScratch* S, unsigned* k1, unsigned* k2) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  unsigned nx = kNone;
-  if (nf <= (unsigned)kCandCap) {  // small window: select over a copy of all finite keys
-    if (tid == 0) S->count = 0u;
-    __syncthreads();
-    for (int base = tid - lane; base < n; base += kThreads) {
-      const int e = base + lane;
-      const unsigned k = e < n ? keys[e] : kNone;
-      append_warp(k != kNone, k != kNone ? key_of(k) : kNone, cand, kCandCap, &S->count);
-    }
-    __syncthreads();
-    *k1 = select_keys(cand, (int)nf, r, S, want_next, &nx);
-    *k2 = nx;
-    __syncthreads();
-    return false;  // the keys are as they were
-  }
-  // sample every kSampleStride-th voxel
-  if (tid == 0) S->count = 0u;
-  __syncthreads();
-  for (int j0 = tid - lane; j0 * kSampleStride < n; j0 += kThreads) {
-    const int e = (j0 + lane) * kSampleStride;
-    const unsigned k = e < n ? keys[e] : kNone;
-    append_warp(k != kNone, k != kNone ? key_of(k) : kNone, cand, kCandCap, &S->count);
-  }
-  __syncthreads();
-  const unsigned s = min(S->count, (unsigned)kCandCap);
-  bool done = false;
-  if (s >= 64u) {
-    // sample ranks around the expected one, 4 binomial standard deviations
-    // wide, widened to whole top-11-bit bins of one histogram of the sample
-    const unsigned p = (unsigned)(((unsigned long long)r * s) / nf);
-    const unsigned delta = 2u * (unsigned)sqrtf((float)s) + 4u;
-    const unsigned rlo = p > delta ? p - delta : 0u, rhi = min(p + delta, s - 1u);
-    for (int i = tid; i < kBins; i += kThreads) S->hist[i] = 0u;
-    __syncthreads();
-    for (int base = tid - lane; base < (int)s; base += kThreads) {
-      const int e = base + lane;
-      hist_add_warp(S->hist, e < (int)s ? cand[e] >> 21 : (unsigned)kBins);
-    }
-    __syncthreads();
-    find_digit(S, rlo);
-    const unsigned lo = S->digit << 21;
-    find_digit(S, rhi);
-    const unsigned hi = (S->digit << 21) | 0x1fffffu;
-    // one counting pass: keys below the bracket, keys inside it into cand
-    if (tid == 0) {
-      S->count = 0u;
-      S->below = 0u;
-    }
-    __syncthreads();
-    unsigned below = 0u;
-    for (int base = tid - lane; base < n; base += kThreads) {
-      const int e = base + lane;
-      const unsigned k = e < n ? keys[e] : kNone;
-      const unsigned a = k != kNone ? key_of(k) : kNone;
-      below += (a < lo) ? 1u : 0u;
-      append_warp(a != kNone && a >= lo && a <= hi, a, cand, kCandCap, &S->count);
-    }
-    below = __reduce_add_sync(0xffffffffu, below);
-    if (lane == 0) atomicAdd(&S->below, below);
-    __syncthreads();
-    const unsigned c_lo = S->below, cnt = S->count;
-    if (cnt <= (unsigned)kCandCap && r >= c_lo && r < c_lo + cnt) {
-      *k1 = select_keys(cand, (int)cnt, r - c_lo, S, want_next, &nx);
-      if (want_next && nx == kNone) {
-        // order statistic r + 1 lies above the bracket: the smallest key above it
+    if (round == 2) {
+      *v1 = *v2 = fkey_inv(prefix);
+      if (want_next && r + 1u >= S->hist[d]) {  // the next order statistic is another value
         if (tid == 0) S->next = kNone;
         __syncthreads();
-        for (int e = tid; e < n; e += kThreads) {
-          const unsigned k = keys[e];
-          if (k != kNone) {
-            const unsigned a = key_of(k);
-            if (a > hi) atomicMin(&S->next, a);
-          }
-        }
+        unsigned mn = kNone;
+        for_window(w, [&](float v) {
+          const unsigned k = isfinite(v) ? fkey(of(v)) : 0u;
+          if (k > prefix) mn = min(mn, k);
+        });
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        if ((tid & 31) == 0) atomicMin(&S->next, mn);
         __syncthreads();
-        nx = S->next;
+        *v2 = fkey_inv(S->next);
       }
-      *k2 = nx;
-      done = true;
     }
-    __syncthreads();
-  }
-  if (!done) {  // the whole window (rare for noise-like data)
-    if (rewrite) {
-      for (int e = tid; e < n; e += kThreads)
-        if (keys[e] != kNone) keys[e] = key_of(keys[e]);
-      __syncthreads();
-    }
-    // select_keys needs keys below kNone only: count the kNone slots out by
-    // giving the selection all n slots (they sort last) and the same rank
-    *k1 = select_keys(keys, n, r, S, want_next, &nx);
-    *k2 = nx;
   }
   __syncthreads();
-  return !done && rewrite;  // keys[] now holds key_of of the original keys
 }
 
-__device__ __forceinline__ double key_value(unsigned k) { return (double)fkey_inv(k); }
+// Order statistics r and (want_next) r + 1 among the copies (all in [lo, hi],
+// more than r of them); for a next one outside them, nxt(): its value. False
+// (uniformly) when too many copies share the step of the rank.
+template <class Next>
+__device__ bool select_cand(float lo, float hi, unsigned r, bool want_next, Scratch* S, float* v1, float* v2,
+                            Next nxt) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float* const seg = S->cand + warp * kSegCap;
+  const int n = (int)S->seg[warp];
+  // the step of a copy: a monotone function of its value
+  const float inv = (float)kBins / (hi - lo);
+  const auto digit = [&](float v) { return min(kBins - 1, (int)((v - lo) * inv)); };
+  clear_hist(S);
+  if (tid == 0) {
+    S->n_few = 0u;
+    S->next = kNone;
+  }
+  __syncthreads();
+  for (int i = lane; i < n; i += 32) atomicAdd(&S->hist[digit(seg[i])], 1u);
+  find_digits(S, r, r);
+  const int d = (int)S->digit[0];
+  const unsigned rr = S->rank[0], cnt = S->hist[d];
+  if (cnt > (unsigned)kFewCap) {
+    // ties? one value in the whole step is the answer
+    if (tid == 0) {
+      S->digit[0] = kNone;
+      S->digit[1] = 0u;
+    }
+    __syncthreads();
+    unsigned kmin = kNone, kmax = 0u;
+    for (int i = lane; i < n; i += 32) {
+      if (digit(seg[i]) != d) continue;
+      kmin = min(kmin, fkey(seg[i]));
+      kmax = max(kmax, fkey(seg[i]));
+    }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) {
+      atomicMin(&S->digit[0], kmin);
+      atomicMax(&S->digit[1], kmax);
+    }
+    __syncthreads();
+    const bool same = S->digit[0] == S->digit[1];
+    *v1 = *v2 = fkey_inv(S->digit[0]);
+    __syncthreads();
+    return same && (!want_next || rr + 1u < cnt);
+  }
+  unsigned above = kNone;
+  for (int i = lane; i < n; i += 32) {
+    const float v = seg[i];
+    const int dv = digit(v);
+    if (dv == d) S->few[atomicAdd(&S->n_few, 1u)] = v;
+    else if (dv > d) above = min(above, fkey(v));
+  }
+  if (want_next) {
+    above = __reduce_min_sync(0xffffffffu, above);
+    if (lane == 0) atomicMin(&S->next, above);
+  }
+  __syncthreads();
+  if (tid < (int)cnt) {
+    const float v = S->few[tid];
+    unsigned k = 0u;  // its rank in the step, ties in the order of the list
+    for (int j = 0; j < (int)cnt; ++j) {
+      const float o = S->few[j];
+      k += (o < v || (o == v && j < tid)) ? 1u : 0u;
+    }
+    if (k == rr) S->v1 = v;
+    if (want_next && k == rr + 1u) S->next = fkey(v);
+  }
+  __syncthreads();
+  *v1 = *v2 = S->v1;
+  if (want_next) *v2 = S->next != kNone ? fkey_inv(S->next) : nxt();
+  return true;
+}
+
+// Counts (into *below) the values of(v) under lo and copies those in [lo, hi].
+struct Collect {
+  float lo, hi;
+  float* seg;
+  unsigned n, below, lanes_below;
+  __device__ __forceinline__ void operator()(float a) {  // (NaN: neither)
+    const bool under = a < lo;
+    below += under ? 1u : 0u;
+    const bool in = a <= hi && !under;
+    const unsigned b = __ballot_sync(0xffffffffu, in);
+    const unsigned pos = n + (unsigned)__popc(b & lanes_below);
+    if (in && pos < (unsigned)kSegCap) seg[pos] = a;
+    n += (unsigned)__popc(b);
+  }
+};
+
+// Key bounds around sample ranks p +- 4 binomial standard deviations, widened
+// to whole digits; the sample's histogram is in S->hist.
+__device__ __forceinline__ void bracket_digits(Scratch* S, unsigned ns, unsigned p) {
+  const unsigned delta = 2u * (unsigned)sqrtf((float)ns) + 4u;
+  find_digits(S, p > delta ? p - delta : 0u, min(p + delta, ns - 1u));
+}
 
 // *s + *c += x with Neumaier's compensation (the running error of the float
 // sum is kept in *c).
@@ -291,32 +363,6 @@ __device__ __forceinline__ void neumaier_add(float* s, float* c, float x) {
   *s = t;
 }
 
-// x - b exactly as s + err (Knuth's TwoSum, round-to-nearest float ops).
-__device__ __forceinline__ float two_diff(float x, float b, float* err) {
-  const float s = __fsub_rn(x, b);
-  const float bb = __fsub_rn(s, x);
-  *err = __fadd_rn(__fsub_rn(x, __fsub_rn(s, bb)), __fsub_rn(-b, bb));
-  return s;
-}
-
-// The MAD key of x: the float of |x - m| with m = (a + b) / 2 (a == b for an
-// odd count: one correctly rounded subtraction). For an even count, x - a/2
-// and then - b/2 are taken exactly as sums of two floats and added back, which
-// rounds the exact difference faithfully (within one unit in the last place)
-// in single precision, without the slow FP64 pipe.
-__device__ __forceinline__ unsigned mad_key(float x, float a, float b, bool even) {
-  float d;
-  if (!even) {
-    d = __fsub_rn(x, a);
-  } else {
-    float e1, e2;
-    const float t = two_diff(x, 0.5f * a, &e1);
-    const float u = two_diff(t, 0.5f * b, &e2);
-    d = __fadd_rn(u, __fadd_rn(e1, e2));
-  }
-  return __float_as_uint(fabsf(d)) | 0x80000000u;  // fkey of a non-negative float
-}
-
 __device__ __forceinline__ double block_sum_d(double v, double* part) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -324,34 +370,214 @@ __device__ __forceinline__ double block_sum_d(double v, double* part) {
   if (lane == 0) part[warp] = v;
   __syncthreads();
   double t = 0.0;
-  if (warp == 0) {
-    t = lane < kWarps ? part[lane] : 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) part[32] = t;
-  }
-  __syncthreads();
-  t = part[32];
+  for (int k = 0; k < kWarps; ++k) t += part[k];
   __syncthreads();
   return t;
 }
 
+// Exact median and MAD of the nf finite voxels of the window.
+__device__ double window_mad(const Win& w, Scratch* S) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rows = w.ly * w.lz;
+  Collect col;
+  col.seg = S->cand + warp * kSegCap;
+  col.lanes_below = (1u << lane) - 1u;
+  // a window whose warps' shares fit their segments is copied whole
+  const bool whole = w.share() <= kSegCap;
+  float lo = -FLT_MAX, hi = FLT_MAX;
+  bool bracket = true;
+  unsigned ns = 0u;
+  if (tid == 0) S->finite = S->below = S->n_sample = 0u;
+  if (!whole) {
+    // every 8th voxel of every row (the offset moves with the row), of every
+    // second row where that would overflow the sample's room
+    const int sx = (w.lx + 7) >> 3;
+    int rstep = 1;
+    while ((rows + rstep - 1) / rstep * sx > kSampleCap) ++rstep;
+    const int want = (rows + rstep - 1) / rstep * sx;
+    clear_hist(S);
+    __syncthreads();
+    unsigned c = 0u;
+    for (int i0 = 0; i0 < want; i0 += 4 * kThreads) {
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * kThreads + tid;
+        v[u] = __int_as_float(0x7fc00000);
+        if (i < want) {
+          const int q = i / sx, r = q * rstep, z = r / w.ly, y = r - z * w.ly;
+          const int dx = 8 * (i - q * sx) + ((3 * q) & 7);
+          if (dx < w.lx) v[u] = __ldg(w.base + z * w.plane + y * w.nx + dx);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * kThreads + tid;
+        if (i >= want) break;
+        const bool ok = isfinite(v[u]);
+        S->sample[i] = ok ? v[u] : __int_as_float(0x7fc00000);
+        if (ok) {
+          ++c;
+          atomicAdd(&S->hist[fkey(v[u]) >> 21], 1u);
+        }
+      }
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0 && c) atomicAdd(&S->n_sample, c);
+    __syncthreads();
+    ns = S->n_sample;
+    bracket = ns >= 64u;
+    if (bracket) {
+      bracket_digits(S, ns, (ns - 1u) / 2u);
+      lo = fkey_inv(S->digit[0] << 21);
+      hi = fkey_inv((S->digit[1] << 21) | 0x1fffffu);
+    }
+  }
+  __syncthreads();
+  unsigned finite = 0u;
+  col.lo = lo;
+  col.hi = hi;
+  col.n = col.below = 0u;
+  for_window(w, [&](float v) {
+    v = __fadd_rn(v, __fsub_rn(v, v));  // Inf becomes NaN
+    finite += v == v ? 1u : 0u;
+    col(v);
+  });
+  finite = __reduce_add_sync(0xffffffffu, finite);
+  unsigned below = __reduce_add_sync(0xffffffffu, col.below);
+  if (lane == 0) {
+    S->seg[warp] = col.n;
+    atomicAdd(&S->finite, finite);
+    atomicAdd(&S->below, below);
+  }
+  __syncthreads();
+  const unsigned nf = S->finite;
+  if (nf == 0u) return __longlong_as_double(0x7ff8000000000000LL);  // no finite voxel
+  const unsigned r1 = (nf - 1u) / 2u;
+  const bool even = (nf & 1u) == 0u;
+  // the copies are complete and hold the rank
+  const auto holds = [&](unsigned under) {
+    unsigned n = 0u;
+    bool fits = true;
+    for (int k = 0; k < kWarps; ++k) {
+      n += S->seg[k];
+      fits = fits && S->seg[k] <= (unsigned)kSegCap;
+    }
+    return fits && r1 >= under && r1 < under + n;
+  };
+  float ma = 0.0f, mb = 0.0f;
+  below = S->below;
+  bool done = bracket && holds(below);
+  if (whole) {
+    // the bracket of the copies: their smallest and largest value
+    if (tid == 0) {
+      S->digit[0] = kNone;
+      S->digit[1] = 0u;
+    }
+    __syncthreads();
+    unsigned kmin = kNone, kmax = 0u;
+    for (int i = lane; i < (int)S->seg[warp]; i += 32) {
+      const unsigned k = fkey(col.seg[i]);
+      kmin = min(kmin, k);
+      kmax = max(kmax, k);
+    }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) {
+      atomicMin(&S->digit[0], kmin);
+      atomicMax(&S->digit[1], kmax);
+    }
+    __syncthreads();
+    lo = fkey_inv(S->digit[0]);
+    hi = fkey_inv(S->digit[1]);
+    __syncthreads();
+  }
+  // the smallest value of(x) above hi in the window
+  const auto above = [&](auto of, float top) {
+    unsigned mn = kNone;
+    for_window(w, [&](float v) {
+      const float a = isfinite(v) ? of(v) : __int_as_float(0x7fc00000);
+      if (a > top) mn = min(mn, fkey(a));
+    });
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    __syncthreads();
+    if (lane == 0) atomicMin(&S->next, mn);
+    __syncthreads();
+    return fkey_inv(S->next);
+  };
+  if (done) done = select_cand(lo, hi, r1 - below, even, S, &ma, &mb, [&] { return above(Value{}, hi); });
+  if (!done) select_window(w, Value{}, r1, even, S, &ma, &mb);
+  if (!even) mb = ma;
+  __syncthreads();
+  // the MAD: the same order statistics of |x - m|, m = (ma + mb) / 2
+  const AbsDev dev{ma, mb, even};
+  float d1 = 0.0f, d2 = 0.0f;
+  if (whole) {  // the copies are all finite voxels
+    if (tid == 0) S->digit[1] = 0u;
+    __syncthreads();
+    unsigned kmax = 0u;
+    for (int i = lane; i < (int)S->seg[warp]; i += 32) {
+      const float a = dev(col.seg[i]);
+      col.seg[i] = a;
+      kmax = max(kmax, __float_as_uint(a));
+    }
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) atomicMax(&S->digit[1], kmax);
+    __syncthreads();
+    hi = __uint_as_float(S->digit[1]);
+    __syncthreads();
+    done = select_cand(0.0f, hi, r1, even, S, &d1, &d2, [&] { return d1; });
+  } else {
+    done = ns >= 64u;
+    if (done) {
+      clear_hist(S);
+      if (tid == 0) S->below = 0u;
+      __syncthreads();
+      const int sx = (w.lx + 7) >> 3;
+      int rstep = 1;
+      while ((rows + rstep - 1) / rstep * sx > kSampleCap) ++rstep;
+      const int want = (rows + rstep - 1) / rstep * sx;
+      for (int i = tid; i < want; i += kThreads) {
+        const float v = S->sample[i];
+        if (isfinite(v)) atomicAdd(&S->hist[min(__float_as_uint(dev(v)) >> 20, (unsigned)kBins - 1u)], 1u);
+      }
+      bracket_digits(S, ns, (unsigned)(((unsigned long long)r1 * ns) / nf));
+      lo = __uint_as_float(S->digit[0] << 20);
+      hi = fminf(__uint_as_float((S->digit[1] << 20) | 0xfffffu), FLT_MAX);
+      __syncthreads();
+      col.lo = lo;
+      col.hi = hi;
+      col.n = col.below = 0u;
+      for_window(w, [&](float v) { col(dev(v)); });  // NaN and Inf voxels: |v - m| is NaN or Inf
+      below = __reduce_add_sync(0xffffffffu, col.below);
+      if (lane == 0) {
+        S->seg[warp] = col.n;
+        atomicAdd(&S->below, below);
+      }
+      __syncthreads();
+      below = S->below;
+      done = holds(below);
+    }
+    if (done) done = select_cand(lo, hi, r1 - below, even, S, &d1, &d2, [&] { return above(dev, hi); });
+  }
+  if (!done) select_window(w, dev, r1, even, S, &d1, &d2);
+  const double mad = even ? 0.5 * ((double)d1 + (double)d2) : (double)d1;
+  return kMadToSigma * mad;
+}
+
 }  // namespace nscale
 
-__global__ void __launch_bounds__(nscale::kThreads, 1)
+__global__ void __launch_bounds__(nscale::kThreads, nscale::kBlocksPerSm)
     k_noise_window(const float* __restrict__ cube, nscale::Geo g, int mode, double* __restrict__ sig_out,
                    float* __restrict__ rinv_out) {
   using namespace nscale;
-  const bool std_mode = mode == SC_NOISE_STD;
-  extern __shared__ __align__(16) unsigned char ns_smem[];
-  unsigned* const cand = reinterpret_cast<unsigned*>(ns_smem);  // [kCandCap]
-  unsigned* const keys = cand + kCandCap;                          // [window voxels]
-  __shared__ SelScratch S;
-  __shared__ double dpart[kWarps + 1];
-  __shared__ unsigned s_count;
+  __shared__ Scratch S;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long n_cells = (long long)g.ncx * g.ncy * g.ncz;
-  const long long plane = g.nx * g.ny;
+  Win w;
+  w.plane = g.nx * g.ny;
+  w.nx = g.nx;
   for (long long cell = blockIdx.x; cell < n_cells; cell += gridDim.x) {
     const int cx = (int)(cell % g.ncx);
     const int cy = (int)((cell / g.ncx) % g.ncy);
@@ -360,179 +586,64 @@ __global__ void __launch_bounds__(nscale::kThreads, 1)
     window_range(cx, g.gx, g.wx, g.nx, &x0, &x1);
     window_range(cy, g.gy, g.wy, g.ny, &y0, &y1);
     window_range(cz, g.gz, g.wz, g.nz, &z0, &z1);
-    const int lx = (int)(x1 - x0), ly = (int)(y1 - y0), lz = (int)(z1 - z0);
-    const int n = lx * ly * lz;
-    if (tid == 0) s_count = 0u;
-    // Median bracket (MAD mode, windows larger than the copy-aside buffer): a
-    // sample of every kSampleStride-th voxel, read straight from the cube,
-    // and its top-11-bit histogram give key bounds [lo, hi] around the middle
-    // rank, so that the load pass below can count the keys under lo and copy
-    // those inside into cand.
-    bool med_bracket = !std_mode && n > kCandCap;
-    unsigned lo = 0u, hi = kNone - 1u;
-    if (med_bracket) {
-      if (tid == 0) S.count = 0u;
-      __syncthreads();
-      const int lxy = lx * ly;
-      for (int j0 = tid - lane; j0 * kSampleStride < n; j0 += kThreads) {
-        const int e = (j0 + lane) * kSampleStride;
-        unsigned k = kNone;
-        if (e < n) {
-          const int dz = e / lxy, rem = e - dz * lxy, dy = rem / lx, dx = rem - dy * lx;
-          const float v = __ldg(cube + (z0 + dz) * plane + (y0 + dy) * g.nx + x0 + dx);
-          if (isfinite(v)) k = fkey(v);
-        }
-        append_warp(k != kNone, k, cand, kCandCap, &S.count);
-      }
-      __syncthreads();
-      const unsigned ns = min(S.count, (unsigned)kCandCap);
-      med_bracket = ns >= 64u;
-      if (med_bracket) {
-        const unsigned p = (ns - 1u) / 2u;
-        const unsigned delta = 2u * (unsigned)sqrtf((float)ns) + 4u;
-        for (int i = tid; i < kBins; i += kThreads) S.hist[i] = 0u;
-        __syncthreads();
-        for (int base = tid - lane; base < (int)ns; base += kThreads) {
-          const int e = base + lane;
-          hist_add_warp(S.hist, e < (int)ns ? cand[e] >> 21 : (unsigned)kBins);
-        }
-        __syncthreads();
-        find_digit(&S, p > delta ? p - delta : 0u);
-        lo = S.digit << 21;
-        find_digit(&S, min(p + delta, ns - 1u));
-        hi = (S.digit << 21) | 0x1fffffu;
-      }
-      if (tid == 0) {
-        S.count = 0u;
-        S.below = 0u;
-      }
-    }
-    __syncthreads();
-    // the window's keys: warps over rows, four planes' loads issued together;
-    // with a bracket, also the keys under it counted and those in it copied
-    unsigned finite = 0u, below = 0u;
-    constexpr int kPlanesAtOnce = 4;
-    for (int dz0 = 0; dz0 < lz; dz0 += kPlanesAtOnce) {
-      for (int dy = warp; dy < ly; dy += kWarps) {
-        for (int dx0 = 0; dx0 < lx; dx0 += 32) {
-          const int dx = dx0 + lane;
-          float v[kPlanesAtOnce];
-#pragma unroll
-          for (int u = 0; u < kPlanesAtOnce; ++u)
-            v[u] = (dz0 + u < lz && dx < lx) ? __ldg(cube + (z0 + dz0 + u) * plane + (y0 + dy) * g.nx + x0 + dx)
-                                             : __int_as_float(0x7fc00000);
-#pragma unroll
-          for (int u = 0; u < kPlanesAtOnce; ++u) {
-            const bool ok = isfinite(v[u]);
-            const unsigned k = ok ? fkey(v[u]) : kNone;
-            if (dz0 + u < lz && dx < lx) keys[((dz0 + u) * ly + dy) * lx + dx] = k;
-            finite += ok ? 1u : 0u;
-            if (med_bracket) {
-              below += (ok && k < lo) ? 1u : 0u;
-              append_warp(ok && k >= lo && k <= hi, k, cand, kCandCap, &S.count);
-            }
-          }
-        }
-      }
-    }
-    finite = __reduce_add_sync(0xffffffffu, finite);
-    below = __reduce_add_sync(0xffffffffu, below);
-    if (lane == 0) {
-      atomicAdd(&s_count, finite);
-      if (med_bracket) atomicAdd(&S.below, below);
-    }
-    __syncthreads();
-    const unsigned nf = s_count;
+    w.base = cube + z0 * w.plane + y0 * g.nx + x0;
+    w.lx = (int)(x1 - x0);
+    w.ly = (int)(y1 - y0);
+    w.lz = (int)(z1 - z0);
+    w.split();
+    __syncthreads();  // the previous cell is done with the scratch
     double sigma;
-    if (nf == 0u) {
-      sigma = __longlong_as_double(0x7ff8000000000000LL);  // NaN: no finite voxel
-    } else if (std_mode) {
+    if (mode == SC_NOISE_STD) {
       // float32 sums with Neumaier compensation per thread (the FP64 pipe is
       // slow on this part), combined in double across the block
       float s = 0.0f, sc = 0.0f;
-      for (int e = tid; e < n; e += kThreads)
-        if (keys[e] != kNone) neumaier_add(&s, &sc, fkey_inv(keys[e]));
-      const double mean = block_sum_d((double)s + (double)sc, dpart) / (double)nf;
-      const float mh = __double2float_rn(mean), ml = __double2float_rn(mean - (double)mh);
-      float q = 0.0f, qc = 0.0f;
-      for (int e = tid; e < n; e += kThreads)
-        if (keys[e] != kNone) {
-          const float d = __fsub_rn(__fsub_rn(fkey_inv(keys[e]), mh), ml);
-          neumaier_add(&q, &qc, __fmul_rn(d, d));
+      unsigned finite = 0u;
+      for_window(w, [&](float v) {
+        if (isfinite(v)) {
+          neumaier_add(&s, &sc, v);
+          ++finite;
         }
-      const double qq = block_sum_d((double)q + (double)qc, dpart);
-      sigma = nf > 1u ? sqrt(qq / (double)(nf - 1u)) : 0.0;
-    } else {
-      // median: order statistics (nf - 1) / 2 and nf / 2
-      const unsigned r1 = (nf - 1u) / 2u;
-      const bool even = (nf & 1u) == 0u;
-      unsigned k1 = 0u, k2 = 0u;
-      const unsigned c_lo = S.below, cnt = S.count;
-      if (med_bracket && cnt <= (unsigned)kCandCap && r1 >= c_lo && r1 < c_lo + cnt) {
-        unsigned nx = kNone;
-        k1 = select_keys(cand, (int)cnt, r1 - c_lo, &S, even, &nx);
-        if (even && nx == kNone) {  // the next order statistic lies above the bracket
-          if (tid == 0) S.next = kNone;
-          __syncthreads();
-          for (int e = tid; e < n; e += kThreads) {
-            const unsigned k = keys[e];
-            if (k != kNone && k > hi) atomicMin(&S.next, k);
-          }
-          __syncthreads();
-          nx = S.next;
-        }
-        k2 = nx;
-        __syncthreads();
+      });
+      finite = __reduce_add_sync(0xffffffffu, finite);
+      if (lane == 0) S.part[warp] = finite;
+      const double sum = block_sum_d((double)s + (double)sc, S.dpart);
+      unsigned nf = 0u;
+      for (int k = 0; k < kWarps; ++k) nf += S.part[k];
+      if (nf == 0u) {
+        sigma = __longlong_as_double(0x7ff8000000000000LL);  // NaN: no finite voxel
       } else {
-        select_order(keys, n, nf, r1, even, [](unsigned k) { return k; }, false, cand, &S, &k1, &k2);
+        const double mean = sum / (double)nf;
+        const float mh = __double2float_rn(mean), ml = __double2float_rn(mean - (double)mh);
+        float q = 0.0f, qc = 0.0f;
+        for_window(w, [&](float v) {
+          if (isfinite(v)) {
+            const float d = __fsub_rn(__fsub_rn(v, mh), ml);
+            neumaier_add(&q, &qc, __fmul_rn(d, d));
+          }
+        });
+        const double qq = block_sum_d((double)q + (double)qc, S.dpart);
+        sigma = nf > 1u ? sqrt(qq / (double)(nf - 1u)) : 0.0;
       }
-      // MAD: the same order statistics of |x - m|, m = (k1 + k2) / 2, as
-      // float32 keys computed on the fly
-      const float ma = fkey_inv(k1), mb = even ? fkey_inv(k2) : ma;
-      unsigned a1 = 0u, a2 = 0u;
-      const bool rewrote =
-          select_order(keys, n, nf, r1, even, [=](unsigned k) { return mad_key(fkey_inv(k), ma, mb, even); }, true,
-                       cand, &S, &a1, &a2);
-      const double mad = even ? 0.5 * (key_value(a1) + key_value(a2)) : key_value(a1);
-      sigma = kMadToSigma * mad;
+    } else {
+      sigma = window_mad(w, &S);
       if (mode == SC_NOISE_GAUSS && sigma > 0.0) {
-        // the window's 256-bin histogram (from the keys in shared memory, or
-        // read again from the cube where the selection rewrote them), then a
-        // one-warp fit; the MAD noise stands without a root
+        // the window's 256-bin histogram, then a one-warp fit; the MAD noise
+        // stands without a root
         const float k = gfit::scale_of(sigma);
         __syncthreads();  // the selection is done with S.hist
         for (int i = tid; i < gfit::kBins; i += kThreads) S.hist[i] = 0u;
         __syncthreads();
-        if (!rewrote) {
-          for (int e = tid; e < n; e += kThreads) {
-            const unsigned key = keys[e];
-            const int b = key != kNone ? gfit::bin_of(fkey_inv(key), k) : -1;
-            if (b >= 0) atomicAdd(&S.hist[b], 1u);
-          }
-        } else {
-          for (int dz = 0; dz < lz; ++dz)
-            for (int dy = warp; dy < ly; dy += kWarps)
-              for (int dx = lane; dx < lx; dx += 32) {
-                const int b = gfit::bin_of(__ldg(cube + (z0 + dz) * plane + (y0 + dy) * g.nx + x0 + dx), k);
-                if (b >= 0) atomicAdd(&S.hist[b], 1u);
-              }
-        }
+        for_window(w, [&](float v) {
+          const int b = gfit::bin_of(v, k);
+          if (b >= 0) atomicAdd(&S.hist[b], 1u);
+        });
         __syncthreads();
         if (warp == 0) {
-          double hh[4], x2[4];
-          bool use[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int t = lane + 32 * j;
-            hh[j] = (double)S.hist[gfit::kHalf + t] + (double)S.hist[gfit::kHalf - 1 - t];
-            x2[j] = gfit::xi2_of(t);
-            use[j] = true;
-          }
-          const double tau = gfit::fit_tau(hh, x2, use, gfit::WarpSum6{});
-          if (lane == 0) dpart[0] = tau;
+          const double tau = gfit::fit_tau_warp(S.hist);
+          if (lane == 0) S.dpart[0] = tau;
         }
         __syncthreads();
-        const double tau = dpart[0];
+        const double tau = S.dpart[0];
         if (tau > 0.0) sigma = gfit::noise_of(tau, k);
       }
     }
@@ -540,7 +651,6 @@ __global__ void __launch_bounds__(nscale::kThreads, 1)
       sig_out[cell] = sigma;
       rinv_out[cell] = sigma > 0.0 ? __double2float_rn(1.0 / sigma) : __int_as_float(0x7fc00000);
     }
-    __syncthreads();  // the keys are overwritten by the next cell
   }
 }
 
@@ -584,10 +694,6 @@ __global__ void __launch_bounds__(256) k_noise_apply(const float* in, float* out
   }
 }
 
-size_t noise_window_smem(long long window_voxels) {
-  return sizeof(unsigned) * ((size_t)nscale::kCandCap + (size_t)window_voxels);
-}
-
 namespace {
 nscale::Geo make_geo(const long long dims[3], const int window[3], const int grid[3]) {
   nscale::Geo g;
@@ -611,9 +717,9 @@ cudaError_t launch_noise_window(const float* cube, const long long dims[3], cons
                                 int noise_mode, double* sig_dev, float* rinv_dev, int sms, cudaStream_t s) {
   const nscale::Geo g = make_geo(dims, window, grid);
   const long long cells = (long long)g.ncx * g.ncy * g.ncz;
-  const long long wvox = (long long)min((long long)g.wx, g.nx) * min((long long)g.wy, g.ny) * min((long long)g.wz, g.nz);
-  const int blocks = (int)(cells < sms ? cells : sms);
-  k_noise_window<<<blocks, nscale::kThreads, noise_window_smem(wvox), s>>>(cube, g, noise_mode, sig_dev, rinv_dev);
+  const long long most = (long long)nscale::kBlocksPerSm * sms;
+  const int blocks = (int)(cells < most ? cells : most);
+  k_noise_window<<<blocks, nscale::kThreads, 0, s>>>(cube, g, noise_mode, sig_dev, rinv_dev);
   return cudaGetLastError();
 }
 
@@ -627,11 +733,6 @@ cudaError_t launch_noise_apply(const float* cube, const long long dims[3], const
                   (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
   k_noise_apply<<<blocks, 256, 0, s>>>(cube, out, g, rinv_dev, vec);
   return cudaGetLastError();
-}
-
-void init_noise_scale_attrs() {
-  cudaFuncSetAttribute(k_noise_window, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)noise_window_smem(kNoiseScaleMaxWindow));
 }
 
 }  // namespace sc
