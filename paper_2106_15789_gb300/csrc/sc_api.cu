@@ -52,6 +52,8 @@ struct sc_ctx {
   size_t lk_comp_cap = 0;
   unsigned char* af_buf = nullptr;  // sc_autoflag: noises, flags and statistics (lazy, grown)
   size_t af_cap = 0;
+  void* af_chan = nullptr;          // and its channel passes' brackets and copies (lazy, grown)
+  size_t af_chan_cap = 0;
   uint8_t* stage_mask = nullptr;
   // sc_run_host_many (lazy): two device input / mask sets, the per-channel
   // scales of 16-bit cubes, the copy stream and its events, per-cube results
@@ -766,6 +768,7 @@ void sc_destroy(sc_ctx* c) {
   cudaFree(c->lk_chunk);
   cudaFree(c->lk_tot);
   cudaFree(c->lk_comp);
+  cudaFree(c->af_chan);
   cudaFree(c->af_buf);
   cudaFree(c->sh_P);
   cudaFree(c->sh_nf);
@@ -1704,14 +1707,29 @@ int sc_autoflag(sc_ctx* c, const float* cube_dev, const int64_t* dims, double k,
     }
     c->af_cap = need;
   }
+  // scratch of the channel passes (half a byte per voxel), grown on
+  // demand; without it the channels are measured by a block each
+  const size_t chan_need = ch ? chan_scratch_bytes(d, noise_mode) : 0;
+  if (chan_need > c->af_chan_cap) {
+    cudaFree(c->af_chan);
+    c->af_chan = nullptr;
+    c->af_chan_cap = 0;
+    if (cudaMalloc(&c->af_chan, chan_need) == cudaSuccess) {
+      c->af_chan_cap = chan_need;
+    } else {
+      cudaGetLastError();
+      c->af_chan = nullptr;
+    }
+  }
+  void* const chan_scratch = chan_need > 0 && chan_need <= c->af_chan_cap ? c->af_chan : nullptr;
   double* stats = reinterpret_cast<double*>(c->af_buf);
   float* cn = reinterpret_cast<float*>(c->af_buf + 64);
   float* pn = cn + d[2];
   uint8_t* cf = reinterpret_cast<uint8_t*>(pn + plane);
   uint8_t* pf = cf + d[2];
   CK(launch_autoflag(cube_dev, d, k, ch ? 1 : 0, px ? 1 : 0, noise_mode, out_dev, cn, pn, cf,
-                     pf, stats, c->sms, s));
-  c->stats.launches += (ch ? 3 : 0) + (px ? 3 : 0) + 1;
+                     pf, stats, chan_scratch, c->sms, s));
+  c->stats.launches += (ch ? (chan_scratch ? 7 : 3) : 0) + (px ? 3 : 0) + 1;
   const bool want_counts = n_flagged != nullptr;
   std::vector<uint8_t> cf_h, pf_h;
   if (ch && (chan_flags_host || want_counts)) {

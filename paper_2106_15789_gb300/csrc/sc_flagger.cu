@@ -2,9 +2,16 @@
 // deviates from the median noise across all channels / pixels by more than k
 // times the MAD-based RMS are blanked.
 //
-//   k_chan_noise   one block per channel: the noise of its plane (exact
-//                  median and MAD by radix selection over the plane streamed
-//                  from memory, or compensated sums for STD)
+//   k_chan_sample, k_chan_pass, k_chan_select
+//                  the median and MAD of every channel's plane: a sample of
+//                  the plane brackets the wanted rank, a pass over the whole
+//                  cube counts each plane's values under its bracket and
+//                  copies those inside, and a block per channel finds the
+//                  rank among the copies (twice: values, then |x - m|)
+//                  (and the Gaussian fit, over the plane once more)
+//   k_chan_noise   one block per channel, the plane streamed from memory: STD
+//                  by compensated sums, and (small planes, or no room for the
+//                  copies) median and MAD by radix passes
 //   k_pix_noise    one block per 32 pixels of a row: their spectra staged in
 //                  shared memory, each pixel's noise by one warp with the
 //                  spectrum in registers (exact selections by bisection on
@@ -14,6 +21,7 @@
 //   k_blank        out = NaN on flagged channels and pixels, else in
 //
 // The noises are kept in float32; M, R and the flag test are in double.
+#include <cfloat>
 #include <cstdint>
 
 #include "sc_device.cuh"
@@ -171,6 +179,31 @@ __device__ unsigned stream_select(const float* __restrict__ src, long long n, un
   return prefix;
 }
 
+// Gaussian-fit noise of the finite values of src[0 .. n) with MAD noise
+// sigma_mad > 0: the 256-bin histogram, then the fit (the MAD noise stands
+// without a root). All threads call it.
+__device__ double block_gauss(const float* __restrict__ src, long long n, double sigma_mad, Scratch* S) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const float k = gfit::scale_of(sigma_mad);
+  __syncthreads();  // the selection is done with S->hist
+  for (int i = tid; i < gfit::kBins; i += kThreads) S->hist[i] = 0u;
+  __syncthreads();
+  for (long long i = tid; i < n; i += kThreads) {
+    const int b = gfit::bin_of(__ldg(src + i), k);
+    if (b >= 0) atomicAdd(&S->hist[b], 1u);
+  }
+  __syncthreads();
+  // one warp fits (four folded bins a lane, no block barriers); the others wait
+  if (tid < 32) {
+    const double tau = gfit::fit_tau_warp(S->hist);
+    if (lane == 0) S->dpart[0] = tau;
+  }
+  __syncthreads();
+  const double tau = S->dpart[0];
+  __syncthreads();
+  return tau > 0.0 ? gfit::noise_of(tau, k) : sigma_mad;
+}
+
 // Noise of the finite values of src[0 .. n) (NaN if none) in the S+C sense
 // (mode SC_NOISE_MAD, _STD or _GAUSS); for MAD mode also the median m (the
 // stats kernel needs it). All threads call it and get the same values.
@@ -225,37 +258,7 @@ __device__ void block_noise(const float* __restrict__ src, long long n, int mode
   const double mad = even ? 0.5 * ((double)fkey_inv(a1) + (double)fkey_inv(a2)) : (double)fkey_inv(a1);
   *sigma = kMadToSigma * mad;
   *median = even ? 0.5 * ((double)ma + (double)mb) : (double)ma;
-  if (mode == SC_NOISE_GAUSS && *sigma > 0.0) {
-    // the 256-bin histogram of the finite values, then the fit (the MAD noise
-    // stands without a root)
-    const float k = gfit::scale_of(*sigma);
-    __syncthreads();  // the selection is done with S->hist
-    for (int i = tid; i < gfit::kBins; i += kThreads) S->hist[i] = 0u;
-    __syncthreads();
-    for (long long i = tid; i < n; i += kThreads) {
-      const int b = gfit::bin_of(__ldg(src + i), k);
-      if (b >= 0) atomicAdd(&S->hist[b], 1u);
-    }
-    __syncthreads();
-    // one warp fits (four folded bins a lane, no block barriers); the others wait
-    if (tid < 32) {
-      double hh[4], x2[4];
-      bool use[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int t = lane + 32 * j;
-        hh[j] = (double)S->hist[gfit::kHalf + t] + (double)S->hist[gfit::kHalf - 1 - t];
-        x2[j] = gfit::xi2_of(t);
-        use[j] = true;
-      }
-      const double tau = gfit::fit_tau(hh, x2, use, gfit::WarpSum6{});
-      if (lane == 0) S->dpart[0] = tau;
-    }
-    __syncthreads();
-    const double tau = S->dpart[0];
-    if (tau > 0.0) *sigma = gfit::noise_of(tau, k);
-    __syncthreads();
-  }
+  if (mode == SC_NOISE_GAUSS && *sigma > 0.0) *sigma = block_gauss(src, n, *sigma, S);
 }
 
 // ---- per-pixel noise: a warp per pixel, the spectrum in registers ----------
@@ -278,7 +281,320 @@ __device__ __forceinline__ unsigned warp_select(const unsigned (&k)[VPL], unsign
   return ans;
 }
 
+// ---- per-channel median and MAD by passes over the whole cube ---------------
+//
+// What bounds it: the two passes' reads of the cube. On 600 x 600 x 1024
+// voxels the form with one block per channel (seven passes over each plane by
+// 304 blocks, whose planes do not fit L2 together, and a match_any histogram
+// per value) took 11.3 ms; these kernels take 1.1 ms.
+constexpr int kChanSample = 4096;         // values sampled per plane, four a thread
+constexpr long long kChanMinPlane = 1LL << 15;  // smaller planes: one block streams them as fast
+constexpr int kPassThreads = 256;
+constexpr int kPassWarps = kPassThreads / 32;
+constexpr int kPassRun = 1024;            // consecutive values a warp takes
+constexpr int kFew = 1024;                // copies ranked directly
+
+// A channel's bracket [lo, hi] of the wanted rank and what a pass found.
+struct Chan {
+  float lo, hi;
+  unsigned finite, below, n;  // finite values, those under lo, copies (may exceed the room)
+  float ma, mb;               // the two middle values
+  int even;
+};
+
+// The digits whose cumulative ranges in S->hist hold ranks ra and rb, and the
+// ranks within them.
+__device__ __forceinline__ void find_two(Scratch* S, unsigned ra, unsigned rb, unsigned* da, unsigned* db,
+                                         unsigned* ia) {
+  const unsigned tid = threadIdx.x;
+  __syncthreads();
+  const unsigned a = S->hist[2 * tid], b = S->hist[2 * tid + 1];
+  const unsigned incl = block_scan_incl(a + b, S->part), excl = incl - a - b;
+  if (ra >= excl && ra < incl) {
+    const bool in_a = ra < excl + a;
+    S->digit = 2u * tid + (in_a ? 0u : 1u);
+    S->rank = ra - excl - (in_a ? 0u : a);
+  }
+  if (rb >= excl && rb < incl) S->next = 2u * tid + (rb < excl + a ? 0u : 1u);
+  __syncthreads();
+  *da = S->digit;
+  *db = S->next;
+  *ia = S->rank;
+  __syncthreads();
+}
+
+// Bracket of the median of of(x) over the plane, from a sample at a fixed step
+// (each place moved a little, against patterns in the plane): sample ranks p
+// +- 4 binomial standard deviations, located by the top 11 bits of the keys
+// and then by 2048 equal steps between. Any bracket is checked by the pass's
+// counts. kShift: key bits under a digit (keys below 2^(11 + kShift)).
+template <int kShift, class Of, class Key>
+__device__ void plane_bracket(const float* __restrict__ src, long long n, Of of, Key key, Scratch* S, float* lo,
+                              float* hi) {
+  const unsigned tid = threadIdx.x;
+  const long long step = n / kChanSample;
+  float v[4];
+  unsigned c = 0u;
+  for (int i = tid; i < kBins; i += kThreads) S->hist[i] = 0u;
+  if (tid == 0u) S->count = 0u;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const unsigned j = u * kThreads + tid;
+    v[u] = __ldg(src + j * step + ((unsigned long long)(j * 2654435761u) * (unsigned long long)step >> 32));
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const bool ok = isfinite(v[u]);
+    v[u] = ok ? of(v[u]) : __int_as_float(0x7fc00000);
+    if (ok) {
+      ++c;
+      atomicAdd(&S->hist[min(key(v[u]) >> kShift, (unsigned)kBins - 1u)], 1u);
+    }
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
+  if ((tid & 31u) == 0u) atomicAdd(&S->count, c);
+  __syncthreads();
+  const unsigned ns = S->count;
+  *lo = -FLT_MAX;
+  *hi = FLT_MAX;
+  if (ns < 64u) return;
+  const unsigned p = (ns - 1u) / 2u, delta = 2u * (unsigned)sqrtf((float)ns) + 4u;
+  const unsigned ra = p > delta ? p - delta : 0u, rb = min(p + delta, ns - 1u);
+  unsigned da, db, ia;
+  find_two(S, ra, rb, &da, &db, &ia);
+  const float a = fminf(fmaxf(key.value(da << kShift), -FLT_MAX), FLT_MAX);
+  const float b = fminf(fmaxf(key.value((db << kShift) | ((1u << kShift) - 1u)), -FLT_MAX), FLT_MAX);
+  *lo = a;
+  *hi = b;
+  const float inv = (float)kBins / (b - a);
+  if (!(inv > 0.0f && isfinite(inv))) return;
+  for (int i = tid; i < kBins; i += kThreads) S->hist[i] = 0u;
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    if (v[u] >= a && v[u] <= b) atomicAdd(&S->hist[min(kBins - 1, (int)((v[u] - a) * inv))], 1u);
+  // the ranks among the values from the first digit on
+  find_two(S, ia, ia + (rb - ra), &da, &db, &ia);
+  const float w = (b - a) / (float)kBins;
+  *lo = fmaxf(a, a + (float)da * w);
+  *hi = fminf(b, a + (float)(db + 1u) * w);
+}
+
+struct KeyOfValue {
+  __device__ __forceinline__ unsigned operator()(float v) const { return fkey(v); }
+  __device__ __forceinline__ float value(unsigned k) const { return fkey_inv(k); }
+};
+struct KeyOfDev {
+  __device__ __forceinline__ unsigned operator()(float v) const { return __float_as_uint(v); }
+  __device__ __forceinline__ float value(unsigned k) const { return __uint_as_float(k); }
+};
+
+__device__ __forceinline__ float abs_dev(float x, float a, float b, bool even) {
+  return __uint_as_float(mad_key(x, a, b, even) & 0x7fffffffu);
+}
+
+// Order statistics r and (want_next) r + 1 among the n copies in list (all in
+// [lo, hi], more than r of them). False (uniformly) when the step of the rank
+// holds too many, or the next one lies beyond the copies.
+__device__ bool list_select(const float* __restrict__ list, unsigned n, float lo, float hi, unsigned r, bool want_next,
+                            Scratch* S, float* few, float* v1, float* v2) {
+  const unsigned tid = threadIdx.x, lane = tid & 31u;
+  const float inv = (float)kBins / (hi - lo);  // a step is a monotone function of the value
+  const auto digit = [&](float v) { return (unsigned)min(kBins - 1, (int)((v - lo) * inv)); };
+  for (int i = tid; i < kBins; i += kThreads) S->hist[i] = 0u;
+  if (tid == 0u) S->count = 0u;
+  __syncthreads();
+  for (unsigned i = tid; i < n; i += kThreads) atomicAdd(&S->hist[digit(list[i])], 1u);
+  unsigned d, d2, rr;
+  find_two(S, r, r, &d, &d2, &rr);
+  const unsigned cnt = S->hist[d];
+  if (tid == 0u) S->next = kNone;
+  __syncthreads();
+  const bool many = cnt > (unsigned)kFew;
+  unsigned above = kNone, kmin = kNone, kmax = 0u;
+  for (unsigned i = tid; i < n; i += kThreads) {
+    const float v = list[i];
+    const unsigned dv = digit(v);
+    if (dv == d) {
+      kmin = min(kmin, fkey(v));
+      kmax = max(kmax, fkey(v));
+      if (!many) few[atomicAdd(&S->count, 1u)] = v;
+    } else if (dv > d) {
+      above = min(above, fkey(v));
+    }
+  }
+  above = __reduce_min_sync(0xffffffffu, above);
+  if (lane == 0u) atomicMin(&S->next, above);
+  if (tid == 0u) {
+    S->digit = kNone;
+    S->rank = 0u;
+  }
+  __syncthreads();
+  if (many) {  // ties? one value in the whole step is the answer
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0u) {
+      atomicMin(&S->digit, kmin);
+      atomicMax(&S->rank, kmax);
+    }
+    __syncthreads();
+    const bool same = S->digit == S->rank;
+    *v1 = *v2 = fkey_inv(S->digit);
+    if (want_next && rr + 1u >= cnt) *v2 = fkey_inv(S->next);
+    const bool ok = same && (!want_next || rr + 1u < cnt || S->next != kNone);
+    __syncthreads();
+    return ok;
+  }
+  if (tid < cnt) {
+    const float v = few[tid];
+    unsigned k = 0u;  // its rank in the step, ties in the order of the list
+    for (unsigned j = 0; j < cnt; ++j) {
+      const float o = few[j];
+      k += (o < v || (o == v && j < tid)) ? 1u : 0u;
+    }
+    if (k == rr) S->digit = fkey(v);
+    if (k == rr + 1u) S->rank = fkey(v);
+  }
+  __syncthreads();
+  const unsigned k1 = S->digit, k2 = rr + 1u < cnt ? S->rank : S->next;
+  __syncthreads();
+  *v1 = fkey_inv(k1);
+  *v2 = want_next ? fkey_inv(k2) : *v1;
+  return !want_next || k2 != kNone;
+}
+
 }  // namespace flag
+
+// A block per channel: the bracket of its median.
+__global__ void __launch_bounds__(flag::kThreads, 1)
+    k_chan_sample(const float* __restrict__ cube, long long plane, flag::Chan* ch) {
+  using namespace flag;
+  __shared__ Scratch S;
+  float lo, hi;
+  plane_bracket<21>(cube + (long long)blockIdx.x * plane, plane, [](float x) { return x; }, KeyOfValue{}, &S, &lo, &hi);
+  if (threadIdx.x == 0) ch[blockIdx.x] = Chan{lo, hi, 0u, 0u, 0u, 0.0f, 0.0f, 0};
+}
+
+// A pass over the cube: the values (DEV: their |x - m|) of every channel under
+// its bracket counted and those inside copied to its list. A warp takes runs
+// of kPassRun consecutive values of a plane, its copies staged in shared memory.
+template <bool DEV>
+__global__ void __launch_bounds__(flag::kPassThreads, 4)
+    k_chan_pass(const float* __restrict__ cube, long long plane, int nz, flag::Chan* ch, float* __restrict__ lists,
+                long long room) {
+  using namespace flag;
+  __shared__ float stage[kPassWarps][kPassRun];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lanes_below = (1u << lane) - 1u;
+  const long long runs = (plane + kPassRun - 1) / kPassRun, total = runs * nz;
+  const long long warps = (long long)gridDim.x * kPassWarps;
+  const bool vec = (plane & 3) == 0 && (reinterpret_cast<uintptr_t>(cube) & 15u) == 0;
+  constexpr int kQ = kPassRun / 128;  // float4 loads a lane makes per run
+  for (long long it = (long long)blockIdx.x * kPassWarps + warp; it < total; it += warps) {
+    const int z = (int)(it / runs);
+    const long long p0 = (it - z * runs) * kPassRun;
+    const float* src = cube + z * plane + p0;
+    const int left = (int)min((long long)kPassRun, plane - p0);
+    const float lo = ch[z].lo, hi = ch[z].hi, ma = ch[z].ma, mb = ch[z].mb;
+    const bool even = ch[z].even != 0;
+    float v[kQ][4];
+    if (vec && left == kPassRun) {
+#pragma unroll
+      for (int q = 0; q < kQ; ++q) {
+        const float4 f = __ldg(reinterpret_cast<const float4*>(src) + 32 * q + lane);
+        v[q][0] = f.x, v[q][1] = f.y, v[q][2] = f.z, v[q][3] = f.w;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < kQ; ++q)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int i = 128 * q + 32 * c + lane;
+          v[q][c] = i < left ? __ldg(src + i) : __int_as_float(0x7fc00000);
+        }
+    }
+    unsigned finite = 0u, below = 0u;
+    int n = 0;
+#pragma unroll
+    for (int q = 0; q < kQ; ++q)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        float a = v[q][c];
+        const bool ok = fabsf(a) <= FLT_MAX;  // false for NaN and Inf
+        if (DEV) a = abs_dev(a, ma, mb, even);
+        if (!DEV) finite += ok ? 1u : 0u;
+        below += (ok && a < lo) ? 1u : 0u;
+        const bool in = ok && a >= lo && a <= hi;
+        const unsigned b = __ballot_sync(0xffffffffu, in);
+        if (in) stage[warp][n + __popc(b & lanes_below)] = a;
+        n += __popc(b);
+      }
+    finite = __reduce_add_sync(0xffffffffu, finite);
+    below = __reduce_add_sync(0xffffffffu, below);
+    unsigned at = 0u;
+    if (lane == 0) {
+      if (finite) atomicAdd(&ch[z].finite, finite);
+      if (below) atomicAdd(&ch[z].below, below);
+      if (n) at = atomicAdd(&ch[z].n, (unsigned)n);
+    }
+    at = __shfl_sync(0xffffffffu, at, 0);
+    __syncwarp();
+    float* out = lists + z * room;
+    for (int i = lane; i < n; i += 32)
+      if ((long long)at + i < room) out[at + i] = stage[warp][i];
+    __syncwarp();
+  }
+}
+
+// A block per channel: the median from its copies, and the bracket of the MAD
+// (DEV false); the MAD and the noise (DEV true). Without a usable bracket, by
+// radix passes over the plane.
+template <bool DEV>
+__global__ void __launch_bounds__(flag::kThreads, 1)
+    k_chan_select(const float* __restrict__ cube, long long plane, flag::Chan* ch, const float* __restrict__ lists,
+                  long long room, int mode, float* __restrict__ noise) {
+  using namespace flag;
+  __shared__ Scratch S;
+  __shared__ float few[kFew];
+  const int z = blockIdx.x;
+  const float* src = cube + (long long)z * plane;
+  const Chan c = ch[z];
+  if (c.finite == 0u) {  // no finite voxel: no noise (and no MAD pass to prepare)
+    if (DEV && threadIdx.x == 0) noise[z] = __int_as_float(0x7fc00000);
+    return;
+  }
+  const unsigned r1 = (c.finite - 1u) / 2u;
+  const bool even = (c.finite & 1u) == 0u;
+  float v1 = 0.0f, v2 = 0.0f;
+  bool done = (long long)c.n <= room && r1 >= c.below && r1 - c.below < c.n && c.hi > c.lo;
+  if (done) done = list_select(lists + z * room, c.n, c.lo, c.hi, r1 - c.below, even, &S, few, &v1, &v2);
+  if (!done) {
+    unsigned k2 = 0u;
+    if (DEV) {
+      const float ma = c.ma, mb = c.mb;
+      v1 = fkey_inv(stream_select(src, plane, r1, [=](float x) { return mad_key(x, ma, mb, even); }, &S, even, &k2));
+    } else {
+      v1 = fkey_inv(stream_select(src, plane, r1, [](float x) { return fkey(x); }, &S, even, &k2));
+    }
+    v2 = even ? fkey_inv(k2) : v1;
+  }
+  if (DEV) {
+    const double mad = even ? 0.5 * ((double)v1 + (double)v2) : (double)v1;
+    double sigma = kMadToSigma * mad;
+    if (mode == SC_NOISE_GAUSS && sigma > 0.0) {
+      __syncthreads();  // the selection is done with the scratch
+      sigma = block_gauss(src, plane, sigma, &S);
+    }
+    if (threadIdx.x == 0) noise[z] = __double2float_rn(sigma);
+  } else {
+    float lo, hi;
+    const float ma = v1, mb = v2;
+    __syncthreads();
+    plane_bracket<20>(src, plane, [=](float x) { return abs_dev(x, ma, mb, even); }, KeyOfDev{}, &S, &lo, &hi);
+    if (threadIdx.x == 0) ch[z] = Chan{fmaxf(lo, 0.0f), hi, c.finite, 0u, 0u, v1, v2, even ? 1 : 0};
+  }
+}
 
 __global__ void __launch_bounds__(flag::kThreads, 1)
     k_chan_noise(const float* __restrict__ cube, long long plane, int nz, int mode, float* __restrict__ noise) {
@@ -441,14 +757,45 @@ cudaError_t launch_pix(const float* cube, int nx, int ny, int nz, int mode, floa
 }
 }  // namespace
 
+// Room for the copies of one plane: a bracket holds about 6 % of it.
+static long long chan_room(long long plane) { return (plane / 8 + 4 + 3) & ~3LL; }
+
+size_t chan_scratch_bytes(const long long dims[3], int mode) {
+  const long long plane = dims[0] * dims[1];
+  if (mode == SC_NOISE_STD || plane < flag::kChanMinPlane || plane >= (1LL << 32)) return 0;
+  const size_t head = ((size_t)dims[2] * sizeof(flag::Chan) + 15) & ~(size_t)15;
+  return head + sizeof(float) * (size_t)chan_room(plane) * (size_t)dims[2];
+}
+
+static cudaError_t launch_chan_mad(const float* cube, long long plane, int nz, int mode, void* scratch, float* noise,
+                                   int sms, cudaStream_t s) {
+  flag::Chan* ch = static_cast<flag::Chan*>(scratch);
+  const size_t head = ((size_t)nz * sizeof(flag::Chan) + 15) & ~(size_t)15;
+  float* lists = reinterpret_cast<float*>(static_cast<unsigned char*>(scratch) + head);
+  const long long room = chan_room(plane);
+  const long long warps = (plane + flag::kPassRun - 1) / flag::kPassRun * nz;
+  const long long want = (warps + flag::kPassWarps - 1) / flag::kPassWarps;
+  const int grid = (int)(want < 4LL * sms ? want : 4LL * sms);
+  k_chan_sample<<<nz, flag::kThreads, 0, s>>>(cube, plane, ch);
+  k_chan_pass<false><<<grid, flag::kPassThreads, 0, s>>>(cube, plane, nz, ch, lists, room);
+  k_chan_select<false><<<nz, flag::kThreads, 0, s>>>(cube, plane, ch, lists, room, mode, noise);
+  k_chan_pass<true><<<grid, flag::kPassThreads, 0, s>>>(cube, plane, nz, ch, lists, room);
+  k_chan_select<true><<<nz, flag::kThreads, 0, s>>>(cube, plane, ch, lists, room, mode, noise);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k, int channels, int pixels,
                             int mode, float* out, float* chan_noise, float* pix_noise, uint8_t* chan_flags,
-                            uint8_t* pix_flags, double* stats, int sms, cudaStream_t s) {
+                            uint8_t* pix_flags, double* stats, void* chan_scratch, int sms, cudaStream_t s) {
   const int nx = (int)dims[0], ny = (int)dims[1], nz = (int)dims[2];
   const long long plane = (long long)nx * ny, n = plane * nz;
   cudaError_t e = cudaSuccess;
   if (channels) {
-    k_chan_noise<<<nz < 2 * sms ? nz : 2 * sms, flag::kThreads, 0, s>>>(cube, plane, nz, mode, chan_noise);
+    if (chan_scratch) {
+      if ((e = launch_chan_mad(cube, plane, nz, mode, chan_scratch, chan_noise, sms, s)) != cudaSuccess) return e;
+    } else {
+      k_chan_noise<<<nz < 2 * sms ? nz : 2 * sms, flag::kThreads, 0, s>>>(cube, plane, nz, mode, chan_noise);
+    }
     k_noise_stats<<<1, flag::kThreads, 0, s>>>(chan_noise, nz, stats);
     k_flag<<<(nz + 255) / 256, 256, 0, s>>>(chan_noise, nz, stats, k, chan_flags);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -378,7 +378,10 @@ cudaError_t launch_noise_apply(const float* cube, const long long dims[3], const
 constexpr int kFlagMaxChannelsForPixels = 1536;  // spectra staged in shared memory
 cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k, int channels, int pixels,
                             int noise_mode, float* out, float* chan_noise, float* pix_noise, uint8_t* chan_flags,
-                            uint8_t* pix_flags, double* stats, int sms, cudaStream_t s);
+                            uint8_t* pix_flags, double* stats, void* chan_scratch, int sms, cudaStream_t s);
+// Bytes of chan_scratch with which the channel noises take two passes over the
+// cube (0: they do not; null: one block per channel streams its plane).
+size_t chan_scratch_bytes(const long long dims[3], int mode);
 
 constexpr int kLinkMaxRadius = 32;  // merging radii in voxels
 long long link_chunks(long long n);
