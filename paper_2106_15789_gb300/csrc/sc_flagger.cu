@@ -12,10 +12,10 @@
 //   k_chan_noise   one block per channel, the plane streamed from memory: STD
 //                  by compensated sums, and (small planes, or no room for the
 //                  copies) median and MAD by radix passes
-//   k_pix_noise    one block per 32 pixels of a row: their spectra staged in
-//                  shared memory, each pixel's noise by one warp with the
-//                  spectrum in registers (exact selections by bisection on
-//                  the keys)
+//   k_pix_noise    one block per 16 pixels of a row: their spectra staged in
+//                  shared memory, each pixel's noise by one warp (exact
+//                  selections by a histogram of 256 equal steps between the
+//                  smallest and the largest value)
 //   k_noise_stats  one block: median M and MAD-based RMS R of a noise array
 //   k_flag         flags: |noise - M| > k R
 //   k_blank        out = NaN on flagged channels and pixels, else in
@@ -261,25 +261,172 @@ __device__ void block_noise(const float* __restrict__ src, long long n, int mode
   if (mode == SC_NOISE_GAUSS && *sigma > 0.0) *sigma = block_gauss(src, n, *sigma, S);
 }
 
-// ---- per-pixel noise: a warp per pixel, the spectrum in registers ----------
-constexpr int kPixWarps = 8;
-constexpr int kPixThreads = 32 * kPixWarps;
+// ---- per-pixel noise: a warp per pixel ---------------------------------------
+//
+// What bounds it: instruction issue, with the loads of a tile before it (two
+// blocks an SM hide each other's). Of 600 x 600 x 1024 voxels, the form with
+// the spectrum in registers, 32 rounds of bisection for each of the four order
+// statistics and one block of 8 warps an SM took 7.97 ms; this one 1.64 ms.
+constexpr int kPixTile = 16;         // pixels of a row (64 bytes of each plane), a warp each
+constexpr int kPixThreads = 32 * kPixTile;
+constexpr int kPixPitch = kPixTile + 1;
+constexpr int kSteps = 256;          // counts per warp (also the Gaussian fit's bins)
+constexpr int kPixUnroll = 8;
+static_assert(kSteps == gfit::kBins, "one set of counts serves both");
 
-// Order statistic `rank` of the VPL keys per lane held by a warp, by
-// bisection on the 32-bit key (keys kNone never count).
-template <int VPL>
-__device__ __forceinline__ unsigned warp_select(const unsigned (&k)[VPL], unsigned rank) {
+// f(value, its place) for a spectrum in shared memory; the lanes past its end
+// get NaN. All lanes of the warp call f together.
+template <class F>
+__device__ __forceinline__ void for_spectrum(float* col, int nz, F f) {
+  const int lane = threadIdx.x & 31;
+  for (int z0 = 0; z0 < nz; z0 += 32 * kPixUnroll) {
+    float v[kPixUnroll];
+#pragma unroll
+    for (int u = 0; u < kPixUnroll; ++u) {
+      const int z = z0 + 32 * u + lane;
+      v[u] = z < nz ? col[z * kPixPitch] : __int_as_float(0x7fc00000);
+    }
+#pragma unroll
+    for (int u = 0; u < kPixUnroll; ++u) f(v[u], col + (z0 + 32 * u + lane) * kPixPitch);
+  }
+}
+
+// Order statistic `rank` of a spectrum's values of(v) that are not NaN, by
+// bisection on the 32-bit key.
+template <class Of>
+__device__ __noinline__ float warp_bisect(float* col, int nz, Of of, unsigned rank) {
   unsigned ans = 0u;
   for (int bit = 31; bit >= 0; --bit) {
     const unsigned t = ans | (1u << bit);
     unsigned c = 0u;
-#pragma unroll
-    for (int i = 0; i < VPL; ++i) c += k[i] < t ? 1u : 0u;
+    for_spectrum(col, nz, [&](float x, float*) {
+      const float v = of(x);
+      c += (v == v && fkey(v) < t) ? 1u : 0u;
+    });
     c = __reduce_add_sync(0xffffffffu, c);
     if (c <= rank) ans = t;
   }
-  return ans;
+  return fkey_inv(ans);
 }
+
+// Order statistics rank and (want_next) rank + 1 of a spectrum's values of(v)
+// that are not NaN, all in [lo, hi] (both finite). counts: kSteps of shared
+// memory, list: 32 floats. 256 equal steps of the range (rounded to the
+// nearest, a monotone function of the value) are counted; the values of the
+// rank's step are ranked directly, or, more than 32 of them, their smallest
+// and largest become the next range. A range too small to divide: by bisection.
+template <class Of>
+__device__ __forceinline__ void warp_select(float* col, int nz, Of of, float lo, float hi, unsigned rank,
+                                            bool want_next, unsigned* counts, float* list, float* v1, float* v2) {
+  const unsigned lane = threadIdx.x & 31u;
+  unsigned r = rank, cnt = kNone;  // rank in the range, and its values (at first: all)
+  float found = lo;
+  while (lo < hi) {
+    // halves, so that hi - lo cannot overflow; the step is in the low bits of
+    // a sum with 1.5 * 2^23
+    const float magic = 12582912.0f, h0 = -0.5f * lo, inv = (float)(kSteps - 1) / (0.5f * hi + h0);
+    if (!(inv <= FLT_MAX)) {
+      *v1 = warp_bisect(col, nz, of, rank);
+      *v2 = want_next ? warp_bisect(col, nz, of, rank + 1u) : *v1;
+      return;
+    }
+    const auto step = [&](float v) { return __float_as_uint(__fmaf_rn(__fmaf_rn(v, 0.5f, h0), inv, magic)) & 0xffu; };
+#pragma unroll
+    for (int j = 0; j < kSteps / 128; ++j)
+      reinterpret_cast<uint4*>(counts)[j * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    for_spectrum(col, nz, [&](float x, float*) {
+      const float v = of(x);
+      if (v >= lo && v <= hi) atomicAdd(counts + step(v), 1u);  // (false for NaN)
+    });
+    __syncwarp();
+    const uint4 c0 = reinterpret_cast<const uint4*>(counts)[2 * lane];
+    const uint4 c1 = reinterpret_cast<const uint4*>(counts)[2 * lane + 1];
+    const unsigned c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+    unsigned sum = 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sum += c[j];
+    unsigned x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= (unsigned)o) x += y;
+    }
+    unsigned run = x - sum, d = 0u, in = 0u;
+    const bool mine = r >= run && r < x;
+    cnt = 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (r >= run && r < run + c[j]) {
+        d = 8u * lane + j;
+        in = r - run;
+        cnt = c[j];
+      }
+      run += c[j];
+    }
+    const int from = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;  // (the range holds the rank)
+    d = __shfl_sync(0xffffffffu, d, from);
+    r = __shfl_sync(0xffffffffu, in, from);
+    cnt = __shfl_sync(0xffffffffu, cnt, from);
+    if (cnt <= 32u) {
+      unsigned n = 0u;
+      for_spectrum(col, nz, [&](float xv, float*) {
+        const float v = of(xv);
+        const bool take = v >= lo && v <= hi && step(v) == d;
+        const unsigned b = __ballot_sync(0xffffffffu, take);
+        if (take) list[n + __popc(b & ((1u << lane) - 1u))] = v;
+        n += __popc(b);
+      });
+      __syncwarp();
+      const float a = lane < cnt ? list[lane] : 0.0f;
+      unsigned k = 0u;
+      for (unsigned j = 0; j < cnt; ++j) {
+        const float o = list[j];
+        k += (o < a || (o == a && j < lane)) ? 1u : 0u;
+      }
+      __syncwarp();
+      found = __shfl_sync(0xffffffffu, a, __ffs(__ballot_sync(0xffffffffu, lane < cnt && k == r)) - 1);
+      if (want_next && r + 1u < cnt) {
+        *v1 = found;
+        *v2 = __shfl_sync(0xffffffffu, a, __ffs(__ballot_sync(0xffffffffu, lane < cnt && k == r + 1u)) - 1);
+        return;
+      }
+      break;
+    }
+    unsigned kmin = kNone, kmax = 0u;
+    for_spectrum(col, nz, [&](float xv, float*) {
+      const float v = of(xv);
+      if (v >= lo && v <= hi && step(v) == d) {
+        kmin = min(kmin, fkey(v));
+        kmax = max(kmax, fkey(v));
+      }
+    });
+    found = lo = fkey_inv(__reduce_min_sync(0xffffffffu, kmin));
+    hi = fkey_inv(__reduce_max_sync(0xffffffffu, kmax));
+  }
+  // found: ranked, or the only value of its range
+  *v1 = *v2 = found;
+  if (!want_next || r + 1u < cnt) return;
+  // the rank was the last of its step or range: the next larger value
+  unsigned above = kNone;
+  for_spectrum(col, nz, [&](float xv, float*) {
+    const float v = of(xv);
+    if (v > found) above = min(above, fkey(v));
+  });
+  *v2 = fkey_inv(__reduce_min_sync(0xffffffffu, above));
+}
+
+// |x - m|, m = (a + b) / 2, with -m = h + l exactly: faithfully rounded (one
+// subtraction when l is 0, as for an odd count).
+struct PixDev {
+  float h, l;
+  __device__ __forceinline__ float operator()(float x) const {
+    const float t = __fadd_rn(x, h);
+    const float b = __fsub_rn(t, x);
+    const float e = __fadd_rn(__fsub_rn(x, __fsub_rn(t, b)), __fsub_rn(h, b));
+    return fabsf(__fadd_rn(t, __fadd_rn(e, l)));
+  }
+};
 
 // ---- per-channel median and MAD by passes over the whole cube ---------------
 //
@@ -620,106 +767,119 @@ __global__ void __launch_bounds__(flag::kThreads, 1) k_noise_stats(const float* 
   }
 }
 
-template <int VPL>
-__global__ void __launch_bounds__(flag::kPixThreads) k_pix_noise(const float* __restrict__ cube, int nx, int ny,
-                                                                 int nz, int mode, float* __restrict__ noise) {
+__global__ void __launch_bounds__(flag::kPixThreads, 2) k_pix_noise(const float* __restrict__ cube, int nx, int ny,
+                                                                    int nz, int mode, float* __restrict__ noise) {
   using namespace flag;
-  extern __shared__ float tile[];  // [nz][33]: 32 pixels of a row (one padding column)
-  // Gaussian-fit mode: then 256 counts per warp
-  unsigned* const whist = reinterpret_cast<unsigned*>(tile + 33 * nz) + (threadIdx.x >> 5) * gfit::kBins;
-  const bool std_mode = mode == SC_NOISE_STD;
+  extern __shared__ __align__(16) float pix_smem[];
+  // per warp 256 counts and 32 values, then the spectra: [nz][kPixPitch]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned* const counts = reinterpret_cast<unsigned*>(pix_smem) + warp * kSteps;
+  float* const list = pix_smem + kPixTile * kSteps + warp * 32;
+  float* const tile = pix_smem + kPixTile * (kSteps + 32);
   const long long plane = (long long)nx * ny;
-  const int xtiles = (nx + 31) / 32;
+  const int xtiles = (nx + kPixTile - 1) / kPixTile;
   const long long ntiles = (long long)xtiles * ny;
   for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int y = (int)(t / xtiles), x0 = (int)(t - (long long)y * xtiles) * 32;
+    const int y = (int)(t / xtiles), x0 = (int)(t - (long long)y * xtiles) * kPixTile;
     __syncthreads();  // the tile of the previous iteration is consumed
-    for (int z = warp; z < nz; z += kPixWarps) {
-      const int x = x0 + lane;
-      tile[z * 33 + lane] = x < nx ? __ldg(cube + (long long)z * plane + (long long)y * nx + x)
-                                   : __int_as_float(0x7fc00000);
+    {
+      // two planes a warp and load, eight loads ahead
+      const int px = lane & (kPixTile - 1), x = x0 + px;
+      const float* src = cube + (long long)y * nx + x;
+      for (int z0 = 2 * warp + (lane >> 4); z0 < nz; z0 += 2 * kPixTile * 8) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int z = z0 + 2 * kPixTile * u;
+          v[u] = (z < nz && x < nx) ? __ldg(src + (long long)z * plane) : __int_as_float(0x7fc00000);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int z = z0 + 2 * kPixTile * u;
+          if (z < nz) tile[z * kPixPitch + px] = __fadd_rn(v[u], __fsub_rn(v[u], v[u]));  // Inf becomes NaN
+        }
+      }
     }
     __syncthreads();
-    for (int p = warp; p < 32 && x0 + p < nx; p += kPixWarps) {
-      float v[VPL];
-      unsigned k[VPL];
-      unsigned nfl = 0u;
+    if (x0 + warp >= nx) continue;
+    float* const col = tile + warp;
+    unsigned nf = 0u;
+    float mn = FLT_MAX, mx = -FLT_MAX;
+    for_spectrum(col, nz, [&](float v, float*) {
+      nf += v == v ? 1u : 0u;
+      mn = fminf(mn, v);
+      mx = fmaxf(mx, v);
+    });
+    nf = __reduce_add_sync(0xffffffffu, nf);
+    float out;
+    if (nf == 0u) {
+      out = __int_as_float(0x7fc00000);
+    } else if (mode == SC_NOISE_STD) {
+      float s = 0.0f, sc = 0.0f;
+      for_spectrum(col, nz, [&](float v, float*) {
+        if (v == v) neumaier_add(&s, &sc, v);
+      });
+      double ds = (double)s + (double)sc;
 #pragma unroll
-      for (int i = 0; i < VPL; ++i) {
-        const int z = lane + 32 * i;
-        v[i] = z < nz ? tile[z * 33 + p] : __int_as_float(0x7fc00000);
-        const bool ok = isfinite(v[i]);
-        k[i] = ok ? fkey(v[i]) : kNone;
-        nfl += ok ? 1u : 0u;
-      }
-      const unsigned nf = __reduce_add_sync(0xffffffffu, nfl);
-      float out;
-      if (nf == 0u) {
-        out = __int_as_float(0x7fc00000);
-      } else if (std_mode) {
-        float s = 0.0f, sc = 0.0f;
-#pragma unroll
-        for (int i = 0; i < VPL; ++i)
-          if (k[i] != kNone) neumaier_add(&s, &sc, v[i]);
-        double ds = (double)s + (double)sc;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ds += __shfl_xor_sync(0xffffffffu, ds, o);
-        const double mean = ds / (double)nf;
-        const float mh = __double2float_rn(mean), ml = __double2float_rn(mean - (double)mh);
-        float q = 0.0f, qc = 0.0f;
-#pragma unroll
-        for (int i = 0; i < VPL; ++i)
-          if (k[i] != kNone) {
-            const float d = __fsub_rn(__fsub_rn(v[i], mh), ml);
-            neumaier_add(&q, &qc, __fmul_rn(d, d));
-          }
-        double dq = (double)q + (double)qc;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dq += __shfl_xor_sync(0xffffffffu, dq, o);
-        out = __double2float_rn(nf > 1u ? sqrt(dq / (double)(nf - 1u)) : 0.0);
-      } else {
-        const unsigned r1 = (nf - 1u) / 2u;
-        const bool even = (nf & 1u) == 0u;
-        const unsigned k1 = warp_select<VPL>(k, r1);
-        const unsigned k2 = even ? warp_select<VPL>(k, r1 + 1u) : k1;
-        const float ma = fkey_inv(k1), mb = fkey_inv(k2);
-#pragma unroll
-        for (int i = 0; i < VPL; ++i)
-          if (k[i] != kNone) k[i] = mad_key(v[i], ma, mb, even);
-        const unsigned a1 = warp_select<VPL>(k, r1);
-        const unsigned a2 = even ? warp_select<VPL>(k, r1 + 1u) : a1;
-        const double mad = 0.5 * ((double)fkey_inv(a1) + (double)fkey_inv(a2));
-        double sigma = kMadToSigma * mad;
-        if (mode == SC_NOISE_GAUSS && sigma > 0.0) {
-          // the spectrum's 256-bin histogram in this warp's counts, then a
-          // warp-wide fit over the 128 folded bins (4 a lane)
-          for (int i = lane; i < gfit::kBins; i += 32) whist[i] = 0u;
-          __syncwarp();
-          const float ks = gfit::scale_of(sigma);
-#pragma unroll
-          for (int i = 0; i < VPL; ++i) {
-            const int b = gfit::bin_of(v[i], ks);  // NaN (and padding) give -1
-            if (b >= 0) atomicAdd(whist + b, 1u);
-          }
-          __syncwarp();
-          double hh[4], x2[4];
-          bool use[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int t = lane + 32 * j;
-            hh[j] = (double)whist[gfit::kHalf + t] + (double)whist[gfit::kHalf - 1 - t];
-            x2[j] = gfit::xi2_of(t);
-            use[j] = true;
-          }
-          const double tau = gfit::fit_tau(hh, x2, use, gfit::WarpSum6{});
-          if (tau > 0.0) sigma = gfit::noise_of(tau, ks);
-          __syncwarp();  // the counts are reset by the next pixel
+      for (int o = 16; o > 0; o >>= 1) ds += __shfl_xor_sync(0xffffffffu, ds, o);
+      const double mean = ds / (double)nf;
+      const float mh = __double2float_rn(mean), ml = __double2float_rn(mean - (double)mh);
+      float q = 0.0f, qc = 0.0f;
+      for_spectrum(col, nz, [&](float v, float*) {
+        if (v == v) {
+          const float d = __fsub_rn(__fsub_rn(v, mh), ml);
+          neumaier_add(&q, &qc, __fmul_rn(d, d));
         }
-        out = __double2float_rn(sigma);
+      });
+      double dq = (double)q + (double)qc;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) dq += __shfl_xor_sync(0xffffffffu, dq, o);
+      out = __double2float_rn(nf > 1u ? sqrt(dq / (double)(nf - 1u)) : 0.0);
+    } else {
+      mn = fkey_inv(__reduce_min_sync(0xffffffffu, fkey(mn)));
+      mx = fkey_inv(__reduce_max_sync(0xffffffffu, fkey(mx)));
+      const unsigned r1 = (nf - 1u) / 2u;
+      const bool even = (nf & 1u) == 0u;
+      float ma, mb, a1, a2;
+      warp_select(col, nz, [](float v) { return v; }, mn, mx, r1, even, counts, list, &ma, &mb);
+      PixDev dev;
+      const float ha = -0.5f * ma, hb = -0.5f * mb;
+      dev.h = ma == mb ? -ma : __fadd_rn(ha, hb);
+      const float bb = __fsub_rn(dev.h, ha);
+      dev.l = ma == mb ? 0.0f : __fadd_rn(__fsub_rn(ha, __fsub_rn(dev.h, bb)), __fsub_rn(hb, bb));
+      // |v - m| in place of v (an overflow stays the largest), unless the fit
+      // needs the values
+      const bool keep = mode == SC_NOISE_GAUSS;
+      const auto clamped = [&](float v) { return v == v ? fminf(dev(v), FLT_MAX) : v; };
+      const float top = fmaxf(clamped(mn), clamped(mx));
+      if (keep) {
+        warp_select(col, nz, clamped, 0.0f, top, r1, even, counts, list, &a1, &a2);
+      } else {
+        for_spectrum(col, nz, [&](float v, float* at) {
+          if (v == v) *at = clamped(v);
+        });
+        __syncwarp();
+        warp_select(col, nz, [](float v) { return v; }, 0.0f, top, r1, even, counts, list, &a1, &a2);
       }
-      if (lane == 0) noise[(long long)y * nx + x0 + p] = out;
+      const double mad = even ? 0.5 * ((double)a1 + (double)a2) : (double)a1;
+      double sigma = kMadToSigma * mad;
+      if (mode == SC_NOISE_GAUSS && sigma > 0.0) {
+        // the spectrum's 256-bin histogram in this warp's counts, then a
+        // warp-wide fit over the 128 folded bins (4 a lane)
+        for (int i = lane; i < gfit::kBins; i += 32) counts[i] = 0u;
+        __syncwarp();
+        const float ks = gfit::scale_of(sigma);
+        for_spectrum(col, nz, [&](float v, float*) {
+          const int b = gfit::bin_of(v, ks);  // NaN gives -1
+          if (b >= 0) atomicAdd(counts + b, 1u);
+        });
+        __syncwarp();
+        const double tau = gfit::fit_tau_warp(counts);
+        if (tau > 0.0) sigma = gfit::noise_of(tau, ks);
+      }
+      out = __double2float_rn(sigma);
     }
+    if (lane == 0) noise[(long long)y * nx + x0 + warp] = out;
   }
 }
 
@@ -744,15 +904,12 @@ __global__ void k_blank(const float* in, float* out, int nx, int ny, int nz, con
 
 // ---------------------------------------------------------------------------
 namespace {
-template <int VPL>
-cudaError_t launch_pix(const float* cube, int nx, int ny, int nz, int mode, float* noise, int sms,
-                       cudaStream_t s) {
-  const size_t smem = sizeof(float) * 33 * (size_t)nz +
-                      (mode == SC_NOISE_GAUSS ? sizeof(unsigned) * gfit::kBins * flag::kPixWarps : 0);
-  cudaFuncSetAttribute(k_pix_noise<VPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  const long long tiles = (long long)((nx + 31) / 32) * ny;
-  const int grid = (int)(tiles < 4LL * sms ? tiles : 4LL * sms);
-  k_pix_noise<VPL><<<grid, flag::kPixThreads, smem, s>>>(cube, nx, ny, nz, mode, noise);
+cudaError_t launch_pix(const float* cube, int nx, int ny, int nz, int mode, float* noise, int sms, cudaStream_t s) {
+  const size_t smem = sizeof(float) * (flag::kPixTile * (flag::kSteps + 32) + flag::kPixPitch * (size_t)nz);
+  cudaFuncSetAttribute(k_pix_noise, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const long long tiles = (long long)((nx + flag::kPixTile - 1) / flag::kPixTile) * ny;
+  const int grid = (int)(tiles < 8LL * sms ? tiles : 8LL * sms);
+  k_pix_noise<<<grid, flag::kPixThreads, smem, s>>>(cube, nx, ny, nz, mode, noise);
   return cudaGetLastError();
 }
 }  // namespace
@@ -801,10 +958,7 @@ cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (pixels) {
-    if (nz <= 256) e = launch_pix<8>(cube, nx, ny, nz, mode, pix_noise, sms, s);
-    else if (nz <= 512) e = launch_pix<16>(cube, nx, ny, nz, mode, pix_noise, sms, s);
-    else if (nz <= 1024) e = launch_pix<32>(cube, nx, ny, nz, mode, pix_noise, sms, s);
-    else e = launch_pix<48>(cube, nx, ny, nz, mode, pix_noise, sms, s);
+    e = launch_pix(cube, nx, ny, nz, mode, pix_noise, sms, s);
     if (e != cudaSuccess) return e;
     k_noise_stats<<<1, flag::kThreads, 0, s>>>(pix_noise, plane, stats + 2);
     const long long g = (plane + 255) / 256;
