@@ -16,7 +16,7 @@
 //                  shared memory, each pixel's noise by one warp (exact
 //                  selections by a histogram of 256 equal steps between the
 //                  smallest and the largest value)
-//   k_noise_stats  one block: median M and MAD-based RMS R of a noise array
+//   k_array_stats  (sc_select.cu) median M and MAD-based RMS R of a noise array
 //   k_flag         flags: |noise - M| > k R
 //   k_blank        out = NaN on flagged channels and pixels, else in
 //
@@ -754,19 +754,6 @@ __global__ void __launch_bounds__(flag::kThreads, 1)
   }
 }
 
-// stats[0] = median M, stats[1] = R = 1.4826 * MAD of the finite noises
-// (NaN if none).
-__global__ void __launch_bounds__(flag::kThreads, 1) k_noise_stats(const float* __restrict__ noise, long long n,
-                                                                   double* stats) {
-  __shared__ flag::Scratch S;
-  double sigma, m;
-  flag::block_noise(noise, n, SC_NOISE_MAD, &S, &sigma, &m);
-  if (threadIdx.x == 0) {
-    stats[0] = m;
-    stats[1] = sigma;
-  }
-}
-
 __global__ void __launch_bounds__(flag::kPixThreads, 2) k_pix_noise(const float* __restrict__ cube, int nx, int ny,
                                                                     int nz, int mode, float* __restrict__ noise) {
   using namespace flag;
@@ -892,13 +879,48 @@ __global__ void k_flag(const float* __restrict__ noise, long long n, const doubl
   }
 }
 
-__global__ void k_blank(const float* in, float* out, int nx, int ny, int nz, const uint8_t* __restrict__ fchan,
-                        const uint8_t* __restrict__ fpix) {
-  const long long plane = (long long)nx * ny, n = plane * nz;
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-    const long long z = v / plane, p = v - z * plane;
-    const bool f = (fchan && fchan[z]) || (fpix && fpix[p]);
-    out[v] = f ? __int_as_float(0x7fc00000) : in[v];
+// A thread keeps its pixels (VEC: four, else one) and goes through kBlankRun
+// planes, four loads ahead. HBM-bound: 8 bytes a voxel; with a 64-bit division
+// and a 4-byte load and store per voxel 600 x 600 x 1024 voxels took 1.03 ms,
+// now 0.42 ms. out may be in.
+constexpr int kBlankRun = 16;
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_blank(const float* in, float* out, long long plane, int nz,
+                                               const uint8_t* __restrict__ fchan, const uint8_t* __restrict__ fpix) {
+  constexpr int kW = VEC ? 4 : 1;
+  const long long q = blockIdx.x * 256LL + threadIdx.x;
+  if (q * kW >= plane) return;
+  const float qnan = __int_as_float(0x7fc00000);
+  bool pix[kW];
+#pragma unroll
+  for (int c = 0; c < kW; ++c) pix[c] = fpix && fpix[q * kW + c];
+  for (long long z1 = blockIdx.y * (long long)kBlankRun; z1 < nz; z1 += gridDim.y * (long long)kBlankRun) {
+    for (int z0 = 0; z0 < kBlankRun && z1 + z0 < nz; z0 += 4) {
+      float v[4][kW];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const long long z = z1 + z0 + u;
+        if (z >= nz) break;
+        const float* src = in + z * plane + q * kW;
+        if constexpr (VEC) {
+          const float4 f = *reinterpret_cast<const float4*>(src);
+          v[u][0] = f.x, v[u][1] = f.y, v[u][2] = f.z, v[u][3] = f.w;
+        } else {
+          v[u][0] = *src;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const long long z = z1 + z0 + u;
+        if (z >= nz) break;
+        const bool ch = fchan && __ldg(fchan + z);
+#pragma unroll
+        for (int c = 0; c < kW; ++c) v[u][c] = ch || pix[c] ? qnan : v[u][c];
+        float* dst = out + z * plane + q * kW;
+        if constexpr (VEC) *reinterpret_cast<float4*>(dst) = make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
+        else *dst = v[u][0];
+      }
+    }
   }
 }
 
@@ -945,7 +967,7 @@ cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k
                             int mode, float* out, float* chan_noise, float* pix_noise, uint8_t* chan_flags,
                             uint8_t* pix_flags, double* stats, void* chan_scratch, int sms, cudaStream_t s) {
   const int nx = (int)dims[0], ny = (int)dims[1], nz = (int)dims[2];
-  const long long plane = (long long)nx * ny, n = plane * nz;
+  const long long plane = (long long)nx * ny;
   cudaError_t e = cudaSuccess;
   if (channels) {
     if (chan_scratch) {
@@ -953,22 +975,25 @@ cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k
     } else {
       k_chan_noise<<<nz < 2 * sms ? nz : 2 * sms, flag::kThreads, 0, s>>>(cube, plane, nz, mode, chan_noise);
     }
-    k_noise_stats<<<1, flag::kThreads, 0, s>>>(chan_noise, nz, stats);
+    if ((e = launch_array_stats(chan_noise, nz, stats, s)) != cudaSuccess) return e;
     k_flag<<<(nz + 255) / 256, 256, 0, s>>>(chan_noise, nz, stats, k, chan_flags);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (pixels) {
     e = launch_pix(cube, nx, ny, nz, mode, pix_noise, sms, s);
     if (e != cudaSuccess) return e;
-    k_noise_stats<<<1, flag::kThreads, 0, s>>>(pix_noise, plane, stats + 2);
+    if ((e = launch_array_stats(pix_noise, plane, stats + 2, s)) != cudaSuccess) return e;
     const long long g = (plane + 255) / 256;
     k_flag<<<(unsigned)(g < 16LL * sms ? g : 16LL * sms), 256, 0, s>>>(pix_noise, plane, stats + 2, k, pix_flags);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  const long long gb = (n + 255) / 256;
-  k_blank<<<(unsigned)(gb < 16LL * sms ? gb : 16LL * sms), 256, 0, s>>>(cube, out, nx, ny, nz,
-                                                                      channels ? chan_flags : nullptr,
-                                                                      pixels ? pix_flags : nullptr);
+  const uint8_t* const fc = channels ? chan_flags : nullptr;
+  const uint8_t* const fp = pixels ? pix_flags : nullptr;
+  const bool vec = plane % 4 == 0 && ((reinterpret_cast<uintptr_t>(cube) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
+  const long long bx = ((vec ? plane / 4 : plane) + 255) / 256, by = (nz + kBlankRun - 1) / kBlankRun;
+  const dim3 grid((unsigned)bx, (unsigned)(by < 65535 ? by : 65535));
+  if (vec) k_blank<true><<<grid, 256, 0, s>>>(cube, out, plane, nz, fc, fp);
+  else k_blank<false><<<grid, 256, 0, s>>>(cube, out, plane, nz, fc, fp);
   return cudaGetLastError();
 }
 

@@ -319,6 +319,8 @@ constexpr long long kSelectGridMin = 1LL << 26;
 cudaError_t launch_select_lists(DevState* st, const float* src, long long n, Lists L, int pair, int sms,
                                 cudaStream_t s, int* launches);
 void init_select_attrs();
+// stats[0] = median, stats[1] = 1.4826 MAD of the finite values of x[0 .. n) (NaN if none).
+cudaError_t launch_array_stats(const float* x, long long n, double* stats, cudaStream_t s);
 cudaError_t launch_select_full(DevState* st, int which, int pair, int sms, cudaStream_t s);
 // The clip of the voxels that the candidate pass left undecided, or of all by a full pass.
 cudaError_t launch_clip(const float* src, long long n, uint32_t* mbits, DevState* st, Lists L, int sms,
