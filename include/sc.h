@@ -461,16 +461,16 @@ int sc_noise_scale(sc_ctx *ctx, const float *cube_dev, const int64_t *dims, cons
  *   dims         {nx, ny, nz}; nx * ny * nz < 2^31 - 1 (int32 voxel indices).
  *   r_xy, r_z    merging radii in voxels, 0 .. 32.
  *   labels_dev   int32 [nz][ny][nx] device buffer (caller-owned, output): the
- *                detection id of every voxel, 0 for none. Also the
- *                union-find workspace, so it may not alias mask_dev.
+ *                detection id of every voxel, 0 for none. It may not alias
+ *                mask_dev.
  *   *n_out       number of kept detections.
  *   extents_host NULL or int32[extents_cap][7]: for detections 1 .. n (the
  *                first extents_cap of them) x_min, x_max, y_min, y_max,
  *                z_min, z_max and the voxel count.
  *   flags        reserved, pass 0.
- * The library keeps per-chunk and per-detection buffers in the context (grown
- * on demand). Synchronises the stream (the number of detections sizes the
- * second half). Errors: SC_ERR_ARG (NULL pointer, dims, radii, negative
+ * The library keeps buffers in the context (grown on demand): 5/16 byte per
+ * voxel, 8 bytes per run of mask voxels along x, 64 per detection. Synchronises
+ * the stream (the numbers of runs and detections size the later parts). Errors: SC_ERR_ARG (NULL pointer, dims, radii, negative
  * limits), SC_ERR_NOMEM, SC_ERR_CUDA. */
 int sc_link(sc_ctx *ctx, const uint8_t *mask_dev, const int64_t *dims, int r_xy, int r_z, int min_xy, int min_z,
             int max_xy, int max_z, int32_t *labels_dev, int64_t *n_out, int32_t *extents_host, int64_t extents_cap,

@@ -45,11 +45,9 @@ struct sc_ctx {
   double* ns_sig = nullptr;      // sc_noise_scale: noise of every cell (lazy, grown)
   float* ns_rinv = nullptr;      // and its float reciprocal
   size_t ns_cap = 0;             // cells both hold
-  int* lk_chunk = nullptr;       // sc_link: per-chunk root counts / offsets (lazy, grown)
-  size_t lk_chunk_cap = 0;
   int* lk_tot = nullptr;         // sc_link: one device int (a total)
-  int* lk_comp = nullptr;        // sc_link: [4 arrays of cap][7 or 1 ints] per detection
-  size_t lk_comp_cap = 0;
+  void *lk_bits = nullptr, *lk_runs = nullptr, *lk_comp = nullptr;  // the mask's bits, runs, detections (lazy, grown)
+  size_t lk_bits_cap = 0, lk_runs_cap = 0, lk_comp_cap = 0;
   unsigned char* af_buf = nullptr;  // sc_autoflag: noises, flags and statistics (lazy, grown)
   size_t af_cap = 0;
   void* af_chan = nullptr;          // and its channel passes' brackets and copies (lazy, grown)
@@ -446,6 +444,21 @@ uint32_t half_flags(uint32_t flags) {
   return (flags & (SC_FLAG_GENERIC | SC_FLAG_SAMPLED_GAUSS)) ? flags & ~(uint32_t)SC_FLAG_HALF_DIRECT : flags;
 }
 
+// Grows a device buffer of the context (its contents are not kept).
+int ensure_bytes(void** p, size_t* cap, size_t need) {
+  if (need <= *cap) return SC_OK;
+  cudaFree(*p);
+  *p = nullptr;
+  *cap = 0;
+  if (cudaMalloc(p, need) != cudaSuccess) {
+    cudaGetLastError();
+    *p = nullptr;
+    return SC_ERR_NOMEM;
+  }
+  *cap = need;
+  return SC_OK;
+}
+
 // Device staging cube and mask of max_voxels elements (allocated on first use).
 int ensure_stage(sc_ctx* c) {
   if (c->stage_cube) return SC_OK;
@@ -765,7 +778,8 @@ void sc_destroy(sc_ctx* c) {
   cudaFree(c->stage_mask);
   cudaFree(c->ns_sig);
   cudaFree(c->ns_rinv);
-  cudaFree(c->lk_chunk);
+  cudaFree(c->lk_bits);
+  cudaFree(c->lk_runs);
   cudaFree(c->lk_tot);
   cudaFree(c->lk_comp);
   cudaFree(c->af_chan);
@@ -1620,57 +1634,49 @@ int sc_link(sc_ctx* c, const uint8_t* mask_dev, const int64_t* dims, int r_xy, i
   DeviceGuard guard(c->device);
   cudaStream_t s = (cudaStream_t)cuda_stream;
   c->last = s;
-  const long long chunks = link_chunks(n);
   if (!c->lk_tot && cudaMalloc(&c->lk_tot, sizeof(int) * 2) != cudaSuccess) {
     cudaGetLastError();
     c->lk_tot = nullptr;
     return SC_ERR_NOMEM;
   }
-  if ((size_t)chunks > c->lk_chunk_cap) {
-    cudaFree(c->lk_chunk);
-    c->lk_chunk_cap = 0;
-    if (cudaMalloc(&c->lk_chunk, sizeof(int) * chunks) != cudaSuccess) {
-      cudaGetLastError();
-      c->lk_chunk = nullptr;
-      return SC_ERR_NOMEM;
-    }
-    c->lk_chunk_cap = (size_t)chunks;
+  int rc = ensure_bytes(&c->lk_bits, &c->lk_bits_cap, link_bits_bytes(n));
+  if (rc) return rc;
+  CK(launch_link_runs(mask_dev, d, r_xy, r_z, c->lk_bits, c->lk_tot, s));
+  c->stats.launches += 2;
+  int nruns = 0, ncomp = 0;
+  CK(cudaMemcpyAsync(&nruns, c->lk_tot, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  if (nruns == 0) {  // an empty mask
+    CK(cudaMemsetAsync(labels_dev, 0, sizeof(int) * (size_t)n, s));
+    CK(cudaStreamSynchronize(s));
+    *n_out = 0;
+    return SC_OK;
   }
-  CK(launch_link_components(mask_dev, d, r_xy, r_z, labels_dev, c->lk_chunk, c->lk_tot, c->sms, s));
+  rc = ensure_bytes(&c->lk_runs, &c->lk_runs_cap, link_runs_bytes(nruns));
+  if (rc) return rc;
+  int* const runs = static_cast<int*>(c->lk_runs);
+  CK(launch_link_components(d, r_xy, r_z, c->lk_bits, nruns, runs, c->lk_tot, c->sms, s));
   c->stats.launches += 4;
-  int ncomp = 0;
   CK(cudaMemcpyAsync(&ncomp, c->lk_tot, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   int kept = 0;
-  int *ext = nullptr, *ext_out = nullptr, *keep = nullptr, *new_id = nullptr;
-  if (ncomp > 0) {
-    if ((size_t)ncomp > c->lk_comp_cap) {
-      cudaFree(c->lk_comp);
-      c->lk_comp_cap = 0;
-      if (cudaMalloc(&c->lk_comp, sizeof(int) * 16 * (size_t)ncomp) != cudaSuccess) {
-        cudaGetLastError();
-        c->lk_comp = nullptr;
-        return SC_ERR_NOMEM;
-      }
-      c->lk_comp_cap = (size_t)ncomp;
-    }
-    ext = c->lk_comp;
-    ext_out = ext + 7 * (size_t)ncomp;
-    keep = ext_out + 7 * (size_t)ncomp;
-    new_id = keep + (size_t)ncomp;
-  }
-  // numbering, final labels and extents, then the size filters
-  CK(launch_link_filter(d, labels_dev, c->lk_chunk, ncomp, min_xy, min_z, max_xy, max_z, ext, keep, ext_out, new_id,
-                        c->lk_tot, c->sms, s));
-  c->stats.launches += ncomp > 0 ? 7 : 2;
-  if (ncomp > 0) {
-    CK(cudaMemcpyAsync(&kept, c->lk_tot, sizeof(int), cudaMemcpyDeviceToHost, s));
+  // per detection: two extents rows of 7, a keep flag and a new id
+  rc = ensure_bytes(&c->lk_comp, &c->lk_comp_cap, sizeof(int) * 16 * (size_t)ncomp);
+  if (rc) return rc;
+  int* const ext = static_cast<int*>(c->lk_comp);
+  int* const ext_out = ext + 7 * (size_t)ncomp;
+  int* const keep = ext_out + 7 * (size_t)ncomp;
+  int* const new_id = keep + (size_t)ncomp;
+  // numbering and extents, the size filters, the labels
+  CK(launch_link_filter(d, r_xy, c->lk_bits, nruns, runs, ncomp, min_xy, min_z, max_xy, max_z, ext, keep, ext_out,
+                        new_id, c->lk_tot, labels_dev, c->sms, s));
+  c->stats.launches += 7;
+  CK(cudaMemcpyAsync(&kept, c->lk_tot, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  const long long table = std::min<long long>(kept, extents_cap);
+  if (table > 0) {
+    CK(cudaMemcpyAsync(extents_host, ext_out, sizeof(int) * 7 * (size_t)table, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
-    const long long rows = std::min<long long>(kept, extents_cap);
-    if (rows > 0) {
-      CK(cudaMemcpyAsync(extents_host, ext_out, sizeof(int) * 7 * (size_t)rows, cudaMemcpyDeviceToHost, s));
-      CK(cudaStreamSynchronize(s));
-    }
   }
   *n_out = kept;
   return SC_OK;

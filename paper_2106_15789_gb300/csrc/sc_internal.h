@@ -371,10 +371,6 @@ cudaError_t launch_noise_window(const float* cube, const long long dims[3], cons
 cudaError_t launch_noise_apply(const float* cube, const long long dims[3], const int window[3], const int grid[3],
                                float* out, const float* rinv_dev, int sms, cudaStream_t s);
 
-// Linker: components (lab = roots; chunk_off = exclusive scan of the roots
-// per chunk; *d_total = their number), then ids in raster order of the first
-// voxels with extents, and the size filters (lab renumbered, ext_out = kept
-// rows, *d_total = kept). ext etc. may be null when there is no component.
 // Auto-flagger: channel and pixel noises, their median / RMS (stats[0..1]
 // channels, [2..3] pixels), flags and the blanked cube.
 constexpr int kFlagMaxChannelsForPixels = 1536;  // spectra staged in shared memory
@@ -386,12 +382,19 @@ cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k
 size_t chan_scratch_bytes(const long long dims[3], int mode);
 
 constexpr int kLinkMaxRadius = 32;  // merging radii in voxels
-long long link_chunks(long long n);
-cudaError_t launch_link_components(const uint8_t* mask, const long long dims[3], int r_xy, int r_z, int* lab,
-                                   int* chunk_off, int* d_total, int sms, cudaStream_t s);
-cudaError_t launch_link_filter(const long long dims[3], int* lab, int* chunk_off, int ncomp, int min_xy, int min_z,
-                               int max_xy, int max_z, int* ext, int* keep, int* ext_out, int* new_id, int* d_total,
-                               int sms, cudaStream_t s);
+// Linker, in three steps: the mask as bits and runs (bits: link_bits_bytes of
+// scratch; *d_total = the number of runs), their components (runs:
+// link_runs_bytes of scratch; *d_total = their number), then the extents, the
+// size filters (ext_out = kept rows, *d_total = kept) and the labels.
+size_t link_bits_bytes(long long n);
+size_t link_runs_bytes(long long nruns);
+cudaError_t launch_link_runs(const uint8_t* mask, const long long dims[3], int r_xy, int r_z, void* bits, int* d_total,
+                             cudaStream_t s);
+cudaError_t launch_link_components(const long long dims[3], int r_xy, int r_z, void* bits, long long nruns, int* runs,
+                                   int* d_total, int sms, cudaStream_t s);
+cudaError_t launch_link_filter(const long long dims[3], int r_xy, void* bits, long long nruns, int* runs, int ncomp,
+                               int min_xy, int min_z, int max_xy, int max_z, int* ext, int* keep, int* ext_out,
+                               int* new_id, int* d_total, int* lab, int sms, cudaStream_t s);
 
 // Host helpers.
 int cascade_widths(double fwhm, int w[3]);
