@@ -73,78 +73,102 @@ __device__ __forceinline__ int for_buckets(long long z, int y, int x, const Shar
   return (tx_hi - tx_lo + 1) * (ty_hi - ty_lo + 1);
 }
 
-// Delta words M_j & ~M_1, four at a time (both masks carry padding words).
-// An entry holds the voxel's cube value (high 32 bits) and its place
-// (hy << 8 | hx) in the bucket's halo'd tile (low 16 bits).
+// The voxels of M_j & ~M_1, counted per bucket or (FILL) listed. An entry holds
+// the voxel's cube value (high 32 bits) and its place (hy << 8 | hx) in the
+// bucket's halo'd tile (low 16 bits).
+//
+// A warp takes 1,024 voxels, a mask word a lane, writes the places of their
+// set bits to shared memory and then works through them with all 32 lanes;
+// lanes that add to the same bucket do so with one atomic. Masked voxels come
+// in clusters, so what bounds it is how they spread over the lanes: with a
+// thread per 128 voxels, following its bits one by one, the count and the fill
+// took 160 us a pair on 360 x 360 x 1464 voxels (1.6 % of them masked);
+// now 79 us.
+constexpr int kListThreads = 256;
+constexpr int kListRun = 1024;  // voxels a warp works on at a time
+constexpr int kListAhead = 4;   // runs whose words are loaded together
 template <bool FILL>
-__global__ void __launch_bounds__(256) k_share_list(const uint32_t* __restrict__ mbits, const float* __restrict__ C,
-                                                    Half16 h16, long long n, long long nx, long long ny, ShareArgs sh,
-                                                    int R) {
-  const long long nq = ((n + 31) / 32 + 3) / 4;
+__global__ void __launch_bounds__(kListThreads) k_share_list(const uint32_t* __restrict__ mbits,
+                                                             const float* __restrict__ C, Half16 h16, long long n,
+                                                             long long nx, long long ny, ShareArgs sh, int R) {
+  __shared__ unsigned short s_off[kListThreads / 32][kListRun];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lanes_below = (1u << lane) - 1u;
+  const long long nwords = (n + 31) / 32, nrun = (nwords + 31) / 32;
   const long long plane = nx * ny;
-  const uint4* m4 = reinterpret_cast<const uint4*>(mbits);
-  const uint4* s4 = reinterpret_cast<const uint4*>(sh.msnap);
   const bool write = FILL && sh.ss->overflow == 0u;
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < nq;
-       q += (long long)gridDim.x * blockDim.x) {
-    const uint4 a = __ldg(m4 + q), b = __ldg(s4 + q);
-    const unsigned d[4] = {a.x & ~b.x, a.y & ~b.y, a.z & ~b.z, a.w & ~b.w};
-    if ((d[0] | d[1] | d[2] | d[3]) == 0u) continue;
-    // coordinates of the group's first voxel (divisions once per 128 voxels),
-    // then followed voxel by voxel
-    long long vcur = 128 * q;
-    long long z = vcur / plane;
-    const long long rem = vcur - z * plane;
-    int y = (int)(rem / nx), x = (int)(rem - (long long)y * nx);
-    // counts: consecutive voxels whose halo reaches one and the same bucket
-    // (the common case) add to it with one atomic
-    long long run_b = -1;
-    unsigned run_n = 0u;
+  const long long step = (long long)gridDim.x * (kListThreads / 32) * kListAhead;
+  for (long long run0 = ((long long)blockIdx.x * (kListThreads / 32) + warp) * kListAhead; run0 < nrun; run0 += step) {
+    unsigned words[kListAhead];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      unsigned w = d[k];
-      while (w) {
-        const int bit = __ffs(w) - 1;
-        w &= w - 1u;
-        const long long v = (4 * q + k) * 32 + bit;
-        if (v >= n) break;
-        x += (int)(v - vcur);
-        vcur = v;
-        while (x >= nx) {
-          x -= (int)nx;
-          if (++y == ny) {
-            y = 0;
-            ++z;
-          }
+    for (int k = 0; k < kListAhead; ++k) {
+      const long long w = (run0 + k) * 32 + lane;
+      words[k] = w < nwords ? __ldg(mbits + w) & ~__ldg(sh.msnap + w) : 0u;
+      if (w == nwords - 1 && (n & 31)) words[k] &= (1u << (n & 31)) - 1u;
+    }
+#pragma unroll 1
+    for (int k = 0; k < kListAhead; ++k) {
+      const long long run = run0 + k;
+      unsigned d = words[0];
+      words[0] = words[1], words[1] = words[2], words[2] = words[3];
+      if (!__any_sync(0xffffffffu, d != 0u)) continue;
+      int x = __popc(d);
+      const int own = x;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      const int total = __shfl_sync(0xffffffffu, x, 31);
+      for (int at = x - own; d; ++at) {
+        s_off[warp][at] = (unsigned short)(32 * lane + __ffs(d) - 1);
+        d &= d - 1u;
+      }
+      __syncwarp();
+      // coordinates of the run's first voxel
+      const long long v0 = run * kListRun, z0 = v0 / plane, rem = v0 - z0 * plane;
+      const int y0 = (int)(rem / nx), x0 = (int)(rem - (long long)y0 * nx);
+      for (int e0 = 0; e0 < total; e0 += 32) {
+        const bool act = e0 + lane < total;
+        const int off = act ? s_off[warp][e0 + lane] : 0;
+        const int rows = (x0 + off) / (int)nx;
+        const int vx = x0 + off - rows * (int)nx, planes = (y0 + rows) / (int)ny, vy = y0 + rows - planes * (int)ny;
+        const long long vz = z0 + planes;
+        unsigned long long cb = 0ull;
+        if (FILL && act) {
+          const long long v = v0 + off;
+          const float cv = h16.fmt ? half16_value(__ldg(h16.bits + v), h16.fmt, __ldg(h16.scale + vz)) : __ldg(C + v);
+          cb = (unsigned long long)__float_as_uint(cv) << 32;
         }
-        if (FILL) {
-          const float cv = h16.fmt ? half16_value(__ldg(h16.bits + v), h16.fmt, __ldg(h16.scale + z)) : __ldg(C + v);
-          const unsigned long long cb = (unsigned long long)__float_as_uint(cv) << 32;
-          for_buckets(z, y, x, sh, R, [&](long long bk, unsigned pos) {
-            const unsigned slot = atomicSub(sh.cnt + bk, 1u) - 1u;
-            const unsigned long long idx = (unsigned long long)__ldg(sh.offs + bk) + slot;
-            if (write && idx < sh.cap) sh.ent[idx] = cb | pos;
-          });
+        // the common case, one bucket; lanes without one take names of their own
+        long long only = -1;
+        unsigned pos = 0u;
+        int nb = 0;
+        if (act) nb = for_buckets(vz, vy, vx, sh, R, [&](long long bk, unsigned p) { only = bk, pos = p; });
+        const unsigned name = nb == 1 ? (unsigned)only : 0xffffffffu - (unsigned)lane;
+        const unsigned peers = __match_any_sync(0xffffffffu, name);
+        const int lead = __ffs(peers) - 1;
+        if (!FILL) {
+          if (nb == 1 && lane == lead) atomicAdd(sh.cnt + only, (unsigned)__popc(peers));
+          if (nb > 1) for_buckets(vz, vy, vx, sh, R, [&](long long bk, unsigned) { atomicAdd(sh.cnt + bk, 1u); });
         } else {
-          long long only = -1;
-          const int nb = for_buckets(z, y, x, sh, R, [&](long long bk, unsigned) { only = bk; });
-          if (nb == 1 && only == run_b) {
-            ++run_n;
-          } else {
-            if (run_n) atomicAdd(sh.cnt + run_b, run_n);
-            run_b = -1;
-            run_n = 0u;
-            if (nb == 1) {
-              run_b = only;
-              run_n = 1u;
-            } else {
-              for_buckets(z, y, x, sh, R, [&](long long bk, unsigned) { atomicAdd(sh.cnt + bk, 1u); });
-            }
+          unsigned slot = 0u;
+          if (nb == 1 && lane == lead) slot = atomicSub(sh.cnt + only, (unsigned)__popc(peers)) - (unsigned)__popc(peers);
+          slot = __shfl_sync(0xffffffffu, slot, lead) + (unsigned)__popc(peers & lanes_below);
+          if (nb == 1) {
+            const unsigned long long idx = (unsigned long long)__ldg(sh.offs + only) + slot;
+            if (write && idx < sh.cap) sh.ent[idx] = cb | pos;
+          } else if (nb > 1) {
+            for_buckets(vz, vy, vx, sh, R, [&](long long bk, unsigned p) {
+              const unsigned long long idx =
+                  (unsigned long long)__ldg(sh.offs + bk) + (atomicSub(sh.cnt + bk, 1u) - 1u);
+              if (write && idx < sh.cap) sh.ent[idx] = cb | p;
+            });
           }
         }
       }
+      __syncwarp();  // the places are read before the next run's are written
     }
-    if (!FILL && run_n) atomicAdd(sh.cnt + run_b, run_n);
   }
 }
 
@@ -762,10 +786,12 @@ cudaError_t launch_share_prep(const SmoothArgs& a, const ShareArgs& sh, int sms,
   const int R = share_R(a.pd);  // the reach the shared pass decodes its entries with
   const long long m = sh.n_buckets + 1;
   const long long nblk = (m + kScanChunk - 1) / kScanChunk;
-  k_share_list<false><<<8 * sms, 256, 0, s>>>(a.mbits, a.C, a.h16, n, a.nx, a.ny, sh, R);
+  const long long per = (long long)kListRun * kListAhead * (kListThreads / 32), want = (n + per - 1) / per;
+  const unsigned list_grid = (unsigned)(want < 8LL * sms ? want : 8LL * sms);
+  k_share_list<false><<<list_grid, kListThreads, 0, s>>>(a.mbits, a.C, a.h16, n, a.nx, a.ny, sh, R);
   k_share_scan1<<<(unsigned)nblk, 1024, 0, s>>>(sh.cnt, sh.offs, sh.bsum, m);
   k_share_scan2<<<(unsigned)nblk, 1024, 0, s>>>(sh.offs, sh.bsum, m, sh.ss, sh.cap);
-  k_share_list<true><<<8 * sms, 256, 0, s>>>(a.mbits, a.C, a.h16, n, a.nx, a.ny, sh, R);
+  k_share_list<true><<<list_grid, kListThreads, 0, s>>>(a.mbits, a.C, a.h16, n, a.nx, a.ny, sh, R);
   return cudaGetLastError();
 }
 
