@@ -365,16 +365,35 @@ bool z16_ok(const SmoothArgs& a) {
          (reinterpret_cast<uintptr_t>(a.S) & 15u) == 0 && a.pd.wz <= 31;
 }
 
+constexpr long long kZSmall = 1LL << 22;
+
 cudaError_t launch_smooth_z(const SmoothArgs& a, int sms, cudaStream_t s, bool* done) {
   *done = false;
   if (a.generic || a.pd.h != 0 || a.pd.wz <= 1) return cudaSuccess;
   if (a.h16.fmt && !z16_ok(a)) return cudaSuccess;
   *done = true;
-  if (a.tune_kind == TUNE_Z4 && a.pd.wz <= 31) return launch_z_vpt<4>(a, sms, s);
+  int kind = a.tune_kind;
+  if (kind == TUNE_AUTO && !a.h16.fmt) {
+    // Without a tuned choice: 512 threads a block (the latency of a thread's
+    // plane-to-plane chain bounds the 256-thread forms), 8 voxels a thread
+    // where the ring fits and the planes allow 16-byte copies, else 4; in a
+    // small cube the most blocks. us for w = 7 with 8 x 256 / 4 x 256 / 4 x
+    // 512 / 8 x 512: 64 x 64 x 128: 40 / 36 / 40 / 48; 217 x 331 x 509 (4-byte
+    // copies): 229 / 201 / 181 / 241; 360 x 360 x 1464: 787 / 846 / 726 / 648;
+    // 1200 x 1200 x 1024: 5754 / 6164 / 5264 / 4594. w = 15 is alike, without
+    // the last form.
+    const long long plane = (long long)a.nx * a.ny;
+    const bool vec = plane % 4 == 0 && (reinterpret_cast<uintptr_t>(a.C) & 15u) == 0 &&
+                     (reinterpret_cast<uintptr_t>(a.S) & 15u) == 0;
+    if (plane * a.nz <= kZSmall) kind = TUNE_Z4;
+    else if (vec && a.pd.wz <= 7) kind = TUNE_Z8W;
+    else if (a.pd.wz <= 15) kind = TUNE_Z4W;
+  }
+  if (kind == TUNE_Z4 && a.pd.wz <= 31) return launch_z_vpt<4>(a, sms, s);
   // 512 threads of 4 voxels: twice the warps per scheduler, a 16-slot ring
-  if (a.tune_kind == TUNE_Z4W && a.pd.wz <= 15) return launch_z_vpt<4, 512>(a, sms, s);
+  if (kind == TUNE_Z4W && a.pd.wz <= 15) return launch_z_vpt<4, 512>(a, sms, s);
   // 512 threads of 8 voxels: as many warps, 8 ring slots
-  if (a.tune_kind == TUNE_Z8W && a.pd.wz <= 7) return launch_z_vpt<8, 512>(a, sms, s);
+  if (kind == TUNE_Z8W && a.pd.wz <= 7) return launch_z_vpt<8, 512>(a, sms, s);
   if (a.pd.wz <= 15) return launch_z_vpt<8>(a, sms, s);
   if (a.pd.wz <= 31) return launch_z_vpt<4>(a, sms, s);
   return launch_z_vpt<1>(a, sms, s);
