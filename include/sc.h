@@ -470,8 +470,9 @@ int sc_noise_scale(sc_ctx *ctx, const float *cube_dev, const int64_t *dims, cons
  *   flags        reserved, pass 0.
  * The library keeps buffers in the context (grown on demand): 5/16 byte per
  * voxel, 8 bytes per run of mask voxels along x, 64 per detection. Synchronises
- * the stream (the numbers of runs and detections size the later parts). Errors: SC_ERR_ARG (NULL pointer, dims, radii, negative
- * limits), SC_ERR_NOMEM, SC_ERR_CUDA. */
+ * the stream (the numbers of runs and detections size the later parts).
+ * Errors: SC_ERR_ARG (NULL pointer, dims, radii, negative limits),
+ * SC_ERR_NOMEM, SC_ERR_CUDA. */
 int sc_link(sc_ctx *ctx, const uint8_t *mask_dev, const int64_t *dims, int r_xy, int r_z, int min_xy, int min_z,
             int max_xy, int max_z, int32_t *labels_dev, int64_t *n_out, int32_t *extents_host, int64_t extents_cap,
             uint32_t flags, void *cuda_stream);
