@@ -263,9 +263,8 @@ int measure(sc_ctx* c, const float* src, long long n, int win, float t, int clip
     CK(launch_plan(c->st, c->hist, win, src, n, c->L, t, gauss ? 0 : clip, std_mode, force, s));
     c->stats.launches += 1;
     if (std_mode) {
-      CK(launch_std(src, n, c->st, c->sms, s));
-      CK(launch_std_final(c->st, pair, s));
-      c->stats.launches += 3;
+      CK(launch_std(src, n, c->st, pair, c->sms, s));
+      c->stats.launches += 2;
     } else {
       CK(launch_pass2(src, n, c->mbits, c->st, c->L, c->sms, s));
       int launched = 0;

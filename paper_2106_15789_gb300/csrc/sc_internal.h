@@ -109,6 +109,9 @@ struct DevState {
   BinCfg win;            // windowed bin layout for smoothed cubes
   double sum, sum2;      // STD mode accumulators
   unsigned long long count;
+  float std_shift, std_scale;  // the values are taken as (x - shift) * scale
+  unsigned int std_blocks;     // blocks through the current pass
+  int std_again;               // the first pass asks for a second one
   // counters filled by the candidate pass
   unsigned long long n_cand_med, n_cand_mad, n_amb, n_below;
   NoisePlan plan;
@@ -325,8 +328,7 @@ cudaError_t launch_select_full(DevState* st, int which, int pair, int sms, cudaS
 // The clip of the voxels that the candidate pass left undecided, or of all by a full pass.
 cudaError_t launch_clip(const float* src, long long n, uint32_t* mbits, DevState* st, Lists L, int sms,
                         cudaStream_t s);
-cudaError_t launch_std(const float* src, long long n, DevState* st, int sms, cudaStream_t s);
-cudaError_t launch_std_final(DevState* st, int pair, cudaStream_t s);
+cudaError_t launch_std(const float* src, long long n, DevState* st, int pair, int sms, cudaStream_t s);
 // Gaussian-fit noise (after the MAD measurement of the same array): the
 // 256-bin histogram over +-5 MAD noises into ghist[256], then the fit, which
 // replaces sigma_cur (and sigma[pair] for pair >= 0) and, with clip, marks the

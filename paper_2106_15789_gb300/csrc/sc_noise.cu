@@ -282,6 +282,8 @@ __device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long
   p.n = n;
   st->n_cand_med = st->n_cand_mad = st->n_amb = st->n_below = 0ull;
   st->sum = st->sum2 = 0.0;
+  st->std_blocks = 0u;
+  st->std_again = 0;
   st->count = 0ull;
   if (clip) p.flags |= PLAN_CLIP;
   if (std_mode) p.flags |= PLAN_STD | PLAN_CLIP_FULL;
@@ -310,6 +312,34 @@ __device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long
   p.bound_med = cum[p.b_med_hi + 1] - cum[p.b_med_lo];
   if (p.bound_med > L.cap.med) p.flags |= PLAN_MED_FULL;
 
+  if (std_mode) {
+    // K and 2^e: the lowest and the highest bin with values bound them all
+    int first = 0, last = kNumBins - 1;
+    for (int hi = last; first < hi;) {
+      const int mid = (first + hi) >> 1;
+      if (cum[mid + 1] > 0ull) hi = mid; else first = mid + 1;
+    }
+    for (int lo = 0; lo < last;) {
+      const int mid = (lo + last + 1) >> 1;
+      if (cum[mid] < n) lo = mid; else last = mid - 1;
+    }
+    double top = fmax(fabs(bin_lo_value(first, cfg)), fabs(bin_hi_value(last, cfg)));
+    if (!isfinite(top)) top = 2.0 * (double)fmaxf(__uint_as_float(st->maxabs_bits), st->repl);  // (0: not measured)
+    // no scale for magnitudes up to 2^40 (and some above 2^-40): n squares stay
+    // below 2^128, and what underflows is too small to count
+    int e = 128;
+    if (top > 0.0 && isfinite(top)) frexp(top, &e);  // top < 2^e
+    e = e > -40 && e <= 40 ? 0 : (e > 128 ? 128 : (e < -126 ? -126 : e));
+    st->std_scale = ldexpf(1.0f, -e);
+    // no shift where 0 lies well within the spread (a quarter of the values
+    // beyond 8 times the median's magnitude, on either side of it)
+    const double lo = bin_lo_value(p.b_med_lo, cfg), hi = bin_hi_value(p.b_med_lo, cfg);
+    const double m = isfinite(lo) ? (isfinite(hi) ? 0.5 * (lo + hi) : lo) : (isfinite(hi) ? hi : 0.0);
+    const float far = __double2float_ru(8.0 * fmax(fabs(lo), fabs(hi)));
+    const bool near0 = isfinite(far) && 4ull * cum[bin_of(-far, cfg)] >= n &&
+                       4ull * (n - cum[bin_of(far, cfg) + 1]) >= n;
+    st->std_shift = near0 ? 0.0f : __double2float_rn(m);
+  }
   if (!std_mode) {
     const PlanCtx P{cum, cfg, bin_lo_value(p.b_med_lo, cfg), bin_hi_value(p.b_med_hi, cfg)};
     if (!(isfinite(P.m_min) && isfinite(P.m_max))) {
@@ -938,49 +968,121 @@ cudaError_t launch_select_full(DevState* st, int which, int pair, int sms, cudaS
 }
 
 // ---------------------------------------------------------------------------
-// STD mode: float64 sums (the float32 data's squares can overflow or
-// underflow float32), two passes: mean, then sum of squared deviations.
-__global__ void __launch_bounds__(256) k_std_pass(const float* __restrict__ x, long long n, DevState* st, int second) {
-  __shared__ double s_a[8];
-  __shared__ unsigned long long s_n[8];
-  if (st->plan.flags & PLAN_EMPTY) return;
-  const double mean = second ? st->sum / (double)st->count : 0.0;
-  double acc = 0.0;
-  unsigned long long cnt = 0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float s = __ldg(x + i);
-    if (!isfinite(s)) continue;
-    if (second) {
-      const double d = (double)s - mean;
-      acc = fma(d, d, acc);
-    } else {
-      acc += (double)s;
-    }
-    ++cnt;
-  }
-  double a = acc;
-  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-  cnt = warp_sum_u64(cnt);
-  const int warp = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { s_a[warp] = a; s_n[warp] = cnt; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double at = 0.0;
-    unsigned long long ct = 0;
-    for (int w = 0; w < 8; ++w) { at += s_a[w]; ct += s_n[w]; }
-    if (second) {
-      atomicAdd(&st->sum2, at);
-    } else {
-      atomicAdd(&st->sum, at);
-      atomicAdd(&st->count, ct);
-    }
-  }
+// STD mode: sums of d = (x - K) 2^-e and of d^2 over the finite values, with K
+// in the median's bin and 2^e above all magnitudes (both from the histogram:
+// the squares of float32 data can overflow or underflow float32). The median
+// lies within one standard deviation of the mean, so K costs the variance
+// S2 - S1^2 / n a bit or two, unless its bin is much wider than the spread
+// (data on a large offset): then a second pass takes the mean as K.
+//
+// Each thread keeps its sums as unevaluated pairs of floats: the difference,
+// the square and the additions are exact in pairs (TwoSum, and an FMA for the
+// product's error), and what is rounded is 2^-24 of the pairs' low parts. The
+// float64 conversions and FMAs of the earlier two passes bound them at 268 us
+// each on 256 x 250 x 600 voxels (the pipe is slow on this part); one pass
+// takes 44 us (a read at the measured HBM rate: 23).
+__device__ __forceinline__ void pair_add(float* s, float* c, float x, float rest) {
+  const float t = __fadd_rn(*s, x);
+  const float b = __fsub_rn(t, *s);
+  const float e = __fadd_rn(__fsub_rn(*s, __fsub_rn(t, b)), __fsub_rn(x, b));
+  *c = __fadd_rn(*c, __fadd_rn(e, rest));
+  *s = t;
 }
 
-__global__ void k_std_final(DevState* st, int pair) {
-  if (st->plan.flags & PLAN_EMPTY) return;
-  const unsigned long long c = st->count;
-  const double sd = c > 1ull ? sqrt(st->sum2 / (double)(c - 1ull)) : 0.0;
+// PLAIN: neither shift nor scale.
+template <bool PLAIN>
+__device__ __forceinline__ void std_add(float x, float scale, float shift, float (&s1)[2], float (&s2)[2], unsigned* n) {
+  if (!(fabsf(x) <= FLT_MAX)) return;  // NaN and Inf
+  float h = x, l = 0.0f;
+  if (!PLAIN) {
+    const float xs = __fmul_rn(x, scale);  // a power of two
+    h = __fsub_rn(xs, shift);
+    const float b = __fsub_rn(h, xs);
+    l = __fsub_rn(__fsub_rn(xs, __fsub_rn(h, b)), __fadd_rn(shift, b));
+  }
+  pair_add(&s1[0], &s1[1], h, l);
+  const float p = __fmul_rn(h, h);
+  float e = __fmaf_rn(h, h, -p);
+  if (!PLAIN) e = __fmaf_rn(__fadd_rn(h, h), l, e);
+  pair_add(&s2[0], &s2[1], p, e);
+  ++*n;
+}
+
+template <bool PLAIN>
+__device__ __forceinline__ void std_sums(const float* __restrict__ x, long long n, float scale, float shift,
+                                         float (&s1)[2], float (&s2)[2], unsigned* cnt) {
+  const long long t0 = (long long)blockIdx.x * 256 + threadIdx.x, stride = (long long)gridDim.x * 256;
+  const long long nq = (reinterpret_cast<uintptr_t>(x) & 15u) == 0 ? n >> 2 : 0;
+  for (long long q = t0; q < nq; q += 4 * stride) {
+    float4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      v[u] = q + u * stride < nq ? __ldg(reinterpret_cast<const float4*>(x) + q + u * stride)
+                                 : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      std_add<PLAIN>(v[u].x, scale, shift, s1, s2, cnt);
+      std_add<PLAIN>(v[u].y, scale, shift, s1, s2, cnt);
+      std_add<PLAIN>(v[u].z, scale, shift, s1, s2, cnt);
+      std_add<PLAIN>(v[u].w, scale, shift, s1, s2, cnt);
+    }
+  }
+  for (long long i = 4 * nq + t0; i < n; i += stride) std_add<PLAIN>(__ldg(x + i), scale, shift, s1, s2, cnt);
+}
+
+// The first pass, or the second, which only runs where the first pass's shift
+// was too far from the mean. The last block of a pass forms the result (or
+// asks for the second pass).
+__global__ void __launch_bounds__(256) k_std_pass(const float* __restrict__ x, long long n, DevState* st, int second,
+                                                  int pair) {
+  __shared__ double s_a[8], s_b[8];
+  __shared__ unsigned s_n[8];
+  if ((st->plan.flags & PLAN_EMPTY) || (second && !st->std_again)) return;
+  const float scale = st->std_scale, shift = __fmul_rn(st->std_shift, scale);
+  float p1[2] = {0.0f, 0.0f}, p2[2] = {0.0f, 0.0f};
+  unsigned cnt = 0u;
+  if (scale == 1.0f && shift == 0.0f) std_sums<true>(x, n, scale, shift, p1, p2, &cnt);
+  else std_sums<false>(x, n, scale, shift, p1, p2, &cnt);
+  double s1 = (double)p1[0] + (double)p1[1], s2 = (double)p2[0] + (double)p2[1];
+  for (int o = 16; o > 0; o >>= 1) {
+    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+  }
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  const int warp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    s_a[warp] = s1;
+    s_b[warp] = s2;
+    s_n[warp] = cnt;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  unsigned long long ct = 0ull;
+  s1 = s2 = 0.0;
+  for (int w = 0; w < 8; ++w) {
+    s1 += s_a[w];
+    s2 += s_b[w];
+    ct += s_n[w];
+  }
+  atomicAdd(&st->sum, s1);
+  atomicAdd(&st->sum2, s2);
+  atomicAdd(&st->count, ct);
+  __threadfence();
+  if (atomicAdd(&st->std_blocks, 1u) != gridDim.x - 1u) return;
+  __threadfence();
+  const double c = (double)*(volatile unsigned long long*)&st->count;
+  s1 = *(volatile double*)&st->sum;
+  s2 = *(volatile double*)&st->sum2;
+  const double var = s2 - s1 * s1 / c;
+  if (!second && c > 1.0 && !(var >= s2 * 0x1p-10)) {
+    st->std_again = 1;
+    st->std_shift = __double2float_rn((double)st->std_shift + s1 / c / (double)scale);  // the mean
+    st->sum = st->sum2 = 0.0;
+    st->count = 0ull;
+    st->std_blocks = 0u;
+    return;
+  }
+  const double sd = c > 1.0 ? sqrt(fmax(var, 0.0) / (c - 1.0)) / (double)scale : 0.0;
   const float sg = (float)sd;
   st->sigma_cur = sg;
   st->sigma_cur_d = sd;
@@ -988,16 +1090,11 @@ __global__ void k_std_final(DevState* st, int pair) {
   if (!(sg > 0.0f)) st->warn |= SC_WARN_ZERO_SIGMA;
 }
 
-cudaError_t launch_std(const float* src, long long n, DevState* st, int sms, cudaStream_t s) {
-  long long want = (n + 255) / 256;
-  int grid = (int)(want < 1 ? 1 : (want > 4LL * sms ? 4LL * sms : want));
-  k_std_pass<<<grid, 256, 0, s>>>(src, n, st, 0);
-  k_std_pass<<<grid, 256, 0, s>>>(src, n, st, 1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_std_final(DevState* st, int pair, cudaStream_t s) {
-  k_std_final<<<1, 1, 0, s>>>(st, pair);
+cudaError_t launch_std(const float* src, long long n, DevState* st, int pair, int sms, cudaStream_t s) {
+  const long long want = (n + 4095) / 4096;  // four 16-byte loads a thread
+  const int grid = (int)(want > 6LL * sms ? 6LL * sms : want);
+  k_std_pass<<<grid, 256, 0, s>>>(src, n, st, 0, pair);
+  k_std_pass<<<grid, 256, 0, s>>>(src, n, st, 1, pair);
   return cudaGetLastError();
 }
 

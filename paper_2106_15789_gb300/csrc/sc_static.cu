@@ -99,8 +99,7 @@ extern "C" int sc_noise_static(const float* data_dev, int64_t n, int noise_mode,
   CKS(launch_hist(data_dev, n, st, hist, 0, 0, sms, s));
   CKS(launch_plan(st, hist, 0, data_dev, n, L, 1.0f, 0, std_mode, 0u, s));
   if (std_mode) {
-    CKS(launch_std(data_dev, n, st, sms, s));
-    CKS(launch_std_final(st, SC_MAX_KERNELS, s));
+    CKS(launch_std(data_dev, n, st, SC_MAX_KERNELS, sms, s));
   } else {
     CKS(launch_pass2(data_dev, n, nullptr, st, L, sms, s));
     int launched = 0;

@@ -79,3 +79,24 @@ def test_run_with_full_selection_passes(shape):
         b = ctx.run(cube, kernels, 3.5, flags=sc.SC_FLAG_NO_FAST_SELECT)
     assert a[1] == b[1] and a[2] == b[2]
     assert torch.equal(a[0], b[0])
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 255, 4097, 300001])
+@pytest.mark.parametrize("kind", ["normal", "offset", "far", "outlier", "wide"])
+def test_std(kind, n):
+    """STD mode's sums in pairs of floats: shifts far from the mean, magnitudes
+    at both ends of float32, unaligned data."""
+    x = _data({"far": "normal", "outlier": "normal"}.get(kind, kind), n)
+    if kind == "far":  # the spread below the width of the median's bin
+        x = (np.float32(1.0e6) + x * np.float32(0.5)).astype(np.float32)
+    elif kind == "outlier":
+        x[n // 2] = 3.0e37
+    if not np.isfinite(x).any():
+        x[0] = 1.0
+    d = torch.from_numpy(np.concatenate([x[:1], x])).cuda()[1:]  # rows start 4 bytes off a 16-byte boundary
+    v = x[np.isfinite(x)].astype(np.float64)
+    want = float(np.sqrt(((v - v.mean()) ** 2).sum() / (v.size - 1))) if v.size > 1 else 0.0
+    with Context(0, n + 1) as ctx:
+        got = ctx.noise(d, "std")
+    # one float32 rounding of the result; the sums are good to 2^-40
+    assert abs(got - want) <= 2.0**-24 * 1.01 * abs(want), (got, want)
