@@ -280,7 +280,13 @@ static_assert(TUNE_WS == SC_VARIANT_WS && TUNE_TILE == SC_VARIANT_TILE && TUNE_G
 // kernel take round-robin (at most max_ch chunks). An autotuner factor asks
 // for about that many items per SM; without one, the chunking whose busiest
 // block streams the fewest planes: ceil(items / blocks) items of lz planes
-// plus the 2r halo planes of the spectral boxcar each.
+// plus the 2r halo planes of the spectral boxcar (and, for short items, what
+// filling the pipeline costs) each. Chunks may be as short as kMinChunk planes:
+// in a small cube (2 tiles of 64 x 32) longer ones leave most SMs idle (a first
+// pair of 64 x 64 x 128 voxels took 73 us in 8 items of 32 planes, and takes 16
+// in 64 of 4).
+constexpr int kMinChunk = 4;
+inline long long item_planes(long long lz, long long r) { return lz + 2 * r + (lz < 16 ? 3 : 0); }
 inline long long z_chunks(const SmoothArgs& a, long long tiles, int sms, long long max_ch) {
   max_ch = max_ch < 1 ? 1 : max_ch;
   if (a.tune_zfactor > 0) {
@@ -292,7 +298,7 @@ inline long long z_chunks(const SmoothArgs& a, long long tiles, int sms, long lo
   for (long long zch = 1; zch <= max_ch && zch <= 64; ++zch) {
     const long long lz = (nz + zch - 1) / zch, chunks = (nz + lz - 1) / lz;
     const long long items = tiles * chunks, blocks = items < sms ? items : sms;
-    const long long cost = (items + blocks - 1) / blocks * (lz + 2 * r);
+    const long long cost = (items + blocks - 1) / blocks * item_planes(lz, r);
     if (best_cost < 0 || cost < best_cost) {
       best = zch;
       best_cost = cost;

@@ -1223,13 +1223,14 @@ cudaError_t launch_fx_setup(DevState* st, float repl_value, const PairWeights& W
 // Window of the fine histogram of the raw cube: the bin of the median of |x|
 // gives the scale, and the window spans 2^-20 .. 2^12 of it (as for the
 // smoothed cubes), so the plan of the sigma_0 measurement resolves 128 bins
-// per octave instead of 16. The median |x| comes from kWinSample values at
-// a fixed step through the cube (all of them in a smaller cube): a window 32
+// per octave instead of 16. The median |x| comes from kWinSample values
+// spread through the cube (all of them in a smaller cube): a window 32
 // octaves wide needs its scale only roughly, and the exact selection that
 // follows does not depend on it (a poorly placed window costs candidates,
-// never exactness).
+// never exactness). One block, bound by the latency of its loads: 65,536
+// values in four batches took 44 to 68 us a run, 8,192 in one take 10.
 constexpr int kWinThreads = 1024;
-constexpr long long kWinSample = 65536;
+constexpr long long kWinSample = 8192;
 constexpr int kWinPerThread = (int)(kWinSample / kWinThreads);
 __global__ void __launch_bounds__(kWinThreads) k_window_from_sample(const float* __restrict__ x, Half16 h,
                                                                     long long plane, long long n, DevState* st) {
@@ -1240,15 +1241,17 @@ __global__ void __launch_bounds__(kWinThreads) k_window_from_sample(const float*
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   for (int i = t; i < kNumBins; i += kWinThreads) wh[i] = 0u;
   __syncthreads();
-  // m values step apart (every value of a cube of at most kWinSample)
+  // m values, one from every step of the cube (all of a cube of at most
+  // kWinSample), at places that follow no row or column
   const long long m = n < kWinSample ? n : kWinSample, step = n / (m > 0 ? m : 1);
-  constexpr int kBatch = 16;  // loads in flight per thread
+  constexpr int kBatch = kWinPerThread;  // all loads in flight
   for (int j0 = 0; j0 < kWinPerThread; j0 += kBatch) {
     float v[kBatch];
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
       const long long k = (long long)(j0 + j) * kWinThreads + t;
-      const long long i = k * step;
+      const unsigned long long h32 = (unsigned)k * 2654435761u;
+      const long long i = k * step + (long long)(h32 * (unsigned long long)step >> 32);
       v[j] = __int_as_float(0x7fc00000);
       if (k < m) v[j] = h.fmt ? half16_value(__ldg(h.bits + i), h.fmt, __ldg(h.scale + i / plane)) : __ldg(x + i);
     }

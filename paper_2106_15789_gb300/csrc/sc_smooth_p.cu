@@ -727,11 +727,12 @@ cudaError_t launch_p(const SmoothArgs& a0, const ShareArgs& sh, int sms, cudaStr
   const int r = (a.pd.wz - 1) / 2;
   long long best = -1;
   double best_cost = 0.0;
-  const long long max_ch = std::max(1LL, (long long)a.nz / 16);
+  const long long max_ch = std::max(1LL, (long long)a.nz / kMinChunk);
   for (long long zch = 1; zch <= std::min(max_ch, 64LL); ++zch) {
     const long long lz = (a.nz + zch - 1) / zch;
     const long long chunks = (a.nz + lz - 1) / lz;
-    const double cost = (double)(a.nz + chunks * 2 * r) * tiles / sms + (double)(lz + 2 * r);
+    const long long extra = item_planes(lz, r) - lz;
+    const double cost = (double)(a.nz + chunks * extra) * tiles / sms + (double)(lz + extra);
     if (best < 0 || cost < best_cost) {
       best = lz;
       best_cost = cost;
