@@ -19,18 +19,21 @@
 //
 // A selection takes one pass over the window: a sample of it (every 8th voxel
 // of a row, kept in shared memory) brackets the wanted rank, the pass counts
-// the values under the bracket and copies those inside it, and the rank is
+// the values under the bracket and every lane copies those of its own inside
+// it (4 % of them, to its own column of shared memory: no votes; where few
+// columns of the window are finite, also to a common pool), and the rank is
 // found among the copies by one histogram of 2048 equal steps of the bracket
 // and a direct ranking inside one step. A bracket that misses its rank, or
 // holds more values than the copies' room, costs radix passes over the window
 // instead, so the result is exact whatever the data.
 //
-// What bounds it: instruction issue of the two passes; the 7 windows that share a voxel read it from L2. Blocks of
-// 256 threads, four to an SM, hide each other's barriers and loads. On 360 x
-// 360 x 1464 voxels (48,668 windows of 31^3) the earlier form, one block of
-// 1,024 threads per SM with the window in shared memory, warp-aggregated
-// (match_any) histograms and up to 40 barriers a window on nothing else, took
-// 16.9 ms; this one 6.4 ms.
+// What bounds it: instruction issue of the two passes (2.8 of 4 slots a cycle
+// while a block is resident); the 7 windows that share a voxel read it from
+// L2. Blocks of 256 threads, four to an SM, hide each other's barriers and
+// loads. On 360 x 360 x 1464 voxels (48,668 windows of 31^3) the earlier form,
+// one block of 1,024 threads per SM with the window in shared memory,
+// warp-aggregated (match_any) histograms and up to 40 barriers a window, took
+// 16.9 ms; this one 5.2 ms.
 #include <cfloat>
 #include <cstdint>
 
@@ -46,9 +49,9 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kBlocksPerSm = 4;
 constexpr int kBins = 2048;              // steps of a bracket; radix digits of 11, 11 and 10 bits
 constexpr unsigned kNone = 0xffffffffu;  // above the key of every finite value
-constexpr int kSegCap = 640;             // copies each warp keeps of the values in a bracket
-constexpr int kCandCap = kSegCap * kWarps;
-constexpr int kSampleCap = 4096;
+constexpr int kLaneCap = 20;             // copies each thread keeps of its values in a bracket
+constexpr int kPool = 512;               // and those beyond, for the block
+constexpr int kSampleSlots = 16;         // sampled voxels per thread
 constexpr int kUnroll = 8;               // loads in flight per thread
 constexpr int kFewCap = 256;             // copies ranked directly
 
@@ -70,15 +73,17 @@ __device__ __forceinline__ void window_range(int c, int g, int w, long long n, l
 }
 
 struct Scratch {
-  float cand[kCandCap];       // per warp kSegCap copies
-  float sample[kSampleCap];   // NaN: no finite voxel
-  alignas(16) unsigned hist[kBins];
-  float few[kFewCap];
+  float cand[kLaneCap * kThreads];        // a column per thread
+  float pool[kPool];
+  float sample[kSampleSlots * kThreads];  // a column per thread; NaN: no finite voxel
+  union {
+    alignas(16) unsigned hist[kBins];
+    float few[kFewCap];
+  };
   unsigned part[kWarps];
-  unsigned seg[kWarps];       // copies each warp wanted to make (may exceed kSegCap)
-  unsigned digit[2], rank[2], n_few, next, finite, below, n_sample;
+  unsigned digit[2], rank[2], n_few, next, finite, below, n_copies, n_pool, n_sample;
   float v1;
-  double dpart[kWarps + 1];
+  double dpart[kWarps];
 };
 
 // A window: voxel (x, y, z) at base + z plane + y nx + x. A row goes to a
@@ -97,15 +102,19 @@ struct Win {
   __device__ __forceinline__ int step() const { return 1 << (wy + 5 - lw); }  // rows of a turn
   __device__ __forceinline__ int turns() const { return (ly + step() - 1) / step(); }
   __device__ __forceinline__ int sets() const { return kWarps >> wy; }
-  // Most voxels one warp takes.
-  __device__ __forceinline__ int share() const { return turns() * (32 >> lw) * ((lz + sets() - 1) / sets()) * lx; }
+  // Most voxels one thread takes.
+  __device__ __forceinline__ int share() const {
+    return turns() * ((lz + sets() - 1) / sets()) * ((lx + (1 << lw) - 1) >> lw);
+  }
 };
 
 // f(v) for every voxel v of the window, NaN in the lanes left over; all lanes
 // of a warp call f together, kUnroll loads ahead. The turn and the plane are
 // the same for all lanes, so a lane adds its own fixed offset to an address
-// that a warp shares.
-template <class F>
+// that a warp shares. FAST: planes of three or four turns (17 to 32 rows of
+// more than 16 voxels) get code of their own, two planes at a time with a
+// quarter of the address arithmetic; for the passes over every voxel.
+template <bool FAST, class F>
 __device__ __forceinline__ void for_window(const Win& w, F f) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int group = 1 << w.lw, step = w.step(), turns = w.turns(), sets = w.sets();
@@ -116,6 +125,23 @@ __device__ __forceinline__ void for_window(const Win& w, F f) {
     const int dx = x0 + (lane & (group - 1));
     const int rows = dx < w.lx ? w.ly - y0 : 0;  // rows left from the lane's first one on
     const float* const mine = w.base + z0 * w.plane + y0 * w.nx + dx;
+    if (FAST && turns > 2 && turns <= 4) {
+      const float* q = mine;
+      const long long jump = sets * w.plane;
+      const int planes = total / turns;
+      const bool ok[4] = {0 < rows, step < rows, 2 * step < rows, 3 * step < rows};
+      for (int z = 0; z < planes; z += 2, q += 2 * jump) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          v[u] = __int_as_float(0x7fc00000);
+          if (ok[u & 3] && (u < 4 || z + 1 < planes)) v[u] = __ldg(q + (u >> 2) * jump + (u & 3) * turn);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f(v[u]);
+      }
+      continue;
+    }
     long long at = 0;
     int k = 0;
     for (int t0 = 0; t0 < total; t0 += kUnroll) {
@@ -220,7 +246,7 @@ __device__ __noinline__ void select_window(const Win& w, Of of, unsigned r, bool
     __syncthreads();
     clear_hist(S);
     __syncthreads();
-    for_window(w, [&](float v) {
+    for_window<false>(w, [&](float v) {
       const unsigned k = isfinite(v) ? fkey(of(v)) : kNone;
       const bool in = k != kNone && (k & pmask) == prefix;
       const unsigned d = in ? (k >> shift) & dmask : kNone;
@@ -242,7 +268,7 @@ __device__ __noinline__ void select_window(const Win& w, Of of, unsigned r, bool
         if (tid == 0) S->next = kNone;
         __syncthreads();
         unsigned mn = kNone;
-        for_window(w, [&](float v) {
+        for_window<false>(w, [&](float v) {
           const unsigned k = isfinite(v) ? fkey(of(v)) : 0u;
           if (k > prefix) mn = min(mn, k);
         });
@@ -260,11 +286,15 @@ __device__ __noinline__ void select_window(const Win& w, Of of, unsigned r, bool
 // more than r of them); for a next one outside them, nxt(): its value. False
 // (uniformly) when too many copies share the step of the rank.
 template <class Next>
-__device__ bool select_cand(float lo, float hi, unsigned r, bool want_next, Scratch* S, float* v1, float* v2,
+__device__ bool select_cand(int n, float lo, float hi, unsigned r, bool want_next, Scratch* S, float* v1, float* v2,
                             Next nxt) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float* const seg = S->cand + warp * kSegCap;
-  const int n = (int)S->seg[warp];
+  const int tid = threadIdx.x, lane = tid & 31;
+  // f(v) for this thread's n copies, kThreads apart, and its part of the pool
+  const int np = (int)S->n_pool;
+  const auto copies = [&](auto f) {
+    for (int i = 0; i < n; ++i) f(S->cand[i * kThreads + tid]);
+    for (int i = tid; i < np; i += kThreads) f(S->pool[i]);
+  };
   // the step of a copy: a monotone function of its value
   const float inv = (float)kBins / (hi - lo);
   const auto digit = [&](float v) { return min(kBins - 1, (int)((v - lo) * inv)); };
@@ -274,23 +304,24 @@ __device__ bool select_cand(float lo, float hi, unsigned r, bool want_next, Scra
     S->next = kNone;
   }
   __syncthreads();
-  for (int i = lane; i < n; i += 32) atomicAdd(&S->hist[digit(seg[i])], 1u);
+  copies([&](float v) { atomicAdd(&S->hist[digit(v)], 1u); });
   find_digits(S, r, r);
   const int d = (int)S->digit[0];
   const unsigned rr = S->rank[0], cnt = S->hist[d];
   if (cnt > (unsigned)kFewCap) {
     // ties? one value in the whole step is the answer
+    __syncthreads();  // (the digit and the counts are read)
     if (tid == 0) {
       S->digit[0] = kNone;
       S->digit[1] = 0u;
     }
     __syncthreads();
     unsigned kmin = kNone, kmax = 0u;
-    for (int i = lane; i < n; i += 32) {
-      if (digit(seg[i]) != d) continue;
-      kmin = min(kmin, fkey(seg[i]));
-      kmax = max(kmax, fkey(seg[i]));
-    }
+    copies([&](float v) {
+      if (digit(v) != d) return;
+      kmin = min(kmin, fkey(v));
+      kmax = max(kmax, fkey(v));
+    });
     kmin = __reduce_min_sync(0xffffffffu, kmin);
     kmax = __reduce_max_sync(0xffffffffu, kmax);
     if (lane == 0) {
@@ -303,13 +334,13 @@ __device__ bool select_cand(float lo, float hi, unsigned r, bool want_next, Scra
     __syncthreads();
     return same && (!want_next || rr + 1u < cnt);
   }
+  __syncthreads();  // the counts are read: their memory becomes the step's values
   unsigned above = kNone;
-  for (int i = lane; i < n; i += 32) {
-    const float v = seg[i];
+  copies([&](float v) {
     const int dv = digit(v);
     if (dv == d) S->few[atomicAdd(&S->n_few, 1u)] = v;
     else if (dv > d) above = min(above, fkey(v));
-  }
+  });
   if (want_next) {
     above = __reduce_min_sync(0xffffffffu, above);
     if (lane == 0) atomicMin(&S->next, above);
@@ -331,27 +362,130 @@ __device__ bool select_cand(float lo, float hi, unsigned r, bool want_next, Scra
   return true;
 }
 
-// Counts (into *below) the values of(v) under lo and copies those in [lo, hi].
+// Counts the values under lo and copies those in [lo, hi] to the thread's
+// column (n of them) and, once that is full, to the pool.
 struct Collect {
   float lo, hi;
-  float* seg;
-  unsigned n, below, lanes_below;
+  Scratch* S;
+  int n;
+  unsigned below;
   __device__ __forceinline__ void operator()(float a) {  // (NaN: neither)
     const bool under = a < lo;
     below += under ? 1u : 0u;
-    const bool in = a <= hi && !under;
-    const unsigned b = __ballot_sync(0xffffffffu, in);
-    const unsigned pos = n + (unsigned)__popc(b & lanes_below);
-    if (in && pos < (unsigned)kSegCap) seg[pos] = a;
-    n += (unsigned)__popc(b);
+    if (a <= hi && !under) {
+      if (n < kLaneCap) {
+        S->cand[n * kThreads + threadIdx.x] = a;
+        ++n;
+      } else {
+        const unsigned i = atomicAdd(&S->n_pool, 1u);
+        if (i < (unsigned)kPool) S->pool[i] = a;
+      }
+    }
+  }
+  // Adds a pass's counts up (S->below, n_copies, n_pool cleared before it).
+  __device__ __forceinline__ void finish() const {
+    const unsigned b = __reduce_add_sync(0xffffffffu, below), c = __reduce_add_sync(0xffffffffu, (unsigned)n);
+    if ((threadIdx.x & 31) == 0) {
+      atomicAdd(&S->below, b);
+      atomicAdd(&S->n_copies, c);
+    }
   }
 };
 
-// Key bounds around sample ranks p +- 4 binomial standard deviations, widened
-// to whole digits; the sample's histogram is in S->hist.
-__device__ __forceinline__ void bracket_digits(Scratch* S, unsigned ns, unsigned p) {
-  const unsigned delta = 2u * (unsigned)sqrtf((float)ns) + 4u;
-  find_digits(S, p > delta ? p - delta : 0u, min(p + delta, ns - 1u));
+// Bracket [lo, hi] of sample rank p of of(x) over the ns finite sampled voxels
+// (`slots` per thread): 2.5 binomial standard deviations either side (a sample
+// at fixed places scatters less; wider ones overflow the columns where few
+// voxels are finite), located by the keys' bits from kShift on and
+// then by 2048 equal steps between. Any bracket is checked by the pass's counts.
+template <int kShift, class Of, class Key>
+__device__ void sample_bracket(Scratch* S, int slots, Of of, Key key, unsigned ns, unsigned p, float* lo, float* hi) {
+  const float* const mine = S->sample + threadIdx.x;
+  clear_hist(S);
+  __syncthreads();
+  for (int i = 0; i < slots; ++i) {
+    const float v = of(mine[i * kThreads]);
+    if (v == v) atomicAdd(&S->hist[min(key(v) >> kShift, (unsigned)kBins - 1u)], 1u);
+  }
+  const unsigned delta = (unsigned)(1.25f * sqrtf((float)ns)) + 4u;
+  const unsigned ra = p > delta ? p - delta : 0u, rb = min(p + delta, ns - 1u);
+  find_digits(S, ra, rb);
+  const float a = fminf(fmaxf(key.value(S->digit[0] << kShift), -FLT_MAX), FLT_MAX);
+  const float b = fminf(fmaxf(key.value((S->digit[1] << kShift) | ((1u << kShift) - 1u)), -FLT_MAX), FLT_MAX);
+  const unsigned ia = S->rank[0];
+  *lo = a;
+  *hi = b;
+  const float inv = (float)kBins / (b - a);
+  __syncthreads();
+  if (!(inv > 0.0f && inv <= FLT_MAX)) return;
+  clear_hist(S);
+  __syncthreads();
+  for (int i = 0; i < slots; ++i) {
+    const float v = of(mine[i * kThreads]);
+    if (v >= a && v <= b) atomicAdd(&S->hist[min(kBins - 1, (int)((v - a) * inv))], 1u);
+  }
+  // the ranks among the values from the first digit on
+  find_digits(S, ia, ia + (rb - ra));
+  const float step = (b - a) / (float)kBins;
+  *lo = fmaxf(a, a + (float)S->digit[0] * step);
+  *hi = fminf(b, a + (float)(S->digit[1] + 1u) * step);
+  __syncthreads();
+}
+struct KeyOfValue {
+  __device__ __forceinline__ unsigned operator()(float v) const { return fkey(v); }
+  __device__ __forceinline__ float value(unsigned k) const { return fkey_inv(k); }
+};
+struct KeyOfDev {
+  __device__ __forceinline__ unsigned operator()(float v) const { return __float_as_uint(v); }
+  __device__ __forceinline__ float value(unsigned k) const { return __uint_as_float(k); }
+};
+
+// Samples every 8th voxel (of rows over 4,096 voxels fewer) of every rstep-th
+// row, the offset moving with the row, into the threads' columns; returns the
+// slots used, and adds the finite ones to S->n_sample.
+__device__ __forceinline__ int take_sample(const Win& w, Scratch* S) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int lstep = 3;
+  while ((w.lx >> lstep) >= 32 * kSampleSlots) ++lstep;
+  const int rows = w.ly * w.lz, sx = (w.lx + (1 << lstep) - 1) >> lstep;
+  const int ls = sx > 16 ? 5 : (sx > 8 ? 4 : (sx > 4 ? 3 : (sx > 2 ? 2 : 1)));  // 2^ls lanes share a row
+  const int turns = (sx + (1 << ls) - 1) >> ls, at_once = kWarps << (5 - ls);   // rows of a slot
+  int rstep = 1;
+  while (turns * (((rows + rstep - 1) / rstep + at_once - 1) / at_once) > kSampleSlots) ++rstep;
+  const int groups = ((rows + rstep - 1) / rstep + at_once - 1) / at_once;
+  const int q0 = (warp << (5 - ls)) + (lane >> ls);  // the thread's first sampled row
+  const int inc = at_once * rstep, dz = inc / w.ly, dy = inc - dz * w.ly;
+  unsigned c = 0u;
+  int slot = 0;
+  for (int t = 0; t < turns; ++t) {
+    int q = q0, z = q0 * rstep / w.ly, y = q0 * rstep - z * w.ly;
+    const int j = (t << ls) + (lane & ((1 << ls) - 1));
+    for (int g0 = 0; g0 < groups; g0 += 4) {
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int dx = (j << lstep) + ((3 * q) & 7);
+        v[u] = __int_as_float(0x7fc00000);
+        if (z < w.lz && dx < w.lx) v[u] = __ldg(w.base + z * w.plane + y * w.nx + dx);
+        q += at_once;
+        y += dy;
+        z += dz;
+        if (y >= w.ly) {
+          y -= w.ly;
+          ++z;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (g0 + u >= groups) break;
+        const bool ok = isfinite(v[u]);
+        S->sample[(slot++) * kThreads + tid] = ok ? v[u] : __int_as_float(0x7fc00000);
+        c += ok ? 1u : 0u;
+      }
+    }
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0 && c) atomicAdd(&S->n_sample, c);
+  return slot;
 }
 
 // *s + *c += x with Neumaier's compensation (the running error of the float
@@ -376,109 +510,59 @@ __device__ __forceinline__ double block_sum_d(double v, double* part) {
   return t;
 }
 
-// Exact median and MAD of the nf finite voxels of the window.
+// Exact median and MAD noise of the window's finite voxels (NaN if none).
 __device__ double window_mad(const Win& w, Scratch* S) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int rows = w.ly * w.lz;
+  const int tid = threadIdx.x, lane = tid & 31;
   Collect col;
-  col.seg = S->cand + warp * kSegCap;
-  col.lanes_below = (1u << lane) - 1u;
-  // a window whose warps' shares fit their segments is copied whole
-  const bool whole = w.share() <= kSegCap;
+  col.S = S;
+  // a window whose threads' shares fit their columns is copied whole
+  const bool whole = w.share() <= kLaneCap;
   float lo = -FLT_MAX, hi = FLT_MAX;
-  bool bracket = true;
   unsigned ns = 0u;
-  if (tid == 0) S->finite = S->below = S->n_sample = 0u;
+  int slots = 0;
+  if (tid == 0) S->finite = S->below = S->n_copies = S->n_pool = S->n_sample = 0u;
+  __syncthreads();
   if (!whole) {
-    // every 8th voxel of every row (the offset moves with the row), of every
-    // second row where that would overflow the sample's room
-    const int sx = (w.lx + 7) >> 3;
-    int rstep = 1;
-    while ((rows + rstep - 1) / rstep * sx > kSampleCap) ++rstep;
-    const int want = (rows + rstep - 1) / rstep * sx;
-    clear_hist(S);
-    __syncthreads();
-    unsigned c = 0u;
-    for (int i0 = 0; i0 < want; i0 += 4 * kThreads) {
-      float v[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = i0 + u * kThreads + tid;
-        v[u] = __int_as_float(0x7fc00000);
-        if (i < want) {
-          const int q = i / sx, r = q * rstep, z = r / w.ly, y = r - z * w.ly;
-          const int dx = 8 * (i - q * sx) + ((3 * q) & 7);
-          if (dx < w.lx) v[u] = __ldg(w.base + z * w.plane + y * w.nx + dx);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = i0 + u * kThreads + tid;
-        if (i >= want) break;
-        const bool ok = isfinite(v[u]);
-        S->sample[i] = ok ? v[u] : __int_as_float(0x7fc00000);
-        if (ok) {
-          ++c;
-          atomicAdd(&S->hist[fkey(v[u]) >> 21], 1u);
-        }
-      }
-    }
-    c = __reduce_add_sync(0xffffffffu, c);
-    if (lane == 0 && c) atomicAdd(&S->n_sample, c);
+    slots = take_sample(w, S);
     __syncthreads();
     ns = S->n_sample;
-    bracket = ns >= 64u;
-    if (bracket) {
-      bracket_digits(S, ns, (ns - 1u) / 2u);
-      lo = fkey_inv(S->digit[0] << 21);
-      hi = fkey_inv((S->digit[1] << 21) | 0x1fffffu);
-    }
+    if (ns >= 64u) sample_bracket<21>(S, slots, Value{}, KeyOfValue{}, ns, (ns - 1u) / 2u, &lo, &hi);
   }
-  __syncthreads();
+  const bool bracket = whole || ns >= 64u;
   unsigned finite = 0u;
   col.lo = lo;
   col.hi = hi;
-  col.n = col.below = 0u;
-  for_window(w, [&](float v) {
-    v = __fadd_rn(v, __fsub_rn(v, v));  // Inf becomes NaN
-    finite += v == v ? 1u : 0u;
-    col(v);
+  col.n = 0;
+  col.below = 0u;
+  for_window<true>(w, [&](float v) {
+    const bool ok = fabsf(v) <= FLT_MAX;  // false for NaN and Inf
+    finite += ok ? 1u : 0u;
+    col(ok ? v : __int_as_float(0x7fc00000));
   });
   finite = __reduce_add_sync(0xffffffffu, finite);
-  unsigned below = __reduce_add_sync(0xffffffffu, col.below);
-  if (lane == 0) {
-    S->seg[warp] = col.n;
-    atomicAdd(&S->finite, finite);
-    atomicAdd(&S->below, below);
-  }
+  if (lane == 0) atomicAdd(&S->finite, finite);
+  col.finish();
   __syncthreads();
   const unsigned nf = S->finite;
   if (nf == 0u) return __longlong_as_double(0x7ff8000000000000LL);  // no finite voxel
   const unsigned r1 = (nf - 1u) / 2u;
   const bool even = (nf & 1u) == 0u;
   // the copies are complete and hold the rank
-  const auto holds = [&](unsigned under) {
-    unsigned n = 0u;
-    bool fits = true;
-    for (int k = 0; k < kWarps; ++k) {
-      n += S->seg[k];
-      fits = fits && S->seg[k] <= (unsigned)kSegCap;
-    }
-    return fits && r1 >= under && r1 < under + n;
+  const auto holds = [&] {
+    return S->n_pool <= (unsigned)kPool && r1 >= S->below && r1 - S->below < S->n_copies + S->n_pool;
   };
-  float ma = 0.0f, mb = 0.0f;
-  below = S->below;
-  bool done = bracket && holds(below);
-  if (whole) {
-    // the bracket of the copies: their smallest and largest value
+  unsigned below = S->below;
+  bool done = bracket && holds();
+  // the smallest and largest of the copies' values, as their bracket
+  const auto ends = [&](bool both) {
     if (tid == 0) {
       S->digit[0] = kNone;
       S->digit[1] = 0u;
     }
     __syncthreads();
     unsigned kmin = kNone, kmax = 0u;
-    for (int i = lane; i < (int)S->seg[warp]; i += 32) {
-      const unsigned k = fkey(col.seg[i]);
+    for (int i = 0; i < col.n; ++i) {
+      const unsigned k = fkey(S->cand[i * kThreads + tid]);
       kmin = min(kmin, k);
       kmax = max(kmax, k);
     }
@@ -489,14 +573,15 @@ __device__ double window_mad(const Win& w, Scratch* S) {
       atomicMax(&S->digit[1], kmax);
     }
     __syncthreads();
-    lo = fkey_inv(S->digit[0]);
+    lo = both ? fkey_inv(S->digit[0]) : 0.0f;
     hi = fkey_inv(S->digit[1]);
     __syncthreads();
-  }
+  };
+  if (whole) ends(true);
   // the smallest value of(x) above hi in the window
   const auto above = [&](auto of, float top) {
     unsigned mn = kNone;
-    for_window(w, [&](float v) {
+    for_window<false>(w, [&](float v) {
       const float a = isfinite(v) ? of(v) : __int_as_float(0x7fc00000);
       if (a > top) mn = min(mn, fkey(a));
     });
@@ -506,7 +591,9 @@ __device__ double window_mad(const Win& w, Scratch* S) {
     __syncthreads();
     return fkey_inv(S->next);
   };
-  if (done) done = select_cand(lo, hi, r1 - below, even, S, &ma, &mb, [&] { return above(Value{}, hi); });
+  float ma = 0.0f, mb = 0.0f;
+  if (done)
+    done = select_cand(col.n, lo, hi, r1 - below, even, S, &ma, &mb, [&] { return above(Value{}, hi); });
   if (!done) select_window(w, Value{}, r1, even, S, &ma, &mb);
   if (!even) mb = ma;
   __syncthreads();
@@ -514,52 +601,25 @@ __device__ double window_mad(const Win& w, Scratch* S) {
   const AbsDev dev{ma, mb, even};
   float d1 = 0.0f, d2 = 0.0f;
   if (whole) {  // the copies are all finite voxels
-    if (tid == 0) S->digit[1] = 0u;
-    __syncthreads();
-    unsigned kmax = 0u;
-    for (int i = lane; i < (int)S->seg[warp]; i += 32) {
-      const float a = dev(col.seg[i]);
-      col.seg[i] = a;
-      kmax = max(kmax, __float_as_uint(a));
-    }
-    kmax = __reduce_max_sync(0xffffffffu, kmax);
-    if (lane == 0) atomicMax(&S->digit[1], kmax);
-    __syncthreads();
-    hi = __uint_as_float(S->digit[1]);
-    __syncthreads();
-    done = select_cand(0.0f, hi, r1, even, S, &d1, &d2, [&] { return d1; });
+    for (int i = 0; i < col.n; ++i) S->cand[i * kThreads + tid] = dev(S->cand[i * kThreads + tid]);
+    ends(false);
+    done = select_cand(col.n, 0.0f, hi, r1, even, S, &d1, &d2, [&] { return d1; });
   } else {
     done = ns >= 64u;
     if (done) {
-      clear_hist(S);
-      if (tid == 0) S->below = 0u;
-      __syncthreads();
-      const int sx = (w.lx + 7) >> 3;
-      int rstep = 1;
-      while ((rows + rstep - 1) / rstep * sx > kSampleCap) ++rstep;
-      const int want = (rows + rstep - 1) / rstep * sx;
-      for (int i = tid; i < want; i += kThreads) {
-        const float v = S->sample[i];
-        if (isfinite(v)) atomicAdd(&S->hist[min(__float_as_uint(dev(v)) >> 20, (unsigned)kBins - 1u)], 1u);
-      }
-      bracket_digits(S, ns, (unsigned)(((unsigned long long)r1 * ns) / nf));
-      lo = __uint_as_float(S->digit[0] << 20);
-      hi = fminf(__uint_as_float((S->digit[1] << 20) | 0xfffffu), FLT_MAX);
-      __syncthreads();
-      col.lo = lo;
-      col.hi = hi;
-      col.n = col.below = 0u;
-      for_window(w, [&](float v) { col(dev(v)); });  // NaN and Inf voxels: |v - m| is NaN or Inf
-      below = __reduce_add_sync(0xffffffffu, col.below);
-      if (lane == 0) {
-        S->seg[warp] = col.n;
-        atomicAdd(&S->below, below);
-      }
+      if (tid == 0) S->below = S->n_copies = S->n_pool = 0u;
+      sample_bracket<20>(S, slots, dev, KeyOfDev{}, ns, (unsigned)(((unsigned long long)r1 * ns) / nf), &col.lo,
+                         &col.hi);
+      col.n = 0;
+      col.below = 0u;
+      for_window<true>(w, [&](float v) { col(dev(v)); });  // NaN and Inf voxels: |v - m| is NaN or Inf
+      col.finish();
       __syncthreads();
       below = S->below;
-      done = holds(below);
+      done = holds();
     }
-    if (done) done = select_cand(lo, hi, r1 - below, even, S, &d1, &d2, [&] { return above(dev, hi); });
+    if (done)
+      done = select_cand(col.n, col.lo, col.hi, r1 - below, even, S, &d1, &d2, [&] { return above(dev, col.hi); });
   }
   if (!done) select_window(w, dev, r1, even, S, &d1, &d2);
   const double mad = even ? 0.5 * ((double)d1 + (double)d2) : (double)d1;
@@ -598,7 +658,7 @@ __global__ void __launch_bounds__(nscale::kThreads, nscale::kBlocksPerSm)
       // slow on this part), combined in double across the block
       float s = 0.0f, sc = 0.0f;
       unsigned finite = 0u;
-      for_window(w, [&](float v) {
+      for_window<false>(w, [&](float v) {
         if (isfinite(v)) {
           neumaier_add(&s, &sc, v);
           ++finite;
@@ -615,7 +675,7 @@ __global__ void __launch_bounds__(nscale::kThreads, nscale::kBlocksPerSm)
         const double mean = sum / (double)nf;
         const float mh = __double2float_rn(mean), ml = __double2float_rn(mean - (double)mh);
         float q = 0.0f, qc = 0.0f;
-        for_window(w, [&](float v) {
+        for_window<false>(w, [&](float v) {
           if (isfinite(v)) {
             const float d = __fsub_rn(__fsub_rn(v, mh), ml);
             neumaier_add(&q, &qc, __fmul_rn(d, d));
@@ -633,7 +693,7 @@ __global__ void __launch_bounds__(nscale::kThreads, nscale::kBlocksPerSm)
         __syncthreads();  // the selection is done with S.hist
         for (int i = tid; i < gfit::kBins; i += kThreads) S.hist[i] = 0u;
         __syncthreads();
-        for_window(w, [&](float v) {
+        for_window<false>(w, [&](float v) {
           const int b = gfit::bin_of(v, k);
           if (b >= 0) atomicAdd(&S.hist[b], 1u);
         });
