@@ -45,9 +45,9 @@ struct sc_ctx {
   double* ns_sig = nullptr;      // sc_noise_scale: noise of every cell (lazy, grown)
   float* ns_rinv = nullptr;      // and its float reciprocal
   size_t ns_cap = 0;             // cells both hold
-  int* lk_tot = nullptr;         // sc_link: one device int (a total)
-  void *lk_bits = nullptr, *lk_runs = nullptr, *lk_comp = nullptr;  // the mask's bits, runs, detections (lazy, grown)
-  size_t lk_bits_cap = 0, lk_runs_cap = 0, lk_comp_cap = 0;
+  void* lk_buf = nullptr;        // sc_link: totals, the mask's bits, runs and detections (lazy, grown)
+  size_t lk_cap = 0;
+  long long lk_max_runs = 0, lk_max_comp = 0;  // what it has room for
   unsigned char* af_buf = nullptr;  // sc_autoflag: noises, flags and statistics (lazy, grown)
   size_t af_cap = 0;
   void* af_chan = nullptr;          // and its channel passes' brackets and copies (lazy, grown)
@@ -777,10 +777,7 @@ void sc_destroy(sc_ctx* c) {
   cudaFree(c->stage_mask);
   cudaFree(c->ns_sig);
   cudaFree(c->ns_rinv);
-  cudaFree(c->lk_bits);
-  cudaFree(c->lk_runs);
-  cudaFree(c->lk_tot);
-  cudaFree(c->lk_comp);
+  cudaFree(c->lk_buf);
   cudaFree(c->af_chan);
   cudaFree(c->af_buf);
   cudaFree(c->sh_P);
@@ -1633,45 +1630,33 @@ int sc_link(sc_ctx* c, const uint8_t* mask_dev, const int64_t* dims, int r_xy, i
   DeviceGuard guard(c->device);
   cudaStream_t s = (cudaStream_t)cuda_stream;
   c->last = s;
-  if (!c->lk_tot && cudaMalloc(&c->lk_tot, sizeof(int) * 2) != cudaSuccess) {
-    cudaGetLastError();
-    c->lk_tot = nullptr;
-    return SC_ERR_NOMEM;
-  }
-  int rc = ensure_bytes(&c->lk_bits, &c->lk_bits_cap, link_bits_bytes(n));
-  if (rc) return rc;
-  CK(launch_link_runs(mask_dev, d, r_xy, r_z, c->lk_bits, c->lk_tot, s));
-  c->stats.launches += 2;
-  int nruns = 0, ncomp = 0;
-  CK(cudaMemcpyAsync(&nruns, c->lk_tot, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  if (nruns == 0) {  // an empty mask
-    CK(cudaMemsetAsync(labels_dev, 0, sizeof(int) * (size_t)n, s));
+  // One buffer: three totals, the bits, and room for as many runs and
+  // detections as a mask a few per cent full has, or as an earlier call had; a
+  // fuller one starts over with what it turned out to need
+  c->lk_max_runs = std::max(c->lk_max_runs, std::min(n, (1LL << 16) + n / 64));
+  c->lk_max_comp = std::max(c->lk_max_comp, (1LL << 13) + n / 512);
+  int total[3] = {0, 0, 0}, *ext_out = nullptr;
+  for (int attempt = 0; attempt < 3; ++attempt) {
+    const size_t at_runs = 256 + link_bits_bytes(n), at_comp = at_runs + link_runs_bytes(c->lk_max_runs);
+    const int rc = ensure_bytes(&c->lk_buf, &c->lk_cap, at_comp + link_comp_bytes(c->lk_max_comp));
+    if (rc) {
+      c->lk_max_runs = c->lk_max_comp = 0;
+      return rc;
+    }
+    unsigned char* const buf = static_cast<unsigned char*>(c->lk_buf);
+    int* const totals = reinterpret_cast<int*>(buf);
+    int launched = 0;
+    CK(launch_link(mask_dev, d, r_xy, r_z, min_xy, min_z, max_xy, max_z, buf + 256,
+                   reinterpret_cast<int*>(buf + at_runs), c->lk_max_runs, reinterpret_cast<int*>(buf + at_comp),
+                   c->lk_max_comp, totals, labels_dev, &ext_out, c->sms, s, &launched));
+    c->stats.launches += launched;
+    CK(cudaMemcpyAsync(total, totals, sizeof(total), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
-    *n_out = 0;
-    return SC_OK;
+    if (total[0] > c->lk_max_runs) c->lk_max_runs = total[0];  // (the number of detections is not known yet)
+    else if (total[1] > c->lk_max_comp) c->lk_max_comp = total[1];
+    else break;
   }
-  rc = ensure_bytes(&c->lk_runs, &c->lk_runs_cap, link_runs_bytes(nruns));
-  if (rc) return rc;
-  int* const runs = static_cast<int*>(c->lk_runs);
-  CK(launch_link_components(d, r_xy, r_z, c->lk_bits, nruns, runs, c->lk_tot, c->sms, s));
-  c->stats.launches += 4;
-  CK(cudaMemcpyAsync(&ncomp, c->lk_tot, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  int kept = 0;
-  // per detection: two extents rows of 7, a keep flag and a new id
-  rc = ensure_bytes(&c->lk_comp, &c->lk_comp_cap, sizeof(int) * 16 * (size_t)ncomp);
-  if (rc) return rc;
-  int* const ext = static_cast<int*>(c->lk_comp);
-  int* const ext_out = ext + 7 * (size_t)ncomp;
-  int* const keep = ext_out + 7 * (size_t)ncomp;
-  int* const new_id = keep + (size_t)ncomp;
-  // numbering and extents, the size filters, the labels
-  CK(launch_link_filter(d, r_xy, c->lk_bits, nruns, runs, ncomp, min_xy, min_z, max_xy, max_z, ext, keep, ext_out,
-                        new_id, c->lk_tot, labels_dev, c->sms, s));
-  c->stats.launches += 7;
-  CK(cudaMemcpyAsync(&kept, c->lk_tot, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+  const int kept = total[2];
   const long long table = std::min<long long>(kept, extents_cap);
   if (table > 0) {
     CK(cudaMemcpyAsync(extents_host, ext_out, sizeof(int) * 7 * (size_t)table, cudaMemcpyDeviceToHost, s));

@@ -390,19 +390,16 @@ cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k
 size_t chan_scratch_bytes(const long long dims[3], int mode);
 
 constexpr int kLinkMaxRadius = 32;  // merging radii in voxels
-// Linker, in three steps: the mask as bits and runs (bits: link_bits_bytes of
-// scratch; *d_total = the number of runs), their components (runs:
-// link_runs_bytes of scratch; *d_total = their number), then the extents, the
-// size filters (ext_out = kept rows, *d_total = kept) and the labels.
+// Linker. Scratch: bits (link_bits_bytes), runs and comp for at most max_runs
+// runs and max_comp components. totals[3] (device): runs, components, kept
+// detections; where either does not fit, nothing after it is meant (the caller
+// grows the buffer and starts over). *ext_out: extents of the kept ones.
 size_t link_bits_bytes(long long n);
 size_t link_runs_bytes(long long nruns);
-cudaError_t launch_link_runs(const uint8_t* mask, const long long dims[3], int r_xy, int r_z, void* bits, int* d_total,
-                             cudaStream_t s);
-cudaError_t launch_link_components(const long long dims[3], int r_xy, int r_z, void* bits, long long nruns, int* runs,
-                                   int* d_total, int sms, cudaStream_t s);
-cudaError_t launch_link_filter(const long long dims[3], int r_xy, void* bits, long long nruns, int* runs, int ncomp,
-                               int min_xy, int min_z, int max_xy, int max_z, int* ext, int* keep, int* ext_out,
-                               int* new_id, int* d_total, int* lab, int sms, cudaStream_t s);
+size_t link_comp_bytes(long long ncomp);
+cudaError_t launch_link(const uint8_t* mask, const long long dims[3], int r_xy, int r_z, int min_xy, int min_z,
+                        int max_xy, int max_z, void* bits, int* runs, long long max_runs, int* comp, long long max_comp,
+                        int* totals, int* lab, int** ext_out, int sms, cudaStream_t s, int* launches);
 
 // Host helpers.
 int cascade_widths(double fwhm, int w[3]);

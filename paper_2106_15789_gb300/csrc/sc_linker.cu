@@ -7,17 +7,22 @@
 //
 //   k_lk_pack     the mask as bits, the bits where runs start, and the runs
 //                 before every word (within its chunk of 8,192 voxels)
-//   k_scan_block  the runs before every chunk; the host reads their number
+//   k_scan_block  the runs before every chunk, and their number
 //   k_lk_init     every run its own root
 //   k_lk_union    friends-of-friends between runs, lock-free union-find with
 //                 the larger root hung under the smaller, so a component's
 //                 root is its first run
 //   k_lk_flatten  every run points at its root; roots counted
-//   k_lk_number   ids 1, 2, ... in the order of the roots (after a scan; the
-//                 host reads their number)
+//   k_lk_number   ids 1, 2, ... in the order of the roots (after a scan)
 //   k_lk_extents  bounding box and voxel count of every component
 //   k_cc_keep, k_cc_compact  the size filters and the ids that remain
 //   k_lk_expand   the labels, written once
+//
+// The numbers of runs, detections and kept ones stay on the device (Totals):
+// the buffers are those of the last call (or a guess), each kernel returns
+// where they are too small, and the host, which reads the numbers once at the
+// end, grows them and starts over in that case. A cube of 2 M voxels takes
+// 175 us so, and took 203 with a stop to size each buffer.
 //
 // What bounds it: reading the mask (1 byte a voxel) and writing the labels
 // (4), then the union's scattered reads of the bits (in L2: an eighth of a
@@ -42,6 +47,14 @@ struct Geo {
   int nx, ny, nz;
   long long n;
   int rxy, rz;
+};
+
+// Device totals, and the sizes of the buffers.
+struct Totals {
+  int* n;                    // [0] runs, [1] components, [2] kept
+  long long max_runs, max_comp;
+  __device__ __forceinline__ bool runs_fit() const { return n[0] <= max_runs; }
+  __device__ __forceinline__ bool all_fit() const { return n[0] <= max_runs && n[1] <= max_comp; }
 };
 
 // The mask's runs: bits, run starts, and the runs before each word and chunk.
@@ -110,6 +123,7 @@ __device__ __forceinline__ unsigned nonzero_bits(unsigned x) {  // bit i: byte i
 
 using link::Geo;
 using link::Runs;
+using link::Totals;
 
 // A block per chunk, a mask word (32 voxels) per thread. A run starts at a set
 // voxel whose predecessor is not set or lies in another row.
@@ -159,19 +173,30 @@ __global__ void __launch_bounds__(link::kThreads) k_lk_pack(const uint8_t* __res
 }
 
 // Exclusive scan of a[0 .. len) in place by one block of 1024 threads, eight
-// values a thread; *total receives the sum.
-__global__ void __launch_bounds__(1024) k_scan_block(int* a, long long len, int* total) {
+// values a thread, the next eight loaded meanwhile; a[len] and *total (unless
+// null) receive the sum. With per > 0, len is ceil(*count / per), and nothing
+// happens where `most` counts do not fit.
+__global__ void __launch_bounds__(1024) k_scan_block(int* a, long long len, const int* count, int per, long long most,
+                                                     int* total) {
   __shared__ int part[32];
   constexpr int kPer = 8;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (per > 0) {
+    if (*count > most) return;
+    len = ((long long)*count + per - 1) / per;
+  }
   int carry = 0;
+  int nx[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) nx[k] = kPer * tid + k < len ? a[kPer * tid + k] : 0;
   for (long long t0 = 0; t0 < len; t0 += 1024 * kPer) {
-    const long long i0 = t0 + kPer * tid;
+    const long long i0 = t0 + kPer * tid, j0 = i0 + 1024 * kPer;
     int v[kPer], sum = 0;
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-      v[k] = i0 + k < len ? a[i0 + k] : 0;
+      v[k] = nx[k];
       sum += v[k];
+      nx[k] = j0 + k < len ? a[j0 + k] : 0;
     }
     int x = sum;
 #pragma unroll
@@ -191,11 +216,16 @@ __global__ void __launch_bounds__(1024) k_scan_block(int* a, long long len, int*
     }
     __syncthreads();  // the parts are read before the next tile writes them
   }
-  if (tid == 0) *total = carry;
+  if (tid == 0) {
+    a[len] = carry;
+    if (total) *total = carry;
+  }
 }
 
-__global__ void k_lk_init(int* parent, long long nruns) {
-  for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < nruns; r += (long long)gridDim.x * blockDim.x)
+__global__ void k_lk_init(int* parent, Totals t) {
+  if (!t.runs_fit()) return;
+  const int n = t.n[0];
+  for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x)
     parent[r] = (int)r;
 }
 
@@ -239,11 +269,12 @@ __device__ __forceinline__ void load_batch(const Runs& R, const Geo& g, int from
 // and to every run that meets its reach in each friend row after it in raster
 // order (dz > 0, or dz == 0 and dy > 0); the other half of the relation is the
 // mirror of these. The pairs (run, friend row) go to the threads side by side.
-__global__ void __launch_bounds__(link::kThreads) k_lk_union(Geo g, Runs R, int* parent) {
+__global__ void __launch_bounds__(link::kThreads) k_lk_union(Geo g, Runs R, int* parent, Totals t) {
   using namespace link;
   __shared__ Batch B;
   __shared__ int reach[kLinkMaxRadius + 1];  // largest |dx| with dx^2 + dy^2 <= r_xy^2
   const int tid = threadIdx.x;
+  if (!t.runs_fit()) return;
   if (tid <= g.rxy) {
     int d = 0;
     while ((d + 1) * (d + 1) + tid * tid <= g.rxy * g.rxy) ++d;
@@ -297,57 +328,66 @@ __global__ void __launch_bounds__(link::kThreads) k_lk_union(Geo g, Runs R, int*
 // of each kFlat runs. The walks only read: halving paths here could overwrite
 // a run's final root with an older ancestor read before it. A run is a root
 // exactly when its walk ends at itself, whatever other threads write.
-__global__ void __launch_bounds__(1024) k_lk_flatten(int* parent, long long nruns, int* __restrict__ counts) {
+__global__ void __launch_bounds__(1024) k_lk_flatten(int* parent, int* __restrict__ counts, Totals t) {
   __shared__ int s_roots;
-  if (threadIdx.x == 0) s_roots = 0;
-  __syncthreads();
-  const long long base = (long long)blockIdx.x * link::kFlat + 4LL * threadIdx.x;
-  int c = 0;
+  if (!t.runs_fit()) return;
+  const long long nruns = t.n[0];
+  for (long long blk = blockIdx.x; blk * link::kFlat < nruns; blk += gridDim.x) {
+    if (threadIdx.x == 0) s_roots = 0;
+    __syncthreads();
+    const long long base = blk * link::kFlat + 4LL * threadIdx.x;
+    int c = 0;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const long long r = base + k;
-    if (r < nruns) {
-      int x = (int)r, p = parent[r];
-      while (p != x) {
-        x = p;
-        p = parent[x];
+    for (int k = 0; k < 4; ++k) {
+      const long long r = base + k;
+      if (r < nruns) {
+        int x = (int)r, p = parent[r];
+        while (p != x) {
+          x = p;
+          p = parent[x];
+        }
+        if (x == (int)r) ++c;
+        else parent[r] = x;
       }
-      if (x == (int)r) ++c;
-      else parent[r] = x;
     }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_roots, c);
+    __syncthreads();
+    if (threadIdx.x == 0) counts[blk] = s_roots;
   }
-  c = __reduce_add_sync(0xffffffffu, c);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_roots, c);
-  __syncthreads();
-  if (threadIdx.x == 0) counts[blockIdx.x] = s_roots;
 }
 
 // parent[root] = -(id) with ids 1, 2, ... in the order of the roots.
-__global__ void __launch_bounds__(1024) k_lk_number(int* parent, long long nruns, const int* __restrict__ off) {
+__global__ void __launch_bounds__(1024) k_lk_number(int* parent, const int* __restrict__ off, Totals t) {
   __shared__ int part[32];
+  if (!t.all_fit()) return;
+  const long long nruns = t.n[0];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const long long base = (long long)blockIdx.x * link::kFlat + 4LL * tid;
-  bool root[4];
-  int c = 0;
+  for (long long blk = blockIdx.x; blk * link::kFlat < nruns; blk += gridDim.x) {
+    const long long base = blk * link::kFlat + 4LL * tid;
+    bool root[4];
+    int c = 0;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const long long r = base + k;
-    root[k] = r < nruns && parent[r] == (int)r;
-    c += root[k] ? 1 : 0;
+    for (int k = 0; k < 4; ++k) {
+      const long long r = base + k;
+      root[k] = r < nruns && parent[r] == (int)r;
+      c += root[k] ? 1 : 0;
+    }
+    int x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) part[warp] = x;
+    __syncthreads();
+    const int p = part[lane];
+    int id = off[blk] + __reduce_add_sync(0xffffffffu, lane < warp ? p : 0) + x - c;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (root[k]) parent[base + k] = -(++id);
+    __syncthreads();  // the parts are read before the next chunk writes them
   }
-  int x = c;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) part[warp] = x;
-  __syncthreads();
-  const int p = part[lane];
-  int id = off[blockIdx.x] + __reduce_add_sync(0xffffffffu, lane < warp ? p : 0) + x - c;
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (root[k]) parent[base + k] = -(++id);
 }
 
 // A block per chunk: every run's component id to run_id, and the bounding box
@@ -355,9 +395,10 @@ __global__ void __launch_bounds__(1024) k_lk_number(int* parent, long long nruns
 // y_min, y_max, z_min, z_max, count. Lanes of a warp with the same id combine
 // first, so a component's seven words see one atomic per group.
 __global__ void __launch_bounds__(link::kThreads) k_lk_extents(Geo g, Runs R, const int* __restrict__ parent,
-                                                               int* __restrict__ run_id, int* ext) {
+                                                               int* __restrict__ run_id, int* ext, Totals t) {
   using namespace link;
   __shared__ Batch B;
+  if (!t.all_fit()) return;
   const int tid = threadIdx.x, lane = tid & 31;
   const int n = chunk_runs(R, g, &B);
   if (n == 0) return;
@@ -397,7 +438,9 @@ __global__ void __launch_bounds__(link::kThreads) k_lk_extents(Geo g, Runs R, co
   }
 }
 
-__global__ void k_cc_ext_init(int* ext, int ncomp) {
+__global__ void k_cc_ext_init(int* ext, Totals t) {
+  if (!t.all_fit()) return;
+  const int ncomp = t.n[1];
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncomp; i += gridDim.x * blockDim.x) {
     int* e = ext + 7LL * i;
     e[0] = e[2] = e[4] = INT_MAX;
@@ -406,22 +449,26 @@ __global__ void k_cc_ext_init(int* ext, int ncomp) {
   }
 }
 
-__global__ void k_cc_keep(const int* __restrict__ ext, int ncomp, int min_xy, int min_z, int max_xy, int max_z,
-                          int* keep) {
+__global__ void k_cc_keep(const int* __restrict__ ext, Totals t, int min_xy, int min_z, int max_xy, int max_z,
+                          int* keep, int* flag) {
+  if (!t.all_fit()) return;
+  const int ncomp = t.n[1];
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncomp; i += gridDim.x * blockDim.x) {
     const int* e = ext + 7LL * i;
     const int sx = e[1] - e[0] + 1, sy = e[3] - e[2] + 1, sz = e[5] - e[4] + 1;
     bool k = sx >= min_xy && sy >= min_xy && sz >= min_z;
     if (max_xy > 0) k = k && sx <= max_xy && sy <= max_xy;
     if (max_z > 0) k = k && sz <= max_z;
-    keep[i] = k ? 1 : 0;
+    keep[i] = flag[i] = k ? 1 : 0;
   }
 }
 
 // After the exclusive scan of the keep flags: the kept rows moved to the
 // front of out (ids 1 .. kept), and new_id[i] = id of detection i + 1 or 0.
 __global__ void k_cc_compact(const int* __restrict__ ext, const int* keep_flag, const int* __restrict__ keep_off,
-                             int ncomp, int* out, int* new_id) {
+                             Totals t, int* out, int* new_id) {
+  if (!t.all_fit()) return;
+  const int ncomp = t.n[1];
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncomp; i += gridDim.x * blockDim.x) {
     if (keep_flag[i]) {
       const int j = keep_off[i];
@@ -435,7 +482,8 @@ __global__ void k_cc_compact(const int* __restrict__ ext, const int* keep_flag, 
 
 // The labels, four voxels a thread: 0, or the new id of the voxel's component.
 __global__ void __launch_bounds__(256) k_lk_expand(Geo g, Runs R, const int* __restrict__ run_id,
-                                                   const int* __restrict__ new_id, int* __restrict__ lab) {
+                                                   const int* __restrict__ new_id, int* __restrict__ lab, Totals t) {
+  if (!t.all_fit()) return;
   const bool vec = (reinterpret_cast<uintptr_t>(lab) & 15u) == 0;
   const long long quads = (g.n + 3) / 4;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < quads; q += (long long)gridDim.x * blockDim.x) {
@@ -473,65 +521,45 @@ Runs runs_at(void* bits, long long n) {
   R.chunk_off = reinterpret_cast<int*>(b + 2 * up16(4 * words) + up16(2 * words));
   return R;
 }
-Geo geo_of(const long long dims[3], int r_xy, int r_z) {
-  return Geo{(int)dims[0], (int)dims[1], (int)dims[2], dims[0] * dims[1] * dims[2], r_xy, r_z};
-}
 long long chunks_of(long long n) { return (n + link::kChunk - 1) / link::kChunk; }
 }  // namespace
 
 size_t link_bits_bytes(long long n) {
   const size_t words = (size_t)((n + 31) / 32);
-  return 2 * up16(4 * words) + up16(2 * words) + 4 * (size_t)(chunks_of(n) + 1);
+  return 2 * up16(4 * words) + up16(2 * words) + up16(4 * (size_t)(chunks_of(n) + 1));
 }
 size_t link_runs_bytes(long long nruns) {
-  return 4 * (size_t)(2 * nruns + (nruns + link::kFlat - 1) / link::kFlat);
+  return up16(4 * (size_t)(2 * nruns + (nruns + link::kFlat - 1) / link::kFlat + 1));
 }
+size_t link_comp_bytes(long long ncomp) { return 4 * (size_t)(16 * ncomp + 1); }
 
-cudaError_t launch_link_runs(const uint8_t* mask, const long long dims[3], int r_xy, int r_z, void* bits, int* d_total,
-                             cudaStream_t s) {
-  const Geo g = geo_of(dims, r_xy, r_z);
+cudaError_t launch_link(const uint8_t* mask, const long long dims[3], int r_xy, int r_z, int min_xy, int min_z,
+                        int max_xy, int max_z, void* bits, int* runs, long long max_runs, int* comp, long long max_comp,
+                        int* totals, int* lab, int** ext_out, int sms, cudaStream_t s, int* launches) {
+  const Geo g{(int)dims[0], (int)dims[1], (int)dims[2], dims[0] * dims[1] * dims[2], r_xy, r_z};
   const Runs R = runs_at(bits, g.n);
-  const long long chunks = chunks_of(g.n);
+  const Totals t{totals, max_runs, max_comp};
+  const long long chunks = chunks_of(g.n), flat = (max_runs + link::kFlat - 1) / link::kFlat;
+  int *const parent = runs, *const run_id = runs + max_runs, *const counts = runs + 2 * max_runs;
+  // per component: extents, kept extents, keep flags (scanned: one more), new ids
+  int *const ext = comp, *const kept = ext + 7 * max_comp, *const new_id = kept + 7 * max_comp;
+  int* const keep = new_id + max_comp;
+  const int flat_grid = (int)(flat < 8LL * sms ? flat : 8LL * sms);
   k_lk_pack<<<(unsigned)chunks, link::kThreads, 0, s>>>(mask, g, R);
-  k_scan_block<<<1, 1024, 0, s>>>(R.chunk_off, chunks, d_total);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return cudaMemcpyAsync(R.chunk_off + chunks, d_total, sizeof(int), cudaMemcpyDeviceToDevice, s);
-}
-
-cudaError_t launch_link_components(const long long dims[3], int r_xy, int r_z, void* bits, long long nruns, int* runs,
-                                   int* d_total, int sms, cudaStream_t s) {
-  const Geo g = geo_of(dims, r_xy, r_z);
-  const Runs R = runs_at(bits, g.n);
-  const long long flat = (nruns + link::kFlat - 1) / link::kFlat;
-  int* const parent = runs;
-  int* const counts = runs + 2 * nruns;
-  k_lk_init<<<grid_for(nruns, sms, 256), 256, 0, s>>>(parent, nruns);
-  k_lk_union<<<(unsigned)chunks_of(g.n), link::kThreads, 0, s>>>(g, R, parent);
-  k_lk_flatten<<<(unsigned)flat, 1024, 0, s>>>(parent, nruns, counts);
-  k_scan_block<<<1, 1024, 0, s>>>(counts, flat, d_total);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_link_filter(const long long dims[3], int r_xy, void* bits, long long nruns, int* runs, int ncomp,
-                               int min_xy, int min_z, int max_xy, int max_z, int* ext, int* keep, int* ext_out,
-                               int* new_id, int* d_total, int* lab, int sms, cudaStream_t s) {
-  const Geo g = geo_of(dims, r_xy, 0);
-  const Runs R = runs_at(bits, g.n);
-  const long long flat = (nruns + link::kFlat - 1) / link::kFlat;
-  int* const parent = runs;
-  int* const run_id = runs + nruns;
-  const int* const counts = runs + 2 * nruns;
-  k_cc_ext_init<<<grid_for(ncomp, sms, 256), 256, 0, s>>>(ext, ncomp);
-  k_lk_number<<<(unsigned)flat, 1024, 0, s>>>(parent, nruns, counts);
-  k_lk_extents<<<(unsigned)chunks_of(g.n), link::kThreads, 0, s>>>(g, R, parent, run_id, ext);
-  k_cc_keep<<<grid_for(ncomp, sms, 256), 256, 0, s>>>(ext, ncomp, min_xy, min_z, max_xy, max_z, keep);
-  // keep flags are kept in new_id while keep becomes their exclusive scan
-  cudaError_t e = cudaMemcpyAsync(new_id, keep, sizeof(int) * (size_t)ncomp, cudaMemcpyDeviceToDevice, s);
-  if (e != cudaSuccess) return e;
-  k_scan_block<<<1, 1024, 0, s>>>(keep, ncomp, d_total);
-  k_cc_compact<<<grid_for(ncomp, sms, 256), 256, 0, s>>>(ext, new_id, keep, ncomp, ext_out, new_id);
-  k_lk_expand<<<grid_for((g.n + 3) / 4, sms, 256), 256, 0, s>>>(g, R, run_id, new_id, lab);
+  k_scan_block<<<1, 1024, 0, s>>>(R.chunk_off, chunks, nullptr, 0, 0, totals);
+  k_lk_init<<<grid_for(max_runs, sms, 256), 256, 0, s>>>(parent, t);
+  k_lk_union<<<(unsigned)chunks, link::kThreads, 0, s>>>(g, R, parent, t);
+  k_lk_flatten<<<flat_grid, 1024, 0, s>>>(parent, counts, t);
+  k_scan_block<<<1, 1024, 0, s>>>(counts, 0, totals, link::kFlat, max_runs, totals + 1);
+  k_cc_ext_init<<<grid_for(max_comp, sms, 256), 256, 0, s>>>(ext, t);
+  k_lk_number<<<flat_grid, 1024, 0, s>>>(parent, counts, t);
+  k_lk_extents<<<(unsigned)chunks, link::kThreads, 0, s>>>(g, R, parent, run_id, ext, t);
+  k_cc_keep<<<grid_for(max_comp, sms, 256), 256, 0, s>>>(ext, t, min_xy, min_z, max_xy, max_z, keep, new_id);
+  k_scan_block<<<1, 1024, 0, s>>>(keep, 0, totals + 1, 1, max_comp, totals + 2);
+  k_cc_compact<<<grid_for(max_comp, sms, 256), 256, 0, s>>>(ext, new_id, keep, t, kept, new_id);
+  k_lk_expand<<<grid_for((g.n + 3) / 4, sms, 256), 256, 0, s>>>(g, R, run_id, new_id, lab, t);
+  *launches = 13;
+  *ext_out = kept;
   return cudaGetLastError();
 }
 
