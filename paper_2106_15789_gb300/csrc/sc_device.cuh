@@ -10,6 +10,16 @@
 
 namespace sc {
 
+// Lets the next kernel, where it is a chained one, take its places now.
+__device__ __forceinline__ void chain_open() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// First thing in a chained kernel: the same, then the wait for the end of the
+// kernel before it (which has itself waited for its own), its writes visible.
+// Nothing is read or written before it.
+__device__ __forceinline__ void chain_begin() {
+  chain_open();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Order-preserving uint32 key of a float: key(a) < key(b) iff a < b for
 // non-NaN a, b (with -0 just below +0).
 __device__ __forceinline__ unsigned int fkey(float s) {

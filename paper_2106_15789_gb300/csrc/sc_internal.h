@@ -308,6 +308,36 @@ inline long long z_chunks(const SmoothArgs& a, long long tiles, int sms, long lo
 }
 
 // ---------------------------------------------------------------------------
+// Launch of a small kernel that follows another one closely (programmatic
+// dependent launch): its blocks take their places while the kernel before it
+// still runs, and wait for its end in chain_begin(), the first thing every
+// such kernel does. That hides the launch and the first fetch of the code,
+// about 1.5 us of each; the kernels around a measurement's selection are
+// ten to eighteen a pair. The wide kernels (smoothing, candidate pass) are
+// launched plainly: their blocks would hold an SM's shared memory while they
+// wait. cluster: blocks per cluster (0: none, or the kernel's own).
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, unsigned cluster,
+                           cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 1;
+  if (cluster > 0) {
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
+  cfg.attrs = at;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Launchers (all enqueue on `s`, return cudaError_t of the launch).
 cudaError_t launch_hist(const float* x, long long n, DevState* st, unsigned long long* hist, int win,
                         int want_maxabs, int sms, cudaStream_t s);

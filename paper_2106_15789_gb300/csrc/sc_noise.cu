@@ -441,6 +441,7 @@ __global__ void __cluster_dims__(kPlanCluster, 1, 1) __launch_bounds__(kPlanThre
   __shared__ NoisePlan s_plan;
   __shared__ int s_bins[2];
   __shared__ unsigned int s_T[2];
+  chain_begin();
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -537,8 +538,8 @@ cudaError_t launch_plan(DevState* st, unsigned long long* hist, int win, const f
                         Lists L, float threshold, int clip, int std_mode, unsigned int force_flags,
                         cudaStream_t s) {
   const size_t smem = (kNumBins + 1) * sizeof(unsigned long long);
-  k_plan<<<kPlanCluster, kPlanThreads, smem, s>>>(st, hist, win, src, n_total, L, threshold, clip, std_mode, force_flags);
-  return cudaGetLastError();
+  return launch_chained(k_plan, kPlanCluster, kPlanThreads, smem, 0, s, st, hist, win, src, n_total, L, threshold, clip,
+                        std_mode, force_flags);
 }
 
 // ---------------------------------------------------------------------------
@@ -605,6 +606,7 @@ __device__ __forceinline__ void p2_load(const float* __restrict__ src, long long
 __global__ void __launch_bounds__(kP2Threads, 2) k_pass2(const float* __restrict__ src, long long n,
                                                          uint32_t* mbits, DevState* st, Lists L) {
   extern __shared__ __align__(16) unsigned char p2_smem[];
+  chain_open();
   const NoisePlan p = st->plan;
   if (p.flags & (PLAN_EMPTY | PLAN_STD)) return;
   const bool do_clip = (p.flags & PLAN_CLIP) && !(p.flags & PLAN_CLIP_FULL) && mbits != nullptr;
@@ -818,6 +820,7 @@ __device__ void sel_result(DevState* st, SelJob* J, int which, int pair);
 
 __global__ void __launch_bounds__(256) k_sel_round(DevState* st, int which, int r) {
   __shared__ unsigned int sh[kSelBins];
+  chain_begin();
   SelJob* J = which ? &st->sel_mad : &st->sel_med;
   const NoisePlan& p = st->plan;
   if (!sel_by_full_passes(p)) return;
@@ -881,6 +884,7 @@ __global__ void __launch_bounds__(256) k_sel_round(DevState* st, int which, int 
 __global__ void __launch_bounds__(256) k_sel_succ(DevState* st, int which, int pair) {
   __shared__ unsigned long long s_c[8];
   __shared__ unsigned int s_m[8];
+  chain_begin();
   SelJob* J = which ? &st->sel_mad : &st->sel_med;
   const NoisePlan& p = st->plan;
   if (!sel_by_full_passes(p)) return;
@@ -959,12 +963,10 @@ __device__ void sel_result(DevState* st, SelJob* J, int which, int pair) {
 cudaError_t launch_select_full(DevState* st, int which, int pair, int sms, cudaStream_t s) {
   const int grid = 2 * sms;
   for (int r = 0; r < 3; ++r) {
-    k_sel_round<<<grid, 256, 0, s>>>(st, which, r);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(k_sel_round, grid, 256, 0, 0, s, st, which, r);
     if (e != cudaSuccess) return e;
   }
-  k_sel_succ<<<grid, 256, 0, s>>>(st, which, pair);
-  return cudaGetLastError();
+  return launch_chained(k_sel_succ, grid, 256, 0, 0, s, st, which, pair);
 }
 
 // ---------------------------------------------------------------------------
@@ -1037,6 +1039,7 @@ __global__ void __launch_bounds__(256) k_std_pass(const float* __restrict__ x, l
                                                   int pair) {
   __shared__ double s_a[8], s_b[8];
   __shared__ unsigned s_n[8];
+  chain_begin();
   if ((st->plan.flags & PLAN_EMPTY) || (second && !st->std_again)) return;
   const float scale = st->std_scale, shift = __fmul_rn(st->std_shift, scale);
   float p1[2] = {0.0f, 0.0f}, p2[2] = {0.0f, 0.0f};
@@ -1093,9 +1096,9 @@ __global__ void __launch_bounds__(256) k_std_pass(const float* __restrict__ x, l
 cudaError_t launch_std(const float* src, long long n, DevState* st, int pair, int sms, cudaStream_t s) {
   const long long want = (n + 4095) / 4096;  // four 16-byte loads a thread
   const int grid = (int)(want > 6LL * sms ? 6LL * sms : want);
-  k_std_pass<<<grid, 256, 0, s>>>(src, n, st, 0, pair);
-  k_std_pass<<<grid, 256, 0, s>>>(src, n, st, 1, pair);
-  return cudaGetLastError();
+  const cudaError_t e = launch_chained(k_std_pass, grid, 256, 0, 0, s, src, n, st, 0, pair);
+  if (e != cudaSuccess) return e;
+  return launch_chained(k_std_pass, grid, 256, 0, 0, s, src, n, st, 1, pair);
 }
 
 // ---------------------------------------------------------------------------
@@ -1144,6 +1147,7 @@ __device__ __forceinline__ void clip_store(uint32_t* mbits, long long ch, int la
 
 __global__ void __launch_bounds__(256) k_clip_full(const float* __restrict__ src, long long n, uint32_t* mbits,
                                                    DevState* st, Lists L) {
+  chain_begin();
   const NoisePlan& p = st->plan;
   if (!(p.flags & PLAN_CLIP) || (p.flags & PLAN_EMPTY)) return;
   const float sg = st->sigma_cur;
@@ -1175,8 +1179,7 @@ cudaError_t launch_clip(const float* src, long long n, uint32_t* mbits, DevState
   const long long cap = (long long)(per_sm > 0 ? per_sm : 4) * sms;
   long long want = (n + 1023) / 1024;
   int grid = (int)(want < 1 ? 1 : (want > cap ? cap : want));
-  k_clip_full<<<grid, 256, 0, s>>>(src, n, mbits, st, L);
-  return cudaGetLastError();
+  return launch_chained(k_clip_full, grid, 256, 0, 0, s, src, n, mbits, st, L);
 }
 
 

@@ -274,6 +274,7 @@ __global__ void __launch_bounds__(select::kThreads, 1)
     k_select(DevState* st, const float* src, long long n, Lists L, int pair, int part, int all) {
   using namespace select;
   __shared__ Smem S;
+  chain_begin();
   cg::cluster_group cl = cg::this_cluster();
   const NoisePlan& p = st->plan;
   const int flags = p.flags;
@@ -367,6 +368,7 @@ __device__ __forceinline__ bool mad_by_grid(const NoisePlan& p) {
 __global__ void __launch_bounds__(kMadThreads) k_mad_digits(DevState* st, Lists L) {
   using namespace select;
   __shared__ unsigned hist[kBins];
+  chain_begin();
   const NoisePlan& p = st->plan;
   if (!mad_by_grid(p)) return;
   for (int i = threadIdx.x; i < kBins; i += kMadThreads) hist[i] = 0u;
@@ -407,6 +409,7 @@ __global__ void __launch_bounds__(kMadThreads) k_mad_digits(DevState* st, Lists 
 __global__ void __launch_bounds__(kMadThreads) k_mad_compact(DevState* st, Lists L) {
   using namespace select;
   __shared__ unsigned part[kMadThreads / 32], s_digit, s_rank, s_count;
+  chain_begin();
   const NoisePlan& p = st->plan;
   if (!mad_by_grid(p)) return;
   const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
@@ -556,8 +559,7 @@ struct ClusterLaunch {
 };
 cudaError_t launch_part(DevState* st, const float* src, long long n, const Lists& L, int pair, int part, int all,
                         unsigned blocks, cudaStream_t s) {
-  ClusterLaunch c(blocks, s);
-  return cudaLaunchKernelEx(&c.cfg, k_select, st, src, n, L, pair, part, all);
+  return launch_chained(k_select, blocks, select::kThreads, 0, blocks, s, st, src, n, L, pair, part, all);
 }
 }  // namespace
 
@@ -584,9 +586,8 @@ cudaError_t launch_select_lists(DevState* st, const float* src, long long n, Lis
   *launches = 4;
   cudaError_t e = launch_part(st, src, n, L, pair, PART_MEDIAN, all, 8u, s);
   if (e != cudaSuccess) return e;
-  k_mad_digits<<<2 * sms, kMadThreads, 0, s>>>(st, L);
-  k_mad_compact<<<2 * sms, kMadThreads, 0, s>>>(st, L);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_chained(k_mad_digits, 2 * sms, kMadThreads, 0, 0, s, st, L)) != cudaSuccess) return e;
+  if ((e = launch_chained(k_mad_compact, 2 * sms, kMadThreads, 0, 0, s, st, L)) != cudaSuccess) return e;
   return launch_part(st, src, n, L, pair, PART_MAD, all, 8u, s);
 }
 

@@ -92,6 +92,8 @@ __global__ void __launch_bounds__(kListThreads) k_share_list(const uint32_t* __r
                                                              const float* __restrict__ C, Half16 h16, long long n,
                                                              long long nx, long long ny, ShareArgs sh, int R) {
   __shared__ unsigned short s_off[kListThreads / 32][kListRun];
+  if (FILL) chain_begin();
+  else chain_open();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lanes_below = (1u << lane) - 1u;
   const long long nwords = (n + 31) / 32, nrun = (nwords + 31) / 32;
@@ -177,6 +179,7 @@ __global__ void __launch_bounds__(kListThreads) k_share_list(const uint32_t* __r
 __global__ void __launch_bounds__(1024) k_share_scan1(const unsigned* __restrict__ cnt, unsigned* __restrict__ offs,
                                                       unsigned long long* __restrict__ bsum, long long m) {
   __shared__ unsigned wsum[32];
+  chain_begin();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const long long base = (long long)blockIdx.x * kScanChunk + 4 * t;
   unsigned v[4], tot = 0;
@@ -216,6 +219,7 @@ __global__ void __launch_bounds__(1024) k_share_scan2(unsigned* __restrict__ off
                                                       const unsigned long long* __restrict__ bsum, long long m,
                                                       ShareState* ss, unsigned long long cap) {
   __shared__ unsigned long long red[32];
+  chain_begin();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   unsigned long long p = 0;
   for (long long i = t; i < blockIdx.x; i += 1024) p += bsum[i];
@@ -790,10 +794,14 @@ cudaError_t launch_share_prep(const SmoothArgs& a, const ShareArgs& sh, int sms,
   const long long per = (long long)kListRun * kListAhead * (kListThreads / 32), want = (n + per - 1) / per;
   const unsigned list_grid = (unsigned)(want < 8LL * sms ? want : 8LL * sms);
   k_share_list<false><<<list_grid, kListThreads, 0, s>>>(a.mbits, a.C, a.h16, n, a.nx, a.ny, sh, R);
-  k_share_scan1<<<(unsigned)nblk, 1024, 0, s>>>(sh.cnt, sh.offs, sh.bsum, m);
-  k_share_scan2<<<(unsigned)nblk, 1024, 0, s>>>(sh.offs, sh.bsum, m, sh.ss, sh.cap);
-  k_share_list<true><<<list_grid, kListThreads, 0, s>>>(a.mbits, a.C, a.h16, n, a.nx, a.ny, sh, R);
-  return cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = launch_chained(k_share_scan1, (unsigned)nblk, 1024, 0, 0, s, sh.cnt, sh.offs, sh.bsum, m);
+  if (e == cudaSuccess)
+    e = launch_chained(k_share_scan2, (unsigned)nblk, 1024, 0, 0, s, sh.offs, sh.bsum, m, sh.ss, sh.cap);
+  if (e == cudaSuccess)
+    e = launch_chained(k_share_list<true>, list_grid, kListThreads, 0, 0, s, a.mbits, a.C, a.h16, n, (long long)a.nx,
+                       (long long)a.ny, sh, R);
+  return e;
 }
 
 cudaError_t launch_smooth_p(const SmoothArgs& a, const ShareArgs& sh, int sms, cudaStream_t s, bool* done) {
