@@ -119,6 +119,27 @@ __device__ __forceinline__ unsigned mad_key(float x, float a, float b, bool even
   return __float_as_uint(fabsf(d)) | 0x80000000u;
 }
 
+// |x - m| of the median m = (a + b) / 2, faithfully rounded: -m = h + l
+// exactly (a TwoSum of the halves; l is 0 for an odd count), then x + h as a
+// sum and its error, to which l is added.
+struct Deviation {
+  float h, l;
+  __device__ __forceinline__ float operator()(float x) const {
+    const float t = __fadd_rn(x, h);
+    const float b = __fsub_rn(t, x);
+    const float e = __fadd_rn(__fsub_rn(x, __fsub_rn(t, b)), __fsub_rn(h, b));
+    return fabsf(__fadd_rn(t, __fadd_rn(e, l)));
+  }
+};
+__device__ __forceinline__ Deviation deviation_of(float a, float b) {
+  const float ha = -0.5f * a, hb = -0.5f * b;
+  Deviation d;
+  d.h = a == b ? -a : __fadd_rn(ha, hb);
+  const float bb = __fsub_rn(d.h, ha);
+  d.l = a == b ? 0.0f : __fadd_rn(__fsub_rn(ha, __fsub_rn(d.h, bb)), __fsub_rn(hb, bb));
+  return d;
+}
+
 // Order statistic `rank` (and, with want_next, rank + 1) of key_of(x) over
 // the finite values x of src[0 .. n), streamed from memory: radix digits of
 // 11, 11 and 10 bits counted in a shared histogram. All threads call it.
@@ -266,7 +287,7 @@ __device__ void block_noise(const float* __restrict__ src, long long n, int mode
 // What bounds it: instruction issue, with the loads of a tile before it (two
 // blocks an SM hide each other's). Of 600 x 600 x 1024 voxels, the form with
 // the spectrum in registers, 32 rounds of bisection for each of the four order
-// statistics and one block of 8 warps an SM took 7.97 ms; this one 1.64 ms.
+// statistics and one block of 8 warps an SM took 7.97 ms; this one 1.60 ms.
 constexpr int kPixTile = 16;         // pixels of a row (64 bytes of each plane), a warp each
 constexpr int kPixThreads = 32 * kPixTile;
 constexpr int kPixPitch = kPixTile + 1;
@@ -315,17 +336,22 @@ __device__ __noinline__ float warp_bisect(float* col, int nz, Of of, unsigned ra
 // nearest, a monotone function of the value) are counted; the values of the
 // rank's step are ranked directly, or, more than 32 of them, their smallest
 // and largest become the next range. A range too small to divide: by bisection.
-template <class Of>
-__device__ __forceinline__ void warp_select(float* col, int nz, Of of, float lo, float hi, unsigned rank,
+// first(v, place) is what the first count takes as of(v) (it may also replace
+// the value in shared memory by that).
+template <class Of, class First>
+__device__ __forceinline__ void warp_select(float* col, int nz, Of of, First first, float lo, float hi, unsigned rank,
                                             bool want_next, unsigned* counts, float* list, float* v1, float* v2) {
   const unsigned lane = threadIdx.x & 31u;
   unsigned r = rank, cnt = kNone;  // rank in the range, and its values (at first: all)
   float found = lo;
+  bool counted = false;
   while (lo < hi) {
     // halves, so that hi - lo cannot overflow; the step is in the low bits of
     // a sum with 1.5 * 2^23
     const float magic = 12582912.0f, h0 = -0.5f * lo, inv = (float)(kSteps - 1) / (0.5f * hi + h0);
     if (!(inv <= FLT_MAX)) {
+      if (!counted) for_spectrum(col, nz, [&](float x, float* at) { first(x, at); });
+      __syncwarp();
       *v1 = warp_bisect(col, nz, of, rank);
       *v2 = want_next ? warp_bisect(col, nz, of, rank + 1u) : *v1;
       return;
@@ -335,10 +361,18 @@ __device__ __forceinline__ void warp_select(float* col, int nz, Of of, float lo,
     for (int j = 0; j < kSteps / 128; ++j)
       reinterpret_cast<uint4*>(counts)[j * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
-    for_spectrum(col, nz, [&](float x, float*) {
-      const float v = of(x);
-      if (v >= lo && v <= hi) atomicAdd(counts + step(v), 1u);  // (false for NaN)
-    });
+    if (!counted) {
+      for_spectrum(col, nz, [&](float x, float* at) {
+        const float v = first(x, at);
+        if (v >= lo && v <= hi) atomicAdd(counts + step(v), 1u);  // (false for NaN)
+      });
+    } else {
+      for_spectrum(col, nz, [&](float x, float*) {
+        const float v = of(x);
+        if (v >= lo && v <= hi) atomicAdd(counts + step(v), 1u);
+      });
+    }
+    counted = true;
     __syncwarp();
     const uint4 c0 = reinterpret_cast<const uint4*>(counts)[2 * lane];
     const uint4 c1 = reinterpret_cast<const uint4*>(counts)[2 * lane + 1];
@@ -416,24 +450,12 @@ __device__ __forceinline__ void warp_select(float* col, int nz, Of of, float lo,
   *v2 = fkey_inv(__reduce_min_sync(0xffffffffu, above));
 }
 
-// |x - m|, m = (a + b) / 2, with -m = h + l exactly: faithfully rounded (one
-// subtraction when l is 0, as for an odd count).
-struct PixDev {
-  float h, l;
-  __device__ __forceinline__ float operator()(float x) const {
-    const float t = __fadd_rn(x, h);
-    const float b = __fsub_rn(t, x);
-    const float e = __fadd_rn(__fsub_rn(x, __fsub_rn(t, b)), __fsub_rn(h, b));
-    return fabsf(__fadd_rn(t, __fadd_rn(e, l)));
-  }
-};
-
 // ---- per-channel median and MAD by passes over the whole cube ---------------
 //
 // What bounds it: the two passes' reads of the cube. On 600 x 600 x 1024
 // voxels the form with one block per channel (seven passes over each plane by
 // 304 blocks, whose planes do not fit L2 together, and a match_any histogram
-// per value) took 11.3 ms; these kernels take 1.1 ms.
+// per value) took 11.3 ms; these kernels take 0.92 ms.
 constexpr int kChanSample = 4096;         // values sampled per plane, four a thread
 constexpr long long kChanMinPlane = 1LL << 15;  // smaller planes: one block streams them as fast
 constexpr int kPassThreads = 256;
@@ -446,7 +468,7 @@ struct Chan {
   float lo, hi;
   unsigned finite, below, n;  // finite values, those under lo, copies (may exceed the room)
   float ma, mb;               // the two middle values
-  int even;
+  Deviation dev;                 // |x - m| of their mean
 };
 
 // The digits whose cumulative ranges in S->hist hold ranks ra and rb, and the
@@ -620,7 +642,7 @@ __global__ void __launch_bounds__(flag::kThreads, 1)
   __shared__ Scratch S;
   float lo, hi;
   plane_bracket<21>(cube + (long long)blockIdx.x * plane, plane, [](float x) { return x; }, KeyOfValue{}, &S, &lo, &hi);
-  if (threadIdx.x == 0) ch[blockIdx.x] = Chan{lo, hi, 0u, 0u, 0u, 0.0f, 0.0f, 0};
+  if (threadIdx.x == 0) ch[blockIdx.x] = Chan{lo, hi, 0u, 0u, 0u, 0.0f, 0.0f, Deviation{0.0f, 0.0f}};
 }
 
 // A pass over the cube: the values (DEV: their |x - m|) of every channel under
@@ -633,7 +655,6 @@ __global__ void __launch_bounds__(flag::kPassThreads, 4)
   using namespace flag;
   __shared__ float stage[kPassWarps][kPassRun];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned lanes_below = (1u << lane) - 1u;
   const long long runs = (plane + kPassRun - 1) / kPassRun, total = runs * nz;
   const long long warps = (long long)gridDim.x * kPassWarps;
   const bool vec = (plane & 3) == 0 && (reinterpret_cast<uintptr_t>(cube) & 15u) == 0;
@@ -643,8 +664,8 @@ __global__ void __launch_bounds__(flag::kPassThreads, 4)
     const long long p0 = (it - z * runs) * kPassRun;
     const float* src = cube + z * plane + p0;
     const int left = (int)min((long long)kPassRun, plane - p0);
-    const float lo = ch[z].lo, hi = ch[z].hi, ma = ch[z].ma, mb = ch[z].mb;
-    const bool even = ch[z].even != 0;
+    const float lo = ch[z].lo, hi = ch[z].hi;
+    const Deviation dev = ch[z].dev;
     float v[kQ][4];
     if (vec && left == kPassRun) {
 #pragma unroll
@@ -661,6 +682,7 @@ __global__ void __launch_bounds__(flag::kPassThreads, 4)
           v[q][c] = i < left ? __ldg(src + i) : __int_as_float(0x7fc00000);
         }
     }
+    // every lane copies to its own column: room for all its values, no votes
     unsigned finite = 0u, below = 0u;
     int n = 0;
 #pragma unroll
@@ -669,28 +691,30 @@ __global__ void __launch_bounds__(flag::kPassThreads, 4)
       for (int c = 0; c < 4; ++c) {
         float a = v[q][c];
         const bool ok = fabsf(a) <= FLT_MAX;  // false for NaN and Inf
-        if (DEV) a = abs_dev(a, ma, mb, even);
-        if (!DEV) finite += ok ? 1u : 0u;
-        below += (ok && a < lo) ? 1u : 0u;
-        const bool in = ok && a >= lo && a <= hi;
-        const unsigned b = __ballot_sync(0xffffffffu, in);
-        if (in) stage[warp][n + __popc(b & lanes_below)] = a;
-        n += __popc(b);
+        if (DEV) a = dev(a);
+        else finite += ok ? 1u : 0u;
+        const bool under = ok && a < lo;
+        below += under ? 1u : 0u;
+        if (ok && !under && a <= hi) stage[warp][32 * n++ + lane] = a;
       }
     finite = __reduce_add_sync(0xffffffffu, finite);
     below = __reduce_add_sync(0xffffffffu, below);
+    int x = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
     unsigned at = 0u;
-    if (lane == 0) {
+    if (lane == 31) {
       if (finite) atomicAdd(&ch[z].finite, finite);
       if (below) atomicAdd(&ch[z].below, below);
-      if (n) at = atomicAdd(&ch[z].n, (unsigned)n);
+      if (x) at = atomicAdd(&ch[z].n, (unsigned)x);
     }
-    at = __shfl_sync(0xffffffffu, at, 0);
-    __syncwarp();
+    at = __shfl_sync(0xffffffffu, at, 31) + (unsigned)(x - n);
     float* out = lists + z * room;
-    for (int i = lane; i < n; i += 32)
-      if ((long long)at + i < room) out[at + i] = stage[warp][i];
-    __syncwarp();
+    for (int i = 0; i < n; ++i)
+      if ((long long)at + i < room) out[at + i] = stage[warp][32 * i + lane];
   }
 }
 
@@ -739,7 +763,7 @@ __global__ void __launch_bounds__(flag::kThreads, 1)
     const float ma = v1, mb = v2;
     __syncthreads();
     plane_bracket<20>(src, plane, [=](float x) { return abs_dev(x, ma, mb, even); }, KeyOfDev{}, &S, &lo, &hi);
-    if (threadIdx.x == 0) ch[z] = Chan{fmaxf(lo, 0.0f), hi, c.finite, 0u, 0u, v1, v2, even ? 1 : 0};
+    if (threadIdx.x == 0) ch[z] = Chan{fmaxf(lo, 0.0f), hi, c.finite, 0u, 0u, ma, mb, deviation_of(ma, mb)};
   }
 }
 
@@ -828,25 +852,24 @@ __global__ void __launch_bounds__(flag::kPixThreads, 2) k_pix_noise(const float*
       const unsigned r1 = (nf - 1u) / 2u;
       const bool even = (nf & 1u) == 0u;
       float ma, mb, a1, a2;
-      warp_select(col, nz, [](float v) { return v; }, mn, mx, r1, even, counts, list, &ma, &mb);
-      PixDev dev;
-      const float ha = -0.5f * ma, hb = -0.5f * mb;
-      dev.h = ma == mb ? -ma : __fadd_rn(ha, hb);
-      const float bb = __fsub_rn(dev.h, ha);
-      dev.l = ma == mb ? 0.0f : __fadd_rn(__fsub_rn(ha, __fsub_rn(dev.h, bb)), __fsub_rn(hb, bb));
+      const auto same = [](float v) { return v; };
+      warp_select(col, nz, same, [](float v, float*) { return v; }, mn, mx, r1, even, counts, list, &ma, &mb);
+      const Deviation dev = deviation_of(ma, mb);
       // |v - m| in place of v (an overflow stays the largest), unless the fit
       // needs the values
       const bool keep = mode == SC_NOISE_GAUSS;
       const auto clamped = [&](float v) { return v == v ? fminf(dev(v), FLT_MAX) : v; };
       const float top = fmaxf(clamped(mn), clamped(mx));
       if (keep) {
-        warp_select(col, nz, clamped, 0.0f, top, r1, even, counts, list, &a1, &a2);
+        warp_select(col, nz, clamped, [&](float v, float*) { return clamped(v); }, 0.0f, top, r1, even, counts, list, &a1,
+                    &a2);
       } else {
-        for_spectrum(col, nz, [&](float v, float* at) {
-          if (v == v) *at = clamped(v);
-        });
-        __syncwarp();
-        warp_select(col, nz, [](float v) { return v; }, 0.0f, top, r1, even, counts, list, &a1, &a2);
+        const auto replace = [&](float v, float* at) {
+          v = clamped(v);
+          if (v == v) *at = v;
+          return v;
+        };
+        warp_select(col, nz, same, replace, 0.0f, top, r1, even, counts, list, &a1, &a2);
       }
       const double mad = even ? 0.5 * ((double)a1 + (double)a2) : (double)a1;
       double sigma = kMadToSigma * mad;
