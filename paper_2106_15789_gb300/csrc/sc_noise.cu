@@ -429,7 +429,7 @@ __device__ __forceinline__ unsigned int last_true(unsigned int lo, unsigned int 
 // Latency-bound: one block with the plan proper on one thread took 40 us a
 // measurement whatever the cube's size (two bisections of 31 dependent steps
 // in float64, and 64 table cells a thread); with the bisections as 33-ary
-// searches by two warps and the table spread over eight SMs it takes 15 us.
+// searches by two warps and the table spread over eight SMs it takes 14 us.
 constexpr int kPlanCluster = 8;
 constexpr int kPlanThreads = 1024;
 __global__ void __cluster_dims__(kPlanCluster, 1, 1) __launch_bounds__(kPlanThreads)
@@ -447,9 +447,17 @@ __global__ void __cluster_dims__(kPlanCluster, 1, 1) __launch_bounds__(kPlanThre
   const int tid = threadIdx.x, warp = tid >> 5;
   const BinCfg cfg = win ? st->win : kFullRange;
   if (rank == 0) {
-    for (int b = tid; b < kNumBins; b += kPlanThreads) {
-      cum[b] = hist[b];
-      hist[b] = 0ull;
+    constexpr int kLoads = (kNumBins + kPlanThreads - 1) / kPlanThreads;
+    unsigned long long h[kLoads];  // all in flight together
+#pragma unroll
+    for (int j = 0; j < kLoads; ++j) h[j] = j * kPlanThreads + tid < kNumBins ? hist[j * kPlanThreads + tid] : 0ull;
+#pragma unroll
+    for (int j = 0; j < kLoads; ++j) {
+      const int b = j * kPlanThreads + tid;
+      if (b < kNumBins) {
+        cum[b] = h[j];
+        hist[b] = 0ull;
+      }
     }
     if (tid == 0) {
       s_bins[0] = s_bins[1] = 0;
@@ -522,7 +530,9 @@ __global__ void __cluster_dims__(kPlanCluster, 1, 1) __launch_bounds__(kPlanThre
                        force_flags);
   }
   cl.sync();
-  if (rank != 0 && tid == 0) s_plan = *cl.map_shared_rank(&s_plan, 0);
+  static_assert(sizeof(NoisePlan) % 4 == 0 && sizeof(NoisePlan) / 4 <= kPlanThreads, "a word per thread");
+  if (rank != 0 && tid < (int)(sizeof(NoisePlan) / 4))
+    reinterpret_cast<unsigned int*>(&s_plan)[tid] = reinterpret_cast<unsigned int*>(cl.map_shared_rank(&s_plan, 0))[tid];
   cl.sync();  // every copy is taken (a block's shared memory stays until its readers are done)
   const int t = rank * kPlanThreads + tid, nt = kPlanCluster * kPlanThreads;
   if (s_plan.flags & (PLAN_MED_FULL | PLAN_MAD_FULL)) {

@@ -133,7 +133,8 @@ __device__ __noinline__ bool select_rank(int nc, Task t, const AbsDev d, Smem* S
   const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const unsigned first = (unsigned)me * kThreads + tid, stride = (unsigned)nc * kThreads;
   for (unsigned i = tid; i < kBins; i += kThreads) S->hist[0][i] = S->hist[1][i] = 0u;
-  for (unsigned i = tid; i < kBins / 2; i += kThreads) S->red[0][i] = S->red[1][i] = 0u;
+  if (nc > 1)
+    for (unsigned i = tid; i < kBins / 2; i += kThreads) S->red[0][i] = S->red[1][i] = 0u;
   if (tid < 2u) S->below[tid] = 0u;
   __syncthreads();
   const unsigned share = kBins / nc;  // digits whose cluster-wide counts this block adds up
@@ -212,7 +213,8 @@ __device__ __noinline__ bool select_rank(int nc, Task t, const AbsDev d, Smem* S
     }
     // the other buffers for the next round (their readers are past a barrier)
     for (unsigned i = tid; i < kBins; i += kThreads) S->hist[par ^ 1][i] = 0u;
-    for (unsigned i = tid; i < kBins / 2; i += kThreads) S->red[par ^ 1][i] = 0u;
+    if (nc > 1)
+      for (unsigned i = tid; i < kBins / 2; i += kThreads) S->red[par ^ 1][i] = 0u;
     if (tid == 0u) S->below[par ^ 1] = 0u;
     __syncthreads();
     if (S->found == 0u) {
