@@ -100,3 +100,19 @@ def test_std(kind, n):
         got = ctx.noise(d, "std")
     # one float32 rounding of the result; the sums are good to 2^-40
     assert abs(got - want) <= 2.0**-24 * 1.01 * abs(want), (got, want)
+
+
+@pytest.mark.parametrize("shapes", [[(40, 230, 230)] * 3, [(40, 230, 230), (9, 250, 251), (64, 256, 256)]])
+def test_full_selection_passes_on_lanes(shapes):
+    """Forced full passes of cubes side by side (a launch per pass) and of one
+    cube alone (all passes in one launch) give the listed selection's run."""
+    g = torch.Generator(device="cuda").manual_seed(4)
+    cubes = [torch.randn(s, generator=g, device="cuda") for s in shapes]
+    kernels = [(0.0, 0), (3.0, 3)]
+    with Context(0, max(c.numel() for c in cubes)) as ctx:
+        masks, sig, sig0 = ctx.run_batch(cubes, kernels, 3.5, flags=sc.SC_FLAG_NO_FAST_SELECT)
+        for i, c in enumerate(cubes):
+            for flags in (0, sc.SC_FLAG_NO_FAST_SELECT):
+                m, s, s0 = ctx.run(c, kernels, 3.5, flags=flags)
+                assert list(s) == list(sig[i]) and s0 == sig0[i]
+                assert torch.equal(m, masks[i])
