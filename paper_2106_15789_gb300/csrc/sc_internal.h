@@ -355,7 +355,7 @@ cudaError_t launch_pass2(const float* src, long long n, uint32_t* mbits, DevStat
 // launch_select_full (which does nothing otherwise; alone: no other stream of
 // the context's lanes is at work).
 constexpr long long kSelectAllMax = 1LL << 21;
-constexpr long long kSelectGridMin = 1LL << 26;
+constexpr long long kSelectGridMin = 1LL << 25;
 cudaError_t launch_select_lists(DevState* st, const float* src, long long n, Lists L, int pair, int sms,
                                 cudaStream_t s, int* launches);
 void init_select_attrs();

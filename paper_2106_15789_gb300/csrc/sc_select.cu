@@ -574,10 +574,13 @@ void init_select_attrs() { cudaFuncSetAttribute(k_select, cudaFuncAttributeNonPo
 
 // One cluster: of 8 blocks up to kSelectAllMax values, of 16 above (the MAD's
 // list of a 217 x 331 x 509 cube, 0.25 M values, takes 37 us then, 50 with 8).
-// Arrays of more than kSelectGridMin values (a list of about 0.5 M) take the
-// MAD's first round by all SMs: 46 us for the four launches on 360 x 360 x
-// 1464 voxels against 73 for one cluster of 16, and 66 against 304 on 1200 x
-// 1200 x 1024.
+// Arrays of more than kSelectGridMin values take the MAD's first round by all
+// SMs. The four launches start before one another's ends, so the line lies
+// where they win on a whole run: 12 pairs on 217 x 331 x 509 voxels (36.6 M)
+// 3.64 ms against 3.70 with one cluster, 20 pairs on 256 x 312 x 640 (51 M)
+// 7.60 against 7.84; a line at 2^24 gave the same. On 360 x 360 x 1464 voxels
+// the launches take 46 us of a measurement against 73, on 1200 x 1200 x 1024
+// 66 against 304.
 cudaError_t launch_select_lists(DevState* st, const float* src, long long n, Lists L, int pair, int sms,
                                 cudaStream_t s, int* launches) {
   const int all = n <= kSelectAllMax ? 1 : 0;

@@ -11,7 +11,7 @@ from paper_2106_15789_gb300 import Context, sc
 pytestmark = pytest.mark.gpu
 
 ALL_MAX = 1 << 21  # kSelectAllMax
-GRID_MIN = 1 << 26  # kSelectGridMin
+GRID_MIN = 1 << 25  # kSelectGridMin
 
 
 def _data(kind: str, n: int) -> np.ndarray:
