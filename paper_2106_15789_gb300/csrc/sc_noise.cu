@@ -562,10 +562,13 @@ cudaError_t launch_plan(DevState* st, unsigned long long* hist, int win, const f
 // undecided voxels are staged per warp) and full columns. Columns and stages
 // are flushed with one atomic each.
 //
-// What bounds it: instruction issue until the MAD candidates took no votes (22
-// instructions a value with a vote per 32 values and 20 % of the groups in the
-// listing path: 1.10 ms on 1200 x 1200 x 1024 values); now 1.07 ms, the read
-// alone 0.88 at the measured HBM rate.
+// What bounds it: the shared-memory pipe (71 % busy, two of three wavefronts
+// bank conflicts of the lookups) and issue (60 %, 17 instructions a value). With
+// a vote per 32 values and the 20 % of the groups that hold a MAD candidate in
+// the listing path it was issue alone (22.7): 1200 x 1200 x 1024 values took
+// 1.10 ms, now 1.07; the read alone is 0.88 at the measured HBM rate. More loads
+// in flight (a cp.async ring in shared memory) cost that pipe more than they
+// gave: 1.27.
 constexpr int kP2Threads = 512;
 constexpr int kP2Warps = kP2Threads / 32;
 constexpr int kP2Unroll = 2;                 // chunks a warp classifies per iteration (the next ones load meanwhile)
