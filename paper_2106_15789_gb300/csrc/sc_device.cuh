@@ -173,4 +173,10 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
   return v;
 }
 
+// Bit i: byte i of x is not 0.
+__device__ __forceinline__ unsigned nonzero_bits(unsigned x) {
+  const unsigned b = ((((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | x) >> 7) & 0x01010101u;
+  return (b * 0x01020408u) >> 24 & 0xfu;
+}
+
 }  // namespace sc

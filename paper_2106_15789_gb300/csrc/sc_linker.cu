@@ -114,11 +114,6 @@ __device__ __forceinline__ int run_length(const unsigned* __restrict__ bits, lon
   }
 }
 
-__device__ __forceinline__ unsigned nonzero_bits(unsigned x) {  // bit i: byte i of x is not 0
-  const unsigned b = ((((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | x) >> 7) & 0x01010101u;
-  return (b * 0x01020408u) >> 24 & 0xfu;
-}
-
 }  // namespace link
 
 using link::Geo;
