@@ -77,59 +77,76 @@ __device__ __forceinline__ int for_buckets(long long z, int y, int x, const Shar
 // the voxel's cube value (high 32 bits) and its place (hy << 8 | hx) in the
 // bucket's halo'd tile (low 16 bits).
 //
-// A warp takes 1,024 voxels, a mask word a lane, writes the places of their
-// set bits to shared memory and then works through them with all 32 lanes;
-// lanes that add to the same bucket do so with one atomic. Masked voxels come
-// in clusters, so what bounds it is how they spread over the lanes: with a
+// A warp takes 4,096 voxels, 16 bytes of each mask a lane (the next ones load
+// meanwhile), writes the places of their set bits to shared memory and then
+// works through them with all 32 lanes; lanes that add to the same bucket do
+// so with one atomic. Masked voxels come in clusters, so what bounds it is how
+// they spread over the lanes; single ones are gathered from many words. With a
 // thread per 128 voxels, following its bits one by one, the count and the fill
-// took 160 us a pair on 360 x 360 x 1464 voxels (1.6 % of them masked);
-// now 79 us.
+// took 160 us a pair on 360 x 360 x 1464 voxels (1.6 % of them masked) and 332
+// on 1200 x 1200 x 1024; with a word a lane and 1,024 voxels a warp 79 and
+// 413; now 52 and 227.
 constexpr int kListThreads = 256;
-constexpr int kListRun = 1024;  // voxels a warp works on at a time
-constexpr int kListAhead = 4;   // runs whose words are loaded together
+constexpr int kListRun = 4096;    // voxels a warp works on at a time
+constexpr int kListStage = 1024;  // places staged at a time
 template <bool FILL>
 __global__ void __launch_bounds__(kListThreads) k_share_list(const uint32_t* __restrict__ mbits,
                                                              const float* __restrict__ C, Half16 h16, long long n,
                                                              long long nx, long long ny, ShareArgs sh, int R) {
-  __shared__ unsigned short s_off[kListThreads / 32][kListRun];
+  __shared__ unsigned short s_off[kListThreads / 32][kListStage];
   if (FILL) chain_begin();
   else chain_open();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lanes_below = (1u << lane) - 1u;
-  const long long nwords = (n + 31) / 32, nrun = (nwords + 31) / 32;
+  const long long nwords = (n + 31) / 32, nrun = (nwords + 127) / 128;
   const long long plane = nx * ny;
   const bool write = FILL && sh.ss->overflow == 0u;
-  const long long step = (long long)gridDim.x * (kListThreads / 32) * kListAhead;
-  for (long long run0 = ((long long)blockIdx.x * (kListThreads / 32) + warp) * kListAhead; run0 < nrun; run0 += step) {
-    unsigned words[kListAhead];
+  const uint4* const m4 = reinterpret_cast<const uint4*>(mbits);  // (both masks carry padding words)
+  const uint4* const s4 = reinterpret_cast<const uint4*>(sh.msnap);
+  const long long step = (long long)gridDim.x * (kListThreads / 32);
+  const auto fetch = [&](long long run, uint4* m, uint4* t) {
+    const long long q = run * 32 + lane;
+    *m = *t = make_uint4(0u, 0u, 0u, 0u);
+    if (run < nrun && 4 * q < nwords) *m = __ldg(m4 + q), *t = __ldg(s4 + q);
+  };
+  long long run = (long long)blockIdx.x * (kListThreads / 32) + warp;
+  uint4 m, t;
+  fetch(run, &m, &t);
+  for (; run < nrun; run += step) {
+    unsigned d[4] = {m.x & ~t.x, m.y & ~t.y, m.z & ~t.z, m.w & ~t.w};
+    fetch(run + step, &m, &t);
+    if (run == nrun - 1) {  // nothing past the cube's last voxel
 #pragma unroll
-    for (int k = 0; k < kListAhead; ++k) {
-      const long long w = (run0 + k) * 32 + lane;
-      words[k] = w < nwords ? __ldg(mbits + w) & ~__ldg(sh.msnap + w) : 0u;
-      if (w == nwords - 1 && (n & 31)) words[k] &= (1u << (n & 31)) - 1u;
+      for (int k = 0; k < 4; ++k) {
+        const long long left = n - ((run * 32 + lane) * 4 + k) * 32;
+        if (left < 32) d[k] &= left > 0 ? (1u << left) - 1u : 0u;
+      }
     }
+    const int all = __popc(d[0]) + __popc(d[1]) + __popc(d[2]) + __popc(d[3]);
+    const int sum = __reduce_add_sync(0xffffffffu, all);
+    if (sum == 0) continue;
+    // coordinates of the run's first voxel
+    const long long v0 = run * kListRun, z0 = v0 / plane, rem = v0 - z0 * plane;
+    const int y0 = (int)(rem / nx), x0 = (int)(rem - (long long)y0 * nx);
+    // all of it at once where there is room, else a word of every lane at a time
+    const int parts = sum <= kListStage ? 1 : 4;
 #pragma unroll 1
-    for (int k = 0; k < kListAhead; ++k) {
-      const long long run = run0 + k;
-      unsigned d = words[0];
-      words[0] = words[1], words[1] = words[2], words[2] = words[3];
-      if (!__any_sync(0xffffffffu, d != 0u)) continue;
-      int x = __popc(d);
-      const int own = x;
+    for (int part = 0; part < parts; ++part) {
+      const int own = parts == 1 ? all : __popc(part == 0 ? d[0] : part == 1 ? d[1] : part == 2 ? d[2] : d[3]);
+      int x = own;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
       }
       const int total = __shfl_sync(0xffffffffu, x, 31);
-      for (int at = x - own; d; ++at) {
-        s_off[warp][at] = (unsigned short)(32 * lane + __ffs(d) - 1);
-        d &= d - 1u;
+      int at = x - own;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        unsigned w = parts == 1 || part == k ? d[k] : 0u;
+        for (; w; w &= w - 1u) s_off[warp][at++] = (unsigned short)(128 * lane + 32 * k + __ffs(w) - 1);
       }
       __syncwarp();
-      // coordinates of the run's first voxel
-      const long long v0 = run * kListRun, z0 = v0 / plane, rem = v0 - z0 * plane;
-      const int y0 = (int)(rem / nx), x0 = (int)(rem - (long long)y0 * nx);
       for (int e0 = 0; e0 < total; e0 += 32) {
         const bool act = e0 + lane < total;
         const int off = act ? s_off[warp][e0 + lane] : 0;
@@ -169,7 +186,7 @@ __global__ void __launch_bounds__(kListThreads) k_share_list(const uint32_t* __r
           }
         }
       }
-      __syncwarp();  // the places are read before the next run's are written
+      __syncwarp();  // the places are read before the next ones are written
     }
   }
 }
@@ -816,7 +833,7 @@ cudaError_t launch_share_prep(const SmoothArgs& a, const ShareArgs& sh, int sms,
   const int R = share_R(a.pd);  // the reach the shared pass decodes its entries with
   const long long m = sh.n_buckets + 1;
   const long long nblk = (m + kScanChunk - 1) / kScanChunk;
-  const long long per = (long long)kListRun * kListAhead * (kListThreads / 32), want = (n + per - 1) / per;
+  const long long per = (long long)kListRun * (kListThreads / 32), want = (n + per - 1) / per;
   const unsigned list_grid = (unsigned)(want < 8LL * sms ? want : 8LL * sms);
   k_share_list<false><<<list_grid, kListThreads, 0, s>>>(a.mbits, a.C, a.h16, n, a.nx, a.ny, sh, R);
   cudaError_t e = cudaGetLastError();
