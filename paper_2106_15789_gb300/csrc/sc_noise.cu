@@ -566,14 +566,16 @@ cudaError_t launch_plan(DevState* st, unsigned long long* hist, int win, const f
 // bank conflicts of the lookups) and issue (60 %, 17 instructions a value). With
 // a vote per 32 values and the 20 % of the groups that hold a MAD candidate in
 // the listing path it was issue alone (22.7): 1200 x 1200 x 1024 values took
-// 1.10 ms, now 1.07; the read alone is 0.88 at the measured HBM rate. More loads
+// 1.10 ms, now 1.06; the read alone is 0.88 at the measured HBM rate. More loads
 // in flight (a cp.async ring in shared memory) cost that pipe more than they
-// gave: 1.27.
+// gave: 1.27. The columns take what two blocks an SM leave: 8 values a lane
+// instead of 11 were flushed more often and cost 0.06 ms a pair where the noise
+// varies by 30 % from channel to channel (more candidates).
 constexpr int kP2Threads = 512;
 constexpr int kP2Warps = kP2Threads / 32;
 constexpr int kP2Unroll = 2;                 // chunks a warp classifies per iteration (the next ones load meanwhile)
-constexpr int kP2Col = 8;                    // a lane's MAD candidates; a chunk adds at most 4
-constexpr int kP2FlushAt = 32;               // flush a list holding more than this after a chunk
+constexpr int kP2Col = 11;                   // a lane's MAD candidates; a chunk adds at most 4
+constexpr int kP2FlushAt = 8;                // flush a list holding more than this after a chunk
 constexpr int kP2Stage = kP2FlushAt + 128;   // one chunk adds at most 128 entries per list
 constexpr size_t kP2Smem = kClsCells + sizeof(float) * kP2Col * kP2Threads +
                            (size_t)kP2Warps * kP2Stage * (sizeof(float) + sizeof(unsigned long long));
