@@ -191,3 +191,18 @@ def test_sampled_gaussian_pairs_shared(ctx, fwhm):
         assert abs(a - b) <= 1e-6 * b, (k, a, b)
     for p in map(tuple, np.argwhere(m != m_ref)):
         assert any(abs(abs(s[p]) / sk - T) < BAND for s, sk in zip(ss, s_ref)), p
+
+
+@pytest.mark.parametrize("shape", [(7, 9, 11), (64, 64, 64), (33, 65, 67), (40, 96, 104)])
+@pytest.mark.parametrize("t", [0.3, 0.6, 2.0])
+def test_correction_lists_at_every_density(ctx, shape, t):
+    """Lists whose runs of 4,096 voxels hold more set bits than are staged at a
+    time, about as many, and few; cubes below one run and with a ragged end."""
+    nz, ny, nx = shape
+    cube = np.random.default_rng(nx).standard_normal(shape).astype(np.float32)
+    cube[:, : ny // 8, :3] = np.nan
+    ctx.set_share_limit(1 << 40)
+    try:
+        check_shared_equals_full(ctx, torch.from_numpy(cube), [(3.0, 0), (3.0, 3), (3.0, 15)], t=t)
+    finally:
+        ctx.set_share_limit(0)
