@@ -421,6 +421,24 @@ cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k
 size_t chan_scratch_bytes(const long long dims[3], int mode);
 
 constexpr int kLinkMaxRadius = 32;  // merging radii in voxels
+// A linker call's totals (device memory, cleared before its kernels) and the
+// room of its buffers. A total counts only where those before it fit: the
+// kernels that would write it return otherwise.
+enum LinkScan { LINK_SCAN_LEN, LINK_SCAN_RUNS, LINK_SCAN_COMPS };
+struct LinkTotals {
+  int* n;  // [0] runs, [1] components, [2] kept
+  long long max_runs, max_comp;
+  __host__ __device__ bool runs_fit() const { return n[0] >= 0 && n[0] <= max_runs; }
+  __host__ __device__ bool all_fit() const { return runs_fit() && n[1] >= 0 && n[1] <= max_comp; }
+  // Entries of a scan: len, or one per `per` runs, or one per component; -1
+  // where the total does not fit or was not counted.
+  __host__ __device__ long long scan_length(int of, int per, long long len) const {
+    if (of == LINK_SCAN_RUNS) return runs_fit() ? ((long long)n[0] + per - 1) / per : -1;
+    if (of == LINK_SCAN_COMPS) return all_fit() ? n[1] : -1;
+    return len;
+  }
+};
+
 // Linker. Scratch: bits (link_bits_bytes), runs and comp for at most max_runs
 // runs and max_comp components. totals[3] (device): runs, components, kept
 // detections; where either does not fit, nothing after it is meant (the caller

@@ -49,14 +49,6 @@ struct Geo {
   int rxy, rz;
 };
 
-// Device totals, and the sizes of the buffers.
-struct Totals {
-  int* n;                    // [0] runs, [1] components, [2] kept
-  long long max_runs, max_comp;
-  __device__ __forceinline__ bool runs_fit() const { return n[0] <= max_runs; }
-  __device__ __forceinline__ bool all_fit() const { return n[0] <= max_runs && n[1] <= max_comp; }
-};
-
 // The mask's runs: bits, run starts, and the runs before each word and chunk.
 struct Runs {
   unsigned* bits;
@@ -118,7 +110,7 @@ __device__ __forceinline__ int run_length(const unsigned* __restrict__ bits, lon
 
 using link::Geo;
 using link::Runs;
-using link::Totals;
+using Totals = LinkTotals;
 
 // A block per chunk, a mask word (32 voxels) per thread. A run starts at a set
 // voxel whose predecessor is not set or lies in another row.
@@ -168,18 +160,15 @@ __global__ void __launch_bounds__(link::kThreads) k_lk_pack(const uint8_t* __res
 }
 
 // Exclusive scan of a[0 .. len) in place by one block of 1024 threads, eight
-// values a thread, the next eight loaded meanwhile; a[len] and *total (unless
-// null) receive the sum. With per > 0, len is ceil(*count / per), and nothing
-// happens where `most` counts do not fit.
-__global__ void __launch_bounds__(1024) k_scan_block(int* a, long long len, const int* count, int per, long long most,
-                                                     int* total) {
+// values a thread, the next eight loaded meanwhile; a[len] and *total receive
+// the sum. The length is t.scan_length(of, per, len): nothing happens where
+// the totals it comes from do not fit.
+__global__ void __launch_bounds__(1024) k_scan_block(int* a, long long len, Totals t, int of, int per, int* total) {
   __shared__ int part[32];
   constexpr int kPer = 8;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (per > 0) {
-    if (*count > most) return;
-    len = ((long long)*count + per - 1) / per;
-  }
+  len = t.scan_length(of, per, len);
+  if (len < 0) return;
   int carry = 0;
   int nx[kPer];
 #pragma unroll
@@ -213,7 +202,7 @@ __global__ void __launch_bounds__(1024) k_scan_block(int* a, long long len, cons
   }
   if (tid == 0) {
     a[len] = carry;
-    if (total) *total = carry;
+    *total = carry;
   }
 }
 
@@ -540,17 +529,20 @@ cudaError_t launch_link(const uint8_t* mask, const long long dims[3], int r_xy, 
   int *const ext = comp, *const kept = ext + 7 * max_comp, *const new_id = kept + 7 * max_comp;
   int* const keep = new_id + max_comp;
   const int flat_grid = (int)(flat < 8LL * sms ? flat : 8LL * sms);
+  // a total that a kernel leaves unwritten (what it counts did not fit) is 0
+  const cudaError_t e = cudaMemsetAsync(totals, 0, 3 * sizeof(int), s);
+  if (e != cudaSuccess) return e;
   k_lk_pack<<<(unsigned)chunks, link::kThreads, 0, s>>>(mask, g, R);
-  k_scan_block<<<1, 1024, 0, s>>>(R.chunk_off, chunks, nullptr, 0, 0, totals);
+  k_scan_block<<<1, 1024, 0, s>>>(R.chunk_off, chunks, t, LINK_SCAN_LEN, 1, totals);
   k_lk_init<<<grid_for(max_runs, sms, 256), 256, 0, s>>>(parent, t);
   k_lk_union<<<(unsigned)chunks, link::kThreads, 0, s>>>(g, R, parent, t);
   k_lk_flatten<<<flat_grid, 1024, 0, s>>>(parent, counts, t);
-  k_scan_block<<<1, 1024, 0, s>>>(counts, 0, totals, link::kFlat, max_runs, totals + 1);
+  k_scan_block<<<1, 1024, 0, s>>>(counts, 0, t, LINK_SCAN_RUNS, link::kFlat, totals + 1);
   k_cc_ext_init<<<grid_for(max_comp, sms, 256), 256, 0, s>>>(ext, t);
   k_lk_number<<<flat_grid, 1024, 0, s>>>(parent, counts, t);
   k_lk_extents<<<(unsigned)chunks, link::kThreads, 0, s>>>(g, R, parent, run_id, ext, t);
   k_cc_keep<<<grid_for(max_comp, sms, 256), 256, 0, s>>>(ext, t, min_xy, min_z, max_xy, max_z, keep, new_id);
-  k_scan_block<<<1, 1024, 0, s>>>(keep, 0, totals + 1, 1, max_comp, totals + 2);
+  k_scan_block<<<1, 1024, 0, s>>>(keep, 0, t, LINK_SCAN_COMPS, 1, totals + 2);
   k_cc_compact<<<grid_for(max_comp, sms, 256), 256, 0, s>>>(ext, new_id, keep, t, kept, new_id);
   k_lk_expand<<<grid_for((g.n + 3) / 4, sms, 256), 256, 0, s>>>(g, R, run_id, new_id, lab, t);
   *launches = 13;

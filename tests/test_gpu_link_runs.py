@@ -44,3 +44,17 @@ def test_room_grows_and_is_kept(r_xy, r_z, density):
         _check(ctx, big, r_xy, r_z)
         _check(ctx, big[:40], r_xy, r_z, min_xy=2, min_z=1)
         _check(ctx, np.zeros((4, 5, 6), np.uint8), 1, 1)
+
+
+def test_restart_in_recycled_memory():
+    """A context whose buffer holds another owner's bytes (all ones: totals of
+    -1) and whose first mask needs more room than the first buffer has."""
+    rng = np.random.default_rng(6)
+    m = (rng.random((96, 128, 160)) < 0.3).astype(np.uint8)
+    for _ in range(2):
+        room = [torch.full((1 << 24,), -1, dtype=torch.int32, device="cuda") for _ in range(4)]
+        torch.cuda.synchronize()
+        del room
+        torch.cuda.empty_cache()  # given back to the driver, for the context to take
+        with Context(0, 1 << 16) as ctx:
+            _check(ctx, m, 1, 1, min_xy=2)
