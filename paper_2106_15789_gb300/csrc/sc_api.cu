@@ -90,7 +90,6 @@ struct sc_ctx {
   // sc_run_batch: extra workspaces ("lanes", full contexts of their own) that
   // run other cubes of the batch concurrently on their own streams
   std::vector<sc_ctx*> lanes;
-  bool among_lanes = false;  // other lanes run beside this one (a batch, or stream jobs)
   std::vector<cudaStream_t> lane_streams;
   std::vector<cudaEvent_t> lane_done;
   cudaEvent_t fork = nullptr;
@@ -272,8 +271,8 @@ int measure(sc_ctx* c, const float* src, long long n, int win, float t, int clip
       CK(launch_select_lists(c->st, src, n, c->L, pair, c->sms, s, &launched));
       c->stats.launches += 1 + launched;
       if (n > kSelectAllMax) {
-        CK(launch_select_full(c->st, pair, !c->among_lanes, c->sms, s, &launched));
-        c->stats.launches += launched;
+        CK(launch_select_full(c->st, pair, c->sms, s));
+        c->stats.launches += kSelectFullLaunches;
       }
     }
   }
@@ -853,7 +852,6 @@ int ensure_lanes(sc_ctx* c) {
       cudaGetLastError();
       return SC_ERR_CUDA;
     }
-    if (lc) lc->among_lanes = true;
     c->lanes.push_back(l == 0 ? c : lc);
     c->lane_streams.push_back(ls);
     c->lane_done.push_back(ev);
@@ -953,10 +951,8 @@ int sc_run_batch(sc_ctx* c, int n_cubes, const float* const* cubes, const int64_
       const int l = i % n_lanes;
       sc_ctx* lc = c->lanes[l];
       cudaStream_t ls = c->lane_streams[l];
-      lc->among_lanes = true;
       const int rc = run_device(lc, cubes[i], dims + 3 * i, kernels, n_kernels, threshold, noise_mode, replacement,
                                 masks[i], rflags, ls);
-      c->among_lanes = false;
       if (rc) return rc;
       CK(cudaMemcpyAsync(&res[i], lc->st, 3 * sizeof(unsigned int), cudaMemcpyDeviceToDevice, ls));
       CK(cudaMemcpyAsync(res[i].sigma, lc->st->sigma, sizeof(float) * n_kernels, cudaMemcpyDeviceToDevice, ls));

@@ -352,16 +352,16 @@ cudaError_t launch_pass2(const float* src, long long n, uint32_t* mbits, DevStat
 // Median and MAD (DevState::m, mad, sigma_cur, sigma[pair] if pair >= 0) from
 // the candidate lists (*launches: kernels launched). Arrays of more than
 // kSelectAllMax values whose plan asks for full passes are left to
-// launch_select_full (which does nothing otherwise; alone: no other stream of
-// the context's lanes is at work).
+// launch_select_full (kSelectFullLaunches kernels, which do nothing otherwise).
 constexpr long long kSelectAllMax = 1LL << 21;
 constexpr long long kSelectGridMin = 1LL << 25;
+constexpr int kSelectFullLaunches = 8;
 cudaError_t launch_select_lists(DevState* st, const float* src, long long n, Lists L, int pair, int sms,
                                 cudaStream_t s, int* launches);
 void init_select_attrs();
 // stats[0] = median, stats[1] = 1.4826 MAD of the finite values of x[0 .. n) (NaN if none).
 cudaError_t launch_array_stats(const float* x, long long n, double* stats, cudaStream_t s);
-cudaError_t launch_select_full(DevState* st, int pair, bool alone, int sms, cudaStream_t s, int* launched);
+cudaError_t launch_select_full(DevState* st, int pair, int sms, cudaStream_t s);
 // The clip of the voxels that the candidate pass left undecided, or of all by a full pass.
 cudaError_t launch_clip(const float* src, long long n, uint32_t* mbits, DevState* st, Lists L, int sms,
                         cudaStream_t s);

@@ -1018,7 +1018,6 @@ __device__ void sel_result(DevState* st, SelJob* J, int which, int pair) {
   }
 }
 
-// The passes by a launch each, and all in one cooperative launch.
 __global__ void __launch_bounds__(256) k_sel_round(DevState* st, int which, int r) {
   chain_begin();
   if (sel_by_full_passes(st->plan)) sel_round(st, which, r);
@@ -1029,42 +1028,13 @@ __global__ void __launch_bounds__(256) k_sel_succ(DevState* st, int which, int p
   if (sel_by_full_passes(st->plan)) sel_succ(st, which, pair);
 }
 
-__global__ void __launch_bounds__(256) k_sel_full(DevState* st, int pair) {
-  if (!sel_by_full_passes(st->plan)) return;
-  const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
-#pragma unroll 1
-  for (int which = 0; which < 2; ++which) {
-#pragma unroll 1
-    for (int r = 0; r < 3; ++r) {
-      sel_round(st, which, r);
-      grid.sync();
-    }
-    sel_succ(st, which, which ? pair : -1);
-    grid.sync();
-  }
-}
-
-// Mostly there is nothing to do, and eight launches that return at once cost
-// about 1 us each: 12 pairs on 217 x 331 x 509 voxels take 3.75 ms with them,
-// 3.64 with the one. But a cooperative grid waits until all of it fits, and
-// next to the kernels of other lanes it waits long (12 cubes on eight lanes:
-// 27.9 ms with the eight launches, 30.6 with the one).
-cudaError_t launch_select_full(DevState* st, int pair, bool alone, int sms, cudaStream_t s, int* launched) {
+// Mostly there is nothing to do, and the eight launches return at once, about
+// 1 us each. One cooperative launch in their place saved most of that (12 pairs
+// on 217 x 331 x 509 voxels: 3.64 ms against 3.75), but a cooperative grid
+// starts only when all of it fits: beside other lanes, another context or a
+// kernel of the program that keeps an SM it waited for them to end.
+cudaError_t launch_select_full(DevState* st, int pair, int sms, cudaStream_t s) {
   const unsigned grid = 2u * (unsigned)sms;
-  if (alone) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(256);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1] = {};
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    *launched = 1;
-    return cudaLaunchKernelEx(&cfg, k_sel_full, st, pair);
-  }
-  *launched = 8;
   cudaError_t e = cudaSuccess;
   for (int which = 0; which < 2 && e == cudaSuccess; ++which) {
     for (int r = 0; r < 3 && e == cudaSuccess; ++r) e = launch_chained(k_sel_round, grid, 256, 0, 0, s, st, which, r);

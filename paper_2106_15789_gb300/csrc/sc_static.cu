@@ -104,7 +104,7 @@ extern "C" int sc_noise_static(const float* data_dev, int64_t n, int noise_mode,
     CKS(launch_pass2(data_dev, n, nullptr, st, L, sms, s));
     int launched = 0;
     CKS(launch_select_lists(st, data_dev, n, L, SC_MAX_KERNELS, sms, s, &launched));
-    if (n > kSelectAllMax) CKS(launch_select_full(st, SC_MAX_KERNELS, true, sms, s, &launched));
+    if (n > kSelectAllMax) CKS(launch_select_full(st, SC_MAX_KERNELS, sms, s));
   }
   if (noise_mode == SC_NOISE_GAUSS) {
     unsigned long long* ghist = reinterpret_cast<unsigned long long*>(base + kOffGHist);

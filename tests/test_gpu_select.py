@@ -104,8 +104,8 @@ def test_std(kind, n):
 
 @pytest.mark.parametrize("shapes", [[(40, 230, 230)] * 3, [(40, 230, 230), (9, 250, 251), (64, 256, 256)]])
 def test_full_selection_passes_on_lanes(shapes):
-    """Forced full passes of cubes side by side (a launch per pass) and of one
-    cube alone (all passes in one launch) give the listed selection's run."""
+    """Forced full passes of cubes side by side and of one cube alone give the
+    listed selection's run."""
     g = torch.Generator(device="cuda").manual_seed(4)
     cubes = [torch.randn(s, generator=g, device="cuda") for s in shapes]
     kernels = [(0.0, 0), (3.0, 3)]
