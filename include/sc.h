@@ -47,7 +47,7 @@ extern "C" {
 
 /* ---- noise estimators (Sect. 4.1: robust RMS from the MAD) ------------ */
 #define SC_NOISE_MAD 0   /* 1.4826 * median(|S - median(S)|), exact medians */
-#define SC_NOISE_STD 1   /* sqrt(sum((S - mean)^2) / (n - 1)) */
+#define SC_NOISE_STD 1   /* sqrt(sum((S - mean)^2) / (n - 1)), summed to float64's precision */
 #define SC_NOISE_GAUSS 2 /* width of the least-squares Gaussian through a histogram of S (below) */
 
 /* SC_NOISE_GAUSS is the library's own definition (the paper names no such

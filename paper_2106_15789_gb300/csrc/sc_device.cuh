@@ -173,6 +173,15 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
   return v;
 }
 
+// x + y as the float nearest to it and what that leaves (Knuth's TwoSum): exact
+// unless the sum overflows.
+__device__ __forceinline__ float two_sum(float x, float y, float* err) {
+  const float s = __fadd_rn(x, y);
+  const float b = __fsub_rn(s, x);
+  *err = __fadd_rn(__fsub_rn(x, __fsub_rn(s, b)), __fsub_rn(y, b));
+  return s;
+}
+
 // Bit i: byte i of x is not 0.
 __device__ __forceinline__ unsigned nonzero_bits(unsigned x) {
   const unsigned b = ((((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | x) >> 7) & 0x01010101u;

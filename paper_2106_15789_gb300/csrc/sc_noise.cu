@@ -341,11 +341,11 @@ __device__ __noinline__ NoisePlan plan_of(DevState* st, const unsigned long long
     }
     double top = fmax(fabs(bin_lo_value(first, cfg)), fabs(bin_hi_value(last, cfg)));
     if (!isfinite(top)) top = 2.0 * (double)fmaxf(__uint_as_float(st->maxabs_bits), st->repl);  // (0: not measured)
-    // no scale for magnitudes up to 2^40 (and some above 2^-40): n squares stay
-    // below 2^128, and what underflows is too small to count
+    // no scale for magnitudes up to 2^40 (and some above 2^-20): n squares stay
+    // below 2^128, and what underflows (2^-150 a value) is 2^-77 of their sum
     int e = 128;
     if (top > 0.0 && isfinite(top)) frexp(top, &e);  // top < 2^e
-    e = e > -40 && e <= 40 ? 0 : (e > 128 ? 128 : (e < -126 ? -126 : e));
+    e = e > -20 && e <= 40 ? 0 : (e > 128 ? 128 : (e < -126 ? -126 : e));
     st->std_scale = ldexpf(1.0f, -e);
     // no shift where 0 lies well within the spread (a quarter of the values
     // beyond 8 times the median's magnitude, on either side of it)
@@ -1046,47 +1046,61 @@ cudaError_t launch_select_full(DevState* st, int pair, int sms, cudaStream_t s) 
 // ---------------------------------------------------------------------------
 // STD mode: sums of d = (x - K) 2^-e and of d^2 over the finite values, with K
 // in the median's bin and 2^e above all magnitudes (both from the histogram:
-// the squares of float32 data can overflow or underflow float32). The median
-// lies within one standard deviation of the mean, so K costs the variance
-// S2 - S1^2 / n a bit or two, unless its bin is much wider than the spread
-// (data on a large offset): then a second pass takes the mean as K.
+// the squares of float32 data can overflow or underflow float32). Where K is
+// so far from the mean that S2 - S1^2 / n would lose a bit (data on an offset
+// of many times their spread), a second pass takes the mean as K.
 //
-// Each thread keeps its sums as unevaluated pairs of floats: the difference,
-// the square and the additions are exact in pairs (TwoSum, and an FMA for the
-// product's error), and what is rounded is 2^-24 of the pairs' low parts. The
-// float64 conversions and FMAs of the earlier two passes bound them at 268 us
-// each on 256 x 250 x 600 voxels (the pipe is slow on this part); one pass
-// takes 44 us (a read at the measured HBM rate: 23).
-__device__ __forceinline__ void pair_add(float* s, float* c, float x, float rest) {
-  const float t = __fadd_rn(*s, x);
-  const float b = __fsub_rn(t, *s);
-  const float e = __fadd_rn(__fsub_rn(*s, __fsub_rn(t, b)), __fsub_rn(x, b));
-  *c = __fadd_rn(*c, __fadd_rn(e, rest));
-  *s = t;
+// Each thread keeps its sums as unevaluated triples of floats: the difference,
+// the square and the additions are exact in the first two parts (TwoSum, and an
+// FMA for a product's error), the third takes what those leave, 2^-48 of the
+// sum, rounded to 2^-24 of itself. So a thread's sums are good to float64's
+// last bit, and the noise is as near to the exact one as with float64 sums
+// about the mean in two passes (2^-50 either way at 10 to 400 M values; pairs
+// of floats gave 2^-44 to 2^-39). The conversions and FMAs of those bound them
+// at 268 us a pass on 256 x 250 x 600 voxels (the float64 pipe is slow on this
+// part); this pass takes 61 us (pairs: 44, a read at the measured HBM rate: 23).
+// a += x + y + low, y and low well below x.
+__device__ __forceinline__ void sum3_add(float (&a)[3], float x, float y, float low) {
+  float e, f, g;
+  a[0] = two_sum(a[0], x, &e);
+  a[1] = two_sum(a[1], e, &f);
+  a[1] = two_sum(a[1], y, &g);
+  a[2] = __fadd_rn(a[2], __fadd_rn(__fadd_rn(f, g), low));
+}
+__device__ __forceinline__ void sum3_add(float (&a)[3], float x) {
+  float e, f;
+  a[0] = two_sum(a[0], x, &e);
+  a[1] = two_sum(a[1], e, &f);
+  a[2] = __fadd_rn(a[2], f);
+}
+__device__ __forceinline__ double sum3_value(const float (&a)[3]) {
+  return (double)a[0] + ((double)a[1] + (double)a[2]);
 }
 
 // PLAIN: neither shift nor scale.
 template <bool PLAIN>
-__device__ __forceinline__ void std_add(float x, float scale, float shift, float (&s1)[2], float (&s2)[2], unsigned* n) {
+__device__ __forceinline__ void std_add(float x, float scale, float shift, float (&s1)[3], float (&s2)[3], unsigned* n) {
   if (!(fabsf(x) <= FLT_MAX)) return;  // NaN and Inf
-  float h = x, l = 0.0f;
-  if (!PLAIN) {
-    const float xs = __fmul_rn(x, scale);  // a power of two
-    h = __fsub_rn(xs, shift);
-    const float b = __fsub_rn(h, xs);
-    l = __fsub_rn(__fsub_rn(xs, __fsub_rn(h, b)), __fadd_rn(shift, b));
+  if (PLAIN) {
+    sum3_add(s1, x);
+    const float p = __fmul_rn(x, x);
+    sum3_add(s2, p, __fmaf_rn(x, x, -p), 0.0f);
+  } else {
+    float l;  // d = h + l
+    const float h = two_sum(__fmul_rn(x, scale), -shift, &l);  // (scale: a power of two)
+    sum3_add(s1, h, l, 0.0f);
+    // d^2 = h^2 + 2 h l + l^2, the first two as products and their errors
+    const float p = __fmul_rn(h, h), h2 = __fadd_rn(h, h), q = __fmul_rn(h2, l);
+    float re;
+    const float r = two_sum(__fmaf_rn(h, h, -p), q, &re);
+    sum3_add(s2, p, r, __fmaf_rn(l, l, __fadd_rn(re, __fmaf_rn(h2, l, -q))));
   }
-  pair_add(&s1[0], &s1[1], h, l);
-  const float p = __fmul_rn(h, h);
-  float e = __fmaf_rn(h, h, -p);
-  if (!PLAIN) e = __fmaf_rn(__fadd_rn(h, h), l, e);
-  pair_add(&s2[0], &s2[1], p, e);
   ++*n;
 }
 
 template <bool PLAIN>
 __device__ __forceinline__ void std_sums(const float* __restrict__ x, long long n, float scale, float shift,
-                                         float (&s1)[2], float (&s2)[2], unsigned* cnt) {
+                                         float (&s1)[3], float (&s2)[3], unsigned* cnt) {
   const long long t0 = (long long)blockIdx.x * 256 + threadIdx.x, stride = (long long)gridDim.x * 256;
   const long long nq = (reinterpret_cast<uintptr_t>(x) & 15u) == 0 ? n >> 2 : 0;
   for (long long q = t0; q < nq; q += 4 * stride) {
@@ -1116,11 +1130,11 @@ __global__ void __launch_bounds__(256) k_std_pass(const float* __restrict__ x, l
   chain_begin();
   if ((st->plan.flags & PLAN_EMPTY) || (second && !st->std_again)) return;
   const float scale = st->std_scale, shift = __fmul_rn(st->std_shift, scale);
-  float p1[2] = {0.0f, 0.0f}, p2[2] = {0.0f, 0.0f};
+  float p1[3] = {0.0f, 0.0f, 0.0f}, p2[3] = {0.0f, 0.0f, 0.0f};
   unsigned cnt = 0u;
   if (scale == 1.0f && shift == 0.0f) std_sums<true>(x, n, scale, shift, p1, p2, &cnt);
   else std_sums<false>(x, n, scale, shift, p1, p2, &cnt);
-  double s1 = (double)p1[0] + (double)p1[1], s2 = (double)p2[0] + (double)p2[1];
+  double s1 = sum3_value(p1), s2 = sum3_value(p2);
   for (int o = 16; o > 0; o >>= 1) {
     s1 += __shfl_xor_sync(0xffffffffu, s1, o);
     s2 += __shfl_xor_sync(0xffffffffu, s2, o);
@@ -1151,7 +1165,7 @@ __global__ void __launch_bounds__(256) k_std_pass(const float* __restrict__ x, l
   s1 = *(volatile double*)&st->sum;
   s2 = *(volatile double*)&st->sum2;
   const double var = s2 - s1 * s1 / c;
-  if (!second && c > 1.0 && !(var >= s2 * 0x1p-10)) {
+  if (!second && c > 1.0 && !(var >= 0.5 * s2)) {
     st->std_again = 1;
     st->std_shift = __double2float_rn((double)st->std_shift + s1 / c / (double)scale);  // the mean
     st->sum = st->sum2 = 0.0;

@@ -46,13 +46,6 @@ constexpr unsigned kNone = 0xffffffffu; // above every key of a finite value
 // Melquiond, "Emulation of FMA and correctly rounded sums", 2008). l == 0 (an
 // odd count, or equal middle values): one addition. Halving a subnormal may
 // round, so medians of tiny values take float64.
-__device__ __forceinline__ float two_sum(float x, float y, float* err) {
-  const float s = __fadd_rn(x, y);
-  const float b = __fsub_rn(s, x);
-  *err = __fadd_rn(__fsub_rn(x, __fsub_rn(s, b)), __fsub_rn(y, b));
-  return s;
-}
-
 __device__ __forceinline__ AbsDev abs_dev_of(float a, float b) {
   AbsDev d;
   d.m = a == b ? (double)a : 0.5 * ((double)a + (double)b);

@@ -98,7 +98,7 @@ def test_std(kind, n):
     want = float(np.sqrt(((v - v.mean()) ** 2).sum() / (v.size - 1))) if v.size > 1 else 0.0
     with Context(0, n + 1) as ctx:
         got = ctx.noise(d, "std")
-    # one float32 rounding of the result; the sums are good to 2^-40
+    # one float32 rounding of the result; the sums are good to 2^-47
     assert abs(got - want) <= 2.0**-24 * 1.01 * abs(want), (got, want)
 
 
