@@ -14,7 +14,10 @@ namespace sc {
 __device__ __forceinline__ void chain_open() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // First thing in a chained kernel: the same, then the wait for the end of the
 // kernel before it (which has itself waited for its own), its writes visible.
-// Nothing is read or written before it.
+// Nothing is read or written before it. The kernels of a chain are resident
+// together, so what one of them writes is no read-only data to those behind it:
+// they take it with plain loads or __ldcg, never with __ldg or through a
+// pointer that is both const and __restrict__.
 __device__ __forceinline__ void chain_begin() {
   chain_open();
   asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(kMadThreads) k_mad_compact(DevState* st, Lists
 #pragma unroll
     for (int u = 0; u < kMadUnroll; ++u) {
       const unsigned long long i = w0 + lane + u * stride;
-      k[u] = i < count ? __float_as_uint(__ldg(L.mad + i)) : kNone;
+      k[u] = i < count ? __float_as_uint(__ldcg(L.mad + i)) : kNone;
     }
 #pragma unroll
     for (int u = 0; u < kMadUnroll; ++u) {

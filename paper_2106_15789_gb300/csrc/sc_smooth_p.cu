@@ -175,12 +175,12 @@ __global__ void __launch_bounds__(kListThreads) k_share_list(const uint32_t* __r
           if (nb == 1 && lane == lead) slot = atomicSub(sh.cnt + only, (unsigned)__popc(peers)) - (unsigned)__popc(peers);
           slot = __shfl_sync(0xffffffffu, slot, lead) + (unsigned)__popc(peers & lanes_below);
           if (nb == 1) {
-            const unsigned long long idx = (unsigned long long)__ldg(sh.offs + only) + slot;
+            const unsigned long long idx = (unsigned long long)__ldcg(sh.offs + only) + slot;
             if (write && idx < sh.cap) sh.ent[idx] = cb | pos;
           } else if (nb > 1) {
             for_buckets(vz, vy, vx, sh, R, [&](long long bk, unsigned p) {
               const unsigned long long idx =
-                  (unsigned long long)__ldg(sh.offs + bk) + (atomicSub(sh.cnt + bk, 1u) - 1u);
+                  (unsigned long long)__ldcg(sh.offs + bk) + (atomicSub(sh.cnt + bk, 1u) - 1u);
               if (write && idx < sh.cap) sh.ent[idx] = cb | p;
             });
           }
@@ -193,8 +193,8 @@ __global__ void __launch_bounds__(kListThreads) k_share_list(const uint32_t* __r
 
 // Exclusive scan of m counts, in chunks of kScanChunk: the chunk's own scan
 // and its total.
-__global__ void __launch_bounds__(1024) k_share_scan1(const unsigned* __restrict__ cnt, unsigned* __restrict__ offs,
-                                                      unsigned long long* __restrict__ bsum, long long m) {
+__global__ void __launch_bounds__(1024) k_share_scan1(const unsigned* cnt, unsigned* offs, unsigned long long* bsum,
+                                                      long long m) {
   __shared__ unsigned wsum[32];
   chain_begin();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(1024) k_share_scan1(const unsigned* __restrict
   unsigned v[4], tot = 0;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    v[k] = base + k < m ? cnt[base + k] : 0u;
+    v[k] = base + k < m ? __ldcg(cnt + base + k) : 0u;
     tot += v[k];
   }
   unsigned inc = tot;  // inclusive scan over the warp
@@ -232,14 +232,13 @@ __global__ void __launch_bounds__(1024) k_share_scan1(const unsigned* __restrict
 
 // Adds the totals of the chunks before each chunk; the last chunk's block
 // records the grand total and whether it exceeds the list's capacity.
-__global__ void __launch_bounds__(1024) k_share_scan2(unsigned* __restrict__ offs,
-                                                      const unsigned long long* __restrict__ bsum, long long m,
+__global__ void __launch_bounds__(1024) k_share_scan2(unsigned* offs, const unsigned long long* bsum, long long m,
                                                       ShareState* ss, unsigned long long cap) {
   __shared__ unsigned long long red[32];
   chain_begin();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   unsigned long long p = 0;
-  for (long long i = t; i < blockIdx.x; i += 1024) p += bsum[i];
+  for (long long i = t; i < blockIdx.x; i += 1024) p += __ldcg(bsum + i);
   for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
   if (lane == 0) red[warp] = p;
   __syncthreads();
@@ -249,7 +248,7 @@ __global__ void __launch_bounds__(1024) k_share_scan2(unsigned* __restrict__ off
   for (int k = t; k < kScanChunk; k += 1024)
     if (base + k < m) offs[base + k] += (unsigned)pre;
   if (blockIdx.x == gridDim.x - 1 && t == 0) {
-    const unsigned long long total = pre + bsum[blockIdx.x];
+    const unsigned long long total = pre + __ldcg(bsum + blockIdx.x);
     ss->total = total;
     ss->overflow = total > cap ? 1u : 0u;
   }
