@@ -1318,11 +1318,16 @@ cudaError_t launch_fx_setup(DevState* st, float repl_value, const PairWeights& W
 // spread through the cube (all of them in a smaller cube): a window 32
 // octaves wide needs its scale only roughly, and the exact selection that
 // follows does not depend on it (a poorly placed window costs candidates,
-// never exactness). One block, bound by the latency of its loads: 65,536
-// values in four batches took 44 to 68 us a run, 8,192 in one take 10.
+// never exactness). Where hardly any of them is finite, up to seven further
+// samples are taken: of a cube that is blank but for one voxel in 8,000 the
+// first may hold none, and full selection passes would follow. One block,
+// bound by the latency of its loads: 65,536 values in four batches took 44 to
+// 68 us, 8,192 in one take 9 to 10 (21 on 360 x 360 x 1464 values and 78 on
+// 1200 x 1200 x 1024 in the first pass over a cube).
 constexpr int kWinThreads = 1024;
 constexpr long long kWinSample = 8192;
 constexpr int kWinPerThread = (int)(kWinSample / kWinThreads);
+constexpr int kWinRounds = 8, kWinEnough = 32;  // samples at most; threads that found a finite value
 __global__ void __launch_bounds__(kWinThreads) k_window_from_sample(const float* __restrict__ x, Half16 h,
                                                                     long long plane, long long n, DevState* st) {
   extern __shared__ unsigned int wh[];  // full-range histogram of the sample
@@ -1335,22 +1340,28 @@ __global__ void __launch_bounds__(kWinThreads) k_window_from_sample(const float*
   // m values, one from every step of the cube (all of a cube of at most
   // kWinSample), at places that follow no row or column
   const long long m = n < kWinSample ? n : kWinSample, step = n / (m > 0 ? m : 1);
-  constexpr int kBatch = kWinPerThread;  // all loads in flight
-  for (int j0 = 0; j0 < kWinPerThread; j0 += kBatch) {
-    float v[kBatch];
+#pragma unroll 1
+  for (int round = 0; round < kWinRounds; ++round) {
+    float v[kWinPerThread];  // all loads in flight
 #pragma unroll
-    for (int j = 0; j < kBatch; ++j) {
-      const long long k = (long long)(j0 + j) * kWinThreads + t;
+    for (int j = 0; j < kWinPerThread; ++j) {
+      const long long k = (long long)j * kWinThreads + t;
       const unsigned long long h32 = (unsigned)k * 2654435761u;
-      const long long i = k * step + (long long)(h32 * (unsigned long long)step >> 32);
+      long long i = k * step + (long long)(h32 * (unsigned long long)step >> 32);
+      if (round > 0)  // further places anywhere in the cube
+        i = (long long)__umul64hi((unsigned long long)(round * kWinSample + k) * 0x9e3779b97f4a7c15ull, (unsigned long long)n);
       v[j] = __int_as_float(0x7fc00000);
       if (k < m) v[j] = h.fmt ? half16_value(__ldg(h.bits + i), h.fmt, __ldg(h.scale + i / plane)) : __ldg(x + i);
     }
+    int any = 0;
 #pragma unroll
-    for (int j = 0; j < kBatch; ++j)
-      if (isfinite(v[j])) atomicAdd(&wh[bin_of(v[j], full)], 1u);
+    for (int j = 0; j < kWinPerThread; ++j) {
+      if (!isfinite(v[j])) continue;
+      atomicAdd(&wh[bin_of(v[j], full)], 1u);
+      any = 1;
+    }
+    if (__syncthreads_count(any) >= kWinEnough || m < kWinSample) break;
   }
-  __syncthreads();
   // thread t holds magnitude bins [t * per, t * per + per), both signs
   constexpr int per = (kBinsPerSign + kWinThreads - 1) / kWinThreads;
   unsigned long long c[per], loc = 0;
