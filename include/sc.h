@@ -468,9 +468,14 @@ int sc_noise_scale(sc_ctx *ctx, const float *cube_dev, const int64_t *dims, cons
  *                first extents_cap of them) x_min, x_max, y_min, y_max,
  *                z_min, z_max and the voxel count.
  *   flags        reserved, pass 0.
- * The library keeps buffers in the context (grown on demand): 5/16 byte per
- * voxel, 8 bytes per run of mask voxels along x, 64 per detection. Synchronises
- * the stream (the numbers of runs and detections size the later parts).
+ * The library keeps a buffer in the context, freed with it: 5/16 byte per
+ * voxel, and 8 bytes for each of 65,536 + n / 64 runs of mask voxels along x and
+ * 64 for each of 8,192 + n / 512 detections before the size limits (n voxels;
+ * together about 9/16 byte per voxel), or for as many as the fullest mask of the
+ * context had. A mask that has more is worked through again with a larger
+ * buffer. Where the device has no memory for it, the call makes do with 8 bytes
+ * per run and 64 per detection that the mask has, and is slower. Synchronises
+ * the stream (the host reads the numbers of runs and detections).
  * Errors: SC_ERR_ARG (NULL pointer, dims, radii, negative limits),
  * SC_ERR_NOMEM, SC_ERR_CUDA. */
 int sc_link(sc_ctx *ctx, const uint8_t *mask_dev, const int64_t *dims, int r_xy, int r_z, int min_xy, int min_z,

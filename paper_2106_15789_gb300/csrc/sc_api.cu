@@ -1629,32 +1629,44 @@ int sc_link(sc_ctx* c, const uint8_t* mask_dev, const int64_t* dims, int r_xy, i
   DeviceGuard guard(c->device);
   cudaStream_t s = (cudaStream_t)cuda_stream;
   c->last = s;
-  // One buffer: three totals, the bits, and room for as many runs and
-  // detections as a mask a few per cent full has, or as an earlier call had; a
-  // fuller one starts over with what it turned out to need
-  c->lk_max_runs = std::max(c->lk_max_runs, std::min(n, (1LL << 16) + n / 64));
-  c->lk_max_comp = std::max(c->lk_max_comp, (1LL << 13) + n / 512);
+  // One buffer: three totals, the runs before each chunk, the bits, and room for
+  // as many runs and detections as a mask a few per cent full has, or as an
+  // earlier call had; a fuller one starts over with what it turned out to need.
+  // Where the device has no memory for that, the bits go to the labels' memory
+  // and the room is what the mask is found to need, step by step.
+  bool tight = false;
+  long long max_runs = std::max(c->lk_max_runs, std::min(n, (1LL << 16) + n / 64)), need_runs = 0;
+  long long max_comp = std::max(c->lk_max_comp, (1LL << 13) + n / 512), need_comp = 0;
   int total[3] = {0, 0, 0}, *ext_out = nullptr;
-  for (int attempt = 0; attempt < 3; ++attempt) {
-    const size_t at_runs = 256 + link_bits_bytes(n), at_comp = at_runs + link_runs_bytes(c->lk_max_runs);
-    const int rc = ensure_bytes(&c->lk_buf, &c->lk_cap, at_comp + link_comp_bytes(c->lk_max_comp));
-    if (rc) {
-      c->lk_max_runs = c->lk_max_comp = 0;
-      return rc;
+  for (int attempt = 0;; ++attempt) {
+    if (attempt == 8) return SC_ERR_INTERNAL;  // (not reached: every attempt learns a number or is the last)
+    const size_t at_bits = 256 + link_chunk_bytes(n), at_runs = at_bits + (tight ? 0 : link_bits_bytes(n));
+    const size_t at_comp = at_runs + link_runs_bytes(max_runs);
+    const int rc = ensure_bytes(&c->lk_buf, &c->lk_cap, at_comp + link_comp_bytes(max_comp));
+    if (rc == SC_ERR_NOMEM && !tight && n >= kLinkMinBitsInLabels) {
+      tight = true;
+      max_runs = std::max(need_runs, std::min(n, 4096LL));
+      max_comp = std::max(need_comp, 512LL);
+      continue;
     }
+    if (rc) return rc;
     unsigned char* const buf = static_cast<unsigned char*>(c->lk_buf);
     int* const totals = reinterpret_cast<int*>(buf);
     int launched = 0;
-    CK(launch_link(mask_dev, d, r_xy, r_z, min_xy, min_z, max_xy, max_z, buf + 256,
-                   reinterpret_cast<int*>(buf + at_runs), c->lk_max_runs, reinterpret_cast<int*>(buf + at_comp),
-                   c->lk_max_comp, totals, labels_dev, &ext_out, c->sms, s, &launched));
+    const cudaError_t e =
+        launch_link(mask_dev, d, r_xy, r_z, min_xy, min_z, max_xy, max_z, tight ? nullptr : buf + at_bits,
+                    reinterpret_cast<int*>(buf + 256), reinterpret_cast<int*>(buf + at_runs), max_runs,
+                    reinterpret_cast<int*>(buf + at_comp), max_comp, totals, labels_dev, &ext_out, c->sms, s, &launched);
+    CK(e);
     c->stats.launches += launched;
     CK(cudaMemcpyAsync(total, totals, sizeof(total), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
-    if (total[0] > c->lk_max_runs) c->lk_max_runs = total[0];  // (the number of detections is not known yet)
-    else if (total[1] > c->lk_max_comp) c->lk_max_comp = total[1];
+    if (total[0] > max_runs) max_runs = need_runs = total[0];  // (the number of detections is not known yet)
+    else if (total[1] > max_comp) max_comp = need_comp = total[1];
     else break;
   }
+  c->lk_max_runs = tight ? 0 : max_runs;
+  c->lk_max_comp = tight ? 0 : max_comp;
   const int kept = total[2];
   const long long table = std::min<long long>(kept, extents_cap);
   if (table > 0) {

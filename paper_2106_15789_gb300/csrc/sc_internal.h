@@ -439,16 +439,21 @@ struct LinkTotals {
   }
 };
 
-// Linker. Scratch: bits (link_bits_bytes), runs and comp for at most max_runs
-// runs and max_comp components. totals[3] (device): runs, components, kept
+// Linker. Scratch: bits (link_bits_bytes; null: in the memory of the labels,
+// which hold that many where n >= kLinkMinBitsInLabels), chunk_off
+// (link_chunk_bytes), runs and comp for at most max_runs runs and max_comp
+// components. totals[3] (device): runs, components, kept
 // detections; where either does not fit, nothing after it is meant (the caller
 // grows the buffer and starts over). *ext_out: extents of the kept ones.
+constexpr long long kLinkMinBitsInLabels = 64;
 size_t link_bits_bytes(long long n);
+size_t link_chunk_bytes(long long n);
 size_t link_runs_bytes(long long nruns);
 size_t link_comp_bytes(long long ncomp);
 cudaError_t launch_link(const uint8_t* mask, const long long dims[3], int r_xy, int r_z, int min_xy, int min_z,
-                        int max_xy, int max_z, void* bits, int* runs, long long max_runs, int* comp, long long max_comp,
-                        int* totals, int* lab, int** ext_out, int sms, cudaStream_t s, int* launches);
+                        int max_xy, int max_z, void* bits, int* chunk_off, int* runs, long long max_runs, int* comp,
+                        long long max_comp, int* totals, int* lab, int** ext_out, int sms, cudaStream_t s,
+                        int* launches);
 
 // Host helpers.
 int cascade_widths(double fwhm, int w[3]);

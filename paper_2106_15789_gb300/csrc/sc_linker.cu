@@ -112,13 +112,17 @@ using link::Geo;
 using link::Runs;
 using Totals = LinkTotals;
 
-// A block per chunk, a mask word (32 voxels) per thread. A run starts at a set
-// voxel whose predecessor is not set or lies in another row.
-__global__ void __launch_bounds__(link::kThreads) k_lk_pack(const uint8_t* __restrict__ mask, Geo g, Runs R) {
-  using namespace link;
-  __shared__ int part[kThreads / 32];
+namespace link {
+// A thread's word (32 voxels) of the block's chunk: its bits, where runs start,
+// and the runs before it and in all of the chunk. A run starts at a set voxel
+// whose predecessor is not set or lies in another row. All threads call it.
+struct Word {
+  unsigned bits, starts;
+  int off, total;
+};
+__device__ __forceinline__ Word pack_word(const uint8_t* __restrict__ mask, const Geo& g, int* part) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const long long w = (long long)blockIdx.x * kThreads + tid, v0 = 32 * w;
+  const long long v0 = 32 * ((long long)blockIdx.x * kThreads + tid);
   unsigned bits = 0u;
   if (v0 + 32 <= g.n && (reinterpret_cast<uintptr_t>(mask) & 15u) == 0) {
     const uint4* m = reinterpret_cast<const uint4*>(mask + v0);
@@ -151,12 +155,22 @@ __global__ void __launch_bounds__(link::kThreads) k_lk_pack(const uint8_t* __res
     if (k < warp) off += part[k];
     total += part[k];
   }
-  if (v0 < g.n) {
-    R.bits[w] = bits;
-    R.starts[w] = starts;
-    R.word_off[w] = (unsigned short)off;
+  return Word{bits, starts, off, total};
+}
+}  // namespace link
+
+// A block per chunk, a mask word per thread.
+__global__ void __launch_bounds__(link::kThreads) k_lk_pack(const uint8_t* __restrict__ mask, Geo g, Runs R) {
+  using namespace link;
+  __shared__ int part[kThreads / 32];
+  const Word a = pack_word(mask, g, part);
+  const long long w = (long long)blockIdx.x * kThreads + threadIdx.x;
+  if (32 * w < g.n) {
+    R.bits[w] = a.bits;
+    R.starts[w] = a.starts;
+    R.word_off[w] = (unsigned short)a.off;
   }
-  if (tid == 0) R.chunk_off[blockIdx.x] = total;
+  if (threadIdx.x == 0) R.chunk_off[blockIdx.x] = a.total;
 }
 
 // Exclusive scan of a[0 .. len) in place by one block of 1024 threads, eight
@@ -487,6 +501,25 @@ __global__ void __launch_bounds__(256) k_lk_expand(Geo g, Runs R, const int* __r
   }
 }
 
+// The same where the bits lie in the memory of the labels: they are taken from
+// the mask once more, a block per chunk and a word per thread.
+__global__ void __launch_bounds__(link::kThreads) k_lk_expand_mask(const uint8_t* __restrict__ mask, Geo g,
+                                                                   const int* __restrict__ chunk_off,
+                                                                   const int* __restrict__ run_id,
+                                                                   const int* __restrict__ new_id,
+                                                                   int* __restrict__ lab, Totals t) {
+  using namespace link;
+  __shared__ int part[kThreads / 32];
+  if (!t.all_fit()) return;
+  const Word a = pack_word(mask, g, part);
+  const long long v0 = 32 * ((long long)blockIdx.x * kThreads + threadIdx.x);
+  int run = __ldg(chunk_off + blockIdx.x) + a.off - 1;
+  for (int i = 0; i < 32 && v0 + i < g.n; ++i) {
+    run += (int)(a.starts >> i & 1u);
+    lab[v0 + i] = a.bits >> i & 1u ? __ldg(new_id + __ldg(run_id + run) - 1) : 0;
+  }
+}
+
 // ---------------------------------------------------------------------------
 namespace {
 inline int grid_for(long long n, int sms, int threads) {
@@ -495,14 +528,14 @@ inline int grid_for(long long n, int sms, int threads) {
   return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
 size_t up16(size_t v) { return (v + 15) & ~(size_t)15; }
-Runs runs_at(void* bits, long long n) {
+Runs runs_at(void* bits, int* chunk_off, long long n) {
   const size_t words = (size_t)((n + 31) / 32);
   unsigned char* b = static_cast<unsigned char*>(bits);
   Runs R;
   R.bits = reinterpret_cast<unsigned*>(b);
   R.starts = reinterpret_cast<unsigned*>(b + up16(4 * words));
   R.word_off = reinterpret_cast<unsigned short*>(b + 2 * up16(4 * words));
-  R.chunk_off = reinterpret_cast<int*>(b + 2 * up16(4 * words) + up16(2 * words));
+  R.chunk_off = chunk_off;
   return R;
 }
 long long chunks_of(long long n) { return (n + link::kChunk - 1) / link::kChunk; }
@@ -510,18 +543,20 @@ long long chunks_of(long long n) { return (n + link::kChunk - 1) / link::kChunk;
 
 size_t link_bits_bytes(long long n) {
   const size_t words = (size_t)((n + 31) / 32);
-  return 2 * up16(4 * words) + up16(2 * words) + up16(4 * (size_t)(chunks_of(n) + 1));
+  return 2 * up16(4 * words) + up16(2 * words);
 }
+size_t link_chunk_bytes(long long n) { return up16(4 * (size_t)(chunks_of(n) + 1)); }
 size_t link_runs_bytes(long long nruns) {
   return up16(4 * (size_t)(2 * nruns + (nruns + link::kFlat - 1) / link::kFlat + 1));
 }
 size_t link_comp_bytes(long long ncomp) { return 4 * (size_t)(16 * ncomp + 1); }
 
 cudaError_t launch_link(const uint8_t* mask, const long long dims[3], int r_xy, int r_z, int min_xy, int min_z,
-                        int max_xy, int max_z, void* bits, int* runs, long long max_runs, int* comp, long long max_comp,
-                        int* totals, int* lab, int** ext_out, int sms, cudaStream_t s, int* launches) {
+                        int max_xy, int max_z, void* bits, int* chunk_off, int* runs, long long max_runs, int* comp,
+                        long long max_comp, int* totals, int* lab, int** ext_out, int sms, cudaStream_t s,
+                        int* launches) {
   const Geo g{(int)dims[0], (int)dims[1], (int)dims[2], dims[0] * dims[1] * dims[2], r_xy, r_z};
-  const Runs R = runs_at(bits, g.n);
+  const Runs R = runs_at(bits ? bits : lab, chunk_off, g.n);
   const Totals t{totals, max_runs, max_comp};
   const long long chunks = chunks_of(g.n), flat = (max_runs + link::kFlat - 1) / link::kFlat;
   int *const parent = runs, *const run_id = runs + max_runs, *const counts = runs + 2 * max_runs;
@@ -544,7 +579,8 @@ cudaError_t launch_link(const uint8_t* mask, const long long dims[3], int r_xy, 
   k_cc_keep<<<grid_for(max_comp, sms, 256), 256, 0, s>>>(ext, t, min_xy, min_z, max_xy, max_z, keep, new_id);
   k_scan_block<<<1, 1024, 0, s>>>(keep, 0, t, LINK_SCAN_COMPS, 1, totals + 2);
   k_cc_compact<<<grid_for(max_comp, sms, 256), 256, 0, s>>>(ext, new_id, keep, t, kept, new_id);
-  k_lk_expand<<<grid_for((g.n + 3) / 4, sms, 256), 256, 0, s>>>(g, R, run_id, new_id, lab, t);
+  if (bits) k_lk_expand<<<grid_for((g.n + 3) / 4, sms, 256), 256, 0, s>>>(g, R, run_id, new_id, lab, t);
+  else k_lk_expand_mask<<<(unsigned)chunks, link::kThreads, 0, s>>>(mask, g, R.chunk_off, run_id, new_id, lab, t);
   *launches = 13;
   *ext_out = kept;
   return cudaGetLastError();
