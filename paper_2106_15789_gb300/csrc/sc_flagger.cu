@@ -97,47 +97,27 @@ __device__ __forceinline__ void neumaier_add(float* s, float* c, float x) {
   *s = t;
 }
 
-__device__ __forceinline__ float two_diff(float x, float b, float* err) {
-  const float s = __fsub_rn(x, b);
-  const float bb = __fsub_rn(s, x);
-  *err = __fadd_rn(__fsub_rn(x, __fsub_rn(s, bb)), __fsub_rn(-b, bb));
-  return s;
-}
-
-// The float of |x - m|, m = (a + b) / 2 (a == b for an odd count): correctly
-// rounded for an odd count, faithfully (TwoSum) for an even one.
-__device__ __forceinline__ unsigned mad_key(float x, float a, float b, bool even) {
-  float d;
-  if (!even) {
-    d = __fsub_rn(x, a);
-  } else {
-    float e1, e2;
-    const float t = two_diff(x, 0.5f * a, &e1);
-    const float u = two_diff(t, 0.5f * b, &e2);
-    d = __fadd_rn(u, __fadd_rn(e1, e2));
-  }
-  return __float_as_uint(fabsf(d)) | 0x80000000u;
-}
-
-// |x - m| of the median m = (a + b) / 2, faithfully rounded: -m = h + l
-// exactly (a TwoSum of the halves; l is 0 for an odd count), then x + h as a
-// sum and its error, to which l is added.
+// |x - m| of the median m = (a + b) / 2 (a == b for an odd count), faithfully
+// rounded (correctly for an odd count): -m = h + l exactly (a TwoSum of the
+// halves; l is 0 for an odd count), then x + h as a sum and its error, to which
+// l is added. NaN where x + h overflows.
 struct Deviation {
   float h, l;
   __device__ __forceinline__ float operator()(float x) const {
-    const float t = __fadd_rn(x, h);
-    const float b = __fsub_rn(t, x);
-    const float e = __fadd_rn(__fsub_rn(x, __fsub_rn(t, b)), __fsub_rn(h, b));
+    float e;
+    const float t = two_sum(x, h, &e);
     return fabsf(__fadd_rn(t, __fadd_rn(e, l)));
   }
 };
 __device__ __forceinline__ Deviation deviation_of(float a, float b) {
-  const float ha = -0.5f * a, hb = -0.5f * b;
-  Deviation d;
-  d.h = a == b ? -a : __fadd_rn(ha, hb);
-  const float bb = __fsub_rn(d.h, ha);
-  d.l = a == b ? 0.0f : __fadd_rn(__fsub_rn(ha, __fsub_rn(d.h, bb)), __fsub_rn(hb, bb));
+  Deviation d{-a, 0.0f};
+  if (a != b) d.h = two_sum(-0.5f * a, -0.5f * b, &d.l);
   return d;
+}
+// Its key (an overflow the largest).
+__device__ __forceinline__ unsigned deviation_key(const Deviation& dev, float x) {
+  const float d = dev(x);
+  return fkey(d == d ? d : INFINITY);
 }
 
 // Order statistic `rank` (and, with want_next, rank + 1) of key_of(x) over
@@ -273,9 +253,10 @@ __device__ void block_noise(const float* __restrict__ src, long long n, int mode
   unsigned k2 = 0u;
   const unsigned k1 = stream_select(src, n, r1, [](float x) { return fkey(x); }, S, even, &k2);
   const float ma = fkey_inv(k1), mb = even ? fkey_inv(k2) : ma;
+  const Deviation dev = deviation_of(ma, mb);
   unsigned a2 = 0u;
   const unsigned a1 =
-      stream_select(src, n, r1, [=](float x) { return mad_key(x, ma, mb, even); }, S, even, &a2);
+      stream_select(src, n, r1, [=](float x) { return deviation_key(dev, x); }, S, even, &a2);
   const double mad = even ? 0.5 * ((double)fkey_inv(a1) + (double)fkey_inv(a2)) : (double)fkey_inv(a1);
   *sigma = kMadToSigma * mad;
   *median = even ? 0.5 * ((double)ma + (double)mb) : (double)ma;
@@ -467,8 +448,7 @@ constexpr int kFew = 1024;                // copies ranked directly
 struct Chan {
   float lo, hi;
   unsigned finite, below, n;  // finite values, those under lo, copies (may exceed the room)
-  float ma, mb;               // the two middle values
-  Deviation dev;                 // |x - m| of their mean
+  Deviation dev;              // |x - m| of the median
 };
 
 // The digits whose cumulative ranges in S->hist hold ranks ra and rb, and the
@@ -559,10 +539,6 @@ struct KeyOfDev {
   __device__ __forceinline__ float value(unsigned k) const { return __uint_as_float(k); }
 };
 
-__device__ __forceinline__ float abs_dev(float x, float a, float b, bool even) {
-  return __uint_as_float(mad_key(x, a, b, even) & 0x7fffffffu);
-}
-
 // Order statistics r and (want_next) r + 1 among the n copies in list (all in
 // [lo, hi], more than r of them). False (uniformly) when the step of the rank
 // holds too many, or the next one lies beyond the copies.
@@ -642,7 +618,7 @@ __global__ void __launch_bounds__(flag::kThreads, 1)
   __shared__ Scratch S;
   float lo, hi;
   plane_bracket<21>(cube + (long long)blockIdx.x * plane, plane, [](float x) { return x; }, KeyOfValue{}, &S, &lo, &hi);
-  if (threadIdx.x == 0) ch[blockIdx.x] = Chan{lo, hi, 0u, 0u, 0u, 0.0f, 0.0f, Deviation{0.0f, 0.0f}};
+  if (threadIdx.x == 0) ch[blockIdx.x] = Chan{lo, hi, 0u, 0u, 0u, Deviation{0.0f, 0.0f}};
 }
 
 // A pass over the cube: the values (DEV: their |x - m|) of every channel under
@@ -743,8 +719,8 @@ __global__ void __launch_bounds__(flag::kThreads, 1)
   if (!done) {
     unsigned k2 = 0u;
     if (DEV) {
-      const float ma = c.ma, mb = c.mb;
-      v1 = fkey_inv(stream_select(src, plane, r1, [=](float x) { return mad_key(x, ma, mb, even); }, &S, even, &k2));
+      const Deviation dev = c.dev;
+      v1 = fkey_inv(stream_select(src, plane, r1, [=](float x) { return deviation_key(dev, x); }, &S, even, &k2));
     } else {
       v1 = fkey_inv(stream_select(src, plane, r1, [](float x) { return fkey(x); }, &S, even, &k2));
     }
@@ -760,10 +736,10 @@ __global__ void __launch_bounds__(flag::kThreads, 1)
     if (threadIdx.x == 0) noise[z] = __double2float_rn(sigma);
   } else {
     float lo, hi;
-    const float ma = v1, mb = v2;
+    const Deviation dev = deviation_of(v1, v2);
     __syncthreads();
-    plane_bracket<20>(src, plane, [=](float x) { return abs_dev(x, ma, mb, even); }, KeyOfDev{}, &S, &lo, &hi);
-    if (threadIdx.x == 0) ch[z] = Chan{fmaxf(lo, 0.0f), hi, c.finite, 0u, 0u, ma, mb, deviation_of(ma, mb)};
+    plane_bracket<20>(src, plane, dev, KeyOfDev{}, &S, &lo, &hi);
+    if (threadIdx.x == 0) ch[z] = Chan{fmaxf(lo, 0.0f), hi, c.finite, 0u, 0u, dev};
   }
 }
 

@@ -136,3 +136,17 @@ def test_short_chunks(ctx, nz):
     a = ctx.run(c, kernels, 3.0)
     b = ctx.run(c, kernels, 3.0, flags=sc.SC_FLAG_GENERIC)
     assert torch.equal(a[0], b[0]) and a[1] == b[1] and a[2] == b[2]
+
+
+def test_planes_on_either_side_of_the_passes(ctx):
+    """The same finite values in planes of the size that takes the passes over
+    the cube and in smaller ones that a block streams: the same noise to the
+    last bit (an even count, whose |x - m| is rounded from two middle values)."""
+    nz, n = 200, 106 * 307  # below 2^15, with 400 blanked voxels above it
+    x = np.random.default_rng(3).standard_normal((nz, n)).astype(np.float32)
+    x += np.linspace(0, 30, nz, dtype=np.float32)[:, None]
+    big = np.full((nz, 181 * 182), np.nan, dtype=np.float32)
+    big[:, :n] = x
+    noises = [ctx.autoflag(torch.from_numpy(a.reshape(shape)).cuda(), 1e9, True, False, "mad")[3]
+              for a, shape in ((x, (nz, 106, 307)), (big, (nz, 181, 182)))]
+    np.testing.assert_array_equal(noises[0], noises[1])
