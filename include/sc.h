@@ -498,8 +498,13 @@ int sc_link(sc_ctx *ctx, const uint8_t *mask_dev, const int64_t *dims, int r_xy,
  *   n_flagged    NULL or int64[2]: flagged channels, flagged pixels.
  *   flags        reserved, pass 0.
  * Pixels mode needs nz <= 1536 (a tile of spectra in shared memory). The
- * library keeps 5 bytes per channel and per pixel in the context. Synchronises
- * when any host output is given. Errors: SC_ERR_ARG (NULL pointer, dims,
+ * library keeps 5 bytes per channel and per pixel in the context and, for
+ * channel noises by MAD or Gaussian fit of planes of 32,768 pixels or more,
+ * scratch of half a byte per voxel, at most 256 MiB (or one channel's), which
+ * larger cubes use for a group of channels at a time. Where the device has no
+ * memory for that the groups are smaller, or a block each measures the
+ * channels: slower, with the same noises. Synchronises when any host output
+ * is given. Errors: SC_ERR_ARG (NULL pointer, dims,
  * k < 0, what, unknown mode), SC_ERR_UNSUPPORTED (pixels with nz > 1536),
  * SC_ERR_NOMEM, SC_ERR_CUDA. */
 #define SC_AUTOFLAG_CHANNELS 0x1u

@@ -50,8 +50,8 @@ struct sc_ctx {
   long long lk_max_runs = 0, lk_max_comp = 0;  // what it has room for
   unsigned char* af_buf = nullptr;  // sc_autoflag: noises, flags and statistics (lazy, grown)
   size_t af_cap = 0;
-  void* af_chan = nullptr;          // and its channel passes' brackets and copies (lazy, grown)
-  size_t af_chan_cap = 0;
+  void* af_chan = nullptr;          // and its channel passes' copies and brackets (lazy, grown)
+  size_t af_chan_cap = 0, af_chan_tried = 0;  // bytes it has, and the most that was asked for
   uint8_t* stage_mask = nullptr;
   // sc_run_host_many (lazy): two device input / mask sets, the per-channel
   // scales of 16-bit cubes, the copy stream and its events, per-cube results
@@ -455,6 +455,23 @@ int ensure_bytes(void** p, size_t* cap, size_t need) {
   }
   *cap = need;
   return SC_OK;
+}
+
+// Channels that the auto-flagger measures at a time (0: each by a block that
+// streams its plane): as many as fit kChanScratchMax bytes of scratch, in groups
+// of one size, or as many as the device has memory for.
+int chan_group(sc_ctx* c, const long long d[3], int noise_mode) {
+  const size_t per = chan_plane_bytes(d, noise_mode);
+  if (per == 0) return 0;
+  const long long nz = d[2], most = std::min(nz, std::max(1LL, (long long)(kChanScratchMax / per)));
+  const long long groups = (nz + most - 1) / most, want = (nz + groups - 1) / groups;
+  if (want * per > c->af_chan_cap && (want * per > c->af_chan_tried || c->af_chan_cap == 0)) {
+    // (a size that the device once had no memory for is not asked for again
+    // while a smaller buffer serves)
+    c->af_chan_tried = want * per;
+    for (long long g = want; g > 0 && ensure_bytes(&c->af_chan, &c->af_chan_cap, g * per) != SC_OK;) g /= 2;
+  }
+  return (int)std::min(want, (long long)(c->af_chan_cap / per));
 }
 
 // Device staging cube and mask of max_voxels elements (allocated on first use).
@@ -1708,29 +1725,15 @@ int sc_autoflag(sc_ctx* c, const float* cube_dev, const int64_t* dims, double k,
     }
     c->af_cap = need;
   }
-  // scratch of the channel passes (half a byte per voxel), grown on
-  // demand; without it the channels are measured by a block each
-  const size_t chan_need = ch ? chan_scratch_bytes(d, noise_mode) : 0;
-  if (chan_need > c->af_chan_cap) {
-    cudaFree(c->af_chan);
-    c->af_chan = nullptr;
-    c->af_chan_cap = 0;
-    if (cudaMalloc(&c->af_chan, chan_need) == cudaSuccess) {
-      c->af_chan_cap = chan_need;
-    } else {
-      cudaGetLastError();
-      c->af_chan = nullptr;
-    }
-  }
-  void* const chan_scratch = chan_need > 0 && chan_need <= c->af_chan_cap ? c->af_chan : nullptr;
+  const int group = ch ? chan_group(c, d, noise_mode) : 0;
   double* stats = reinterpret_cast<double*>(c->af_buf);
   float* cn = reinterpret_cast<float*>(c->af_buf + 64);
   float* pn = cn + d[2];
   uint8_t* cf = reinterpret_cast<uint8_t*>(pn + plane);
   uint8_t* pf = cf + d[2];
   CK(launch_autoflag(cube_dev, d, k, ch ? 1 : 0, px ? 1 : 0, noise_mode, out_dev, cn, pn, cf,
-                     pf, stats, chan_scratch, c->sms, s));
-  c->stats.launches += (ch ? (chan_scratch ? 7 : 3) : 0) + (px ? 3 : 0) + 1;
+                     pf, stats, c->af_chan, group, c->sms, s));
+  c->stats.launches += (ch ? (group > 0 ? kChanLaunches * ((d[2] + group - 1) / group) : 1) + 2 : 0) + (px ? 3 : 0) + 1;
   const bool want_counts = n_flagged != nullptr;
   std::vector<uint8_t> cf_h, pf_h;
   if (ch && (chan_flags_host || want_counts)) {

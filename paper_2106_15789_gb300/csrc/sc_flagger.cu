@@ -938,39 +938,44 @@ cudaError_t launch_pix(const float* cube, int nx, int ny, int nz, int mode, floa
 // Room for the copies of one plane: a bracket holds about 6 % of it.
 static long long chan_room(long long plane) { return (plane / 8 + 4 + 3) & ~3LL; }
 
-size_t chan_scratch_bytes(const long long dims[3], int mode) {
+size_t chan_plane_bytes(const long long dims[3], int mode) {
   const long long plane = dims[0] * dims[1];
   if (mode == SC_NOISE_STD || plane < flag::kChanMinPlane || plane >= (1LL << 32)) return 0;
-  const size_t head = ((size_t)dims[2] * sizeof(flag::Chan) + 15) & ~(size_t)15;
-  return head + sizeof(float) * (size_t)chan_room(plane) * (size_t)dims[2];
+  return sizeof(float) * (size_t)chan_room(plane) + ((sizeof(flag::Chan) + 15) & ~(size_t)15);
 }
 
-static cudaError_t launch_chan_mad(const float* cube, long long plane, int nz, int mode, void* scratch, float* noise,
-                                   int sms, cudaStream_t s) {
-  flag::Chan* ch = static_cast<flag::Chan*>(scratch);
-  const size_t head = ((size_t)nz * sizeof(flag::Chan) + 15) & ~(size_t)15;
-  float* lists = reinterpret_cast<float*>(static_cast<unsigned char*>(scratch) + head);
+// Channels [0, nz) in groups of `group`, whose copies and brackets lie in scratch.
+static cudaError_t launch_chan_mad(const float* cube, long long plane, int nz, int mode, void* scratch, int group,
+                                   float* noise, int sms, cudaStream_t s) {
   const long long room = chan_room(plane);
-  const long long warps = (plane + flag::kPassRun - 1) / flag::kPassRun * nz;
-  const long long want = (warps + flag::kPassWarps - 1) / flag::kPassWarps;
-  const int grid = (int)(want < 4LL * sms ? want : 4LL * sms);
-  k_chan_sample<<<nz, flag::kThreads, 0, s>>>(cube, plane, ch);
-  k_chan_pass<false><<<grid, flag::kPassThreads, 0, s>>>(cube, plane, nz, ch, lists, room);
-  k_chan_select<false><<<nz, flag::kThreads, 0, s>>>(cube, plane, ch, lists, room, mode, noise);
-  k_chan_pass<true><<<grid, flag::kPassThreads, 0, s>>>(cube, plane, nz, ch, lists, room);
-  k_chan_select<true><<<nz, flag::kThreads, 0, s>>>(cube, plane, ch, lists, room, mode, noise);
+  float* const lists = static_cast<float*>(scratch);
+  flag::Chan* const ch = reinterpret_cast<flag::Chan*>(lists + room * group);
+  const long long runs = (plane + flag::kPassRun - 1) / flag::kPassRun;
+  for (int z0 = 0; z0 < nz; z0 += group) {
+    const int n = nz - z0 < group ? nz - z0 : group;
+    const float* const part = cube + z0 * plane;
+    const long long want = (runs * n + flag::kPassWarps - 1) / flag::kPassWarps;
+    const int grid = (int)(want < 4LL * sms ? want : 4LL * sms);
+    k_chan_sample<<<n, flag::kThreads, 0, s>>>(part, plane, ch);
+    k_chan_pass<false><<<grid, flag::kPassThreads, 0, s>>>(part, plane, n, ch, lists, room);
+    k_chan_select<false><<<n, flag::kThreads, 0, s>>>(part, plane, ch, lists, room, mode, noise + z0);
+    k_chan_pass<true><<<grid, flag::kPassThreads, 0, s>>>(part, plane, n, ch, lists, room);
+    k_chan_select<true><<<n, flag::kThreads, 0, s>>>(part, plane, ch, lists, room, mode, noise + z0);
+  }
   return cudaGetLastError();
 }
 
 cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k, int channels, int pixels,
                             int mode, float* out, float* chan_noise, float* pix_noise, uint8_t* chan_flags,
-                            uint8_t* pix_flags, double* stats, void* chan_scratch, int sms, cudaStream_t s) {
+                            uint8_t* pix_flags, double* stats, void* chan_scratch, int chan_group, int sms,
+                            cudaStream_t s) {
   const int nx = (int)dims[0], ny = (int)dims[1], nz = (int)dims[2];
   const long long plane = (long long)nx * ny;
   cudaError_t e = cudaSuccess;
   if (channels) {
-    if (chan_scratch) {
-      if ((e = launch_chan_mad(cube, plane, nz, mode, chan_scratch, chan_noise, sms, s)) != cudaSuccess) return e;
+    if (chan_group > 0) {
+      e = launch_chan_mad(cube, plane, nz, mode, chan_scratch, chan_group, chan_noise, sms, s);
+      if (e != cudaSuccess) return e;
     } else {
       k_chan_noise<<<nz < 2 * sms ? nz : 2 * sms, flag::kThreads, 0, s>>>(cube, plane, nz, mode, chan_noise);
     }

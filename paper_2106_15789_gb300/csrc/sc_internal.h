@@ -415,10 +415,14 @@ cudaError_t launch_noise_apply(const float* cube, const long long dims[3], const
 constexpr int kFlagMaxChannelsForPixels = 1536;  // spectra staged in shared memory
 cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k, int channels, int pixels,
                             int noise_mode, float* out, float* chan_noise, float* pix_noise, uint8_t* chan_flags,
-                            uint8_t* pix_flags, double* stats, void* chan_scratch, int sms, cudaStream_t s);
-// Bytes of chan_scratch with which the channel noises take two passes over the
-// cube (0: they do not; null: one block per channel streams its plane).
-size_t chan_scratch_bytes(const long long dims[3], int mode);
+                            uint8_t* pix_flags, double* stats, void* chan_scratch, int chan_group, int sms,
+                            cudaStream_t s);
+// Bytes of chan_scratch per channel of a group (chan_group channels are
+// measured at a time by two passes over their planes). 0: the planes are not
+// measured so; they are, as with chan_group 0, streamed by a block each.
+size_t chan_plane_bytes(const long long dims[3], int mode);
+constexpr size_t kChanScratchMax = (size_t)1 << 28;  // what a group may take (one channel at least)
+constexpr int kChanLaunches = 5;                     // kernels of a group
 
 constexpr int kLinkMaxRadius = 32;  // merging radii in voxels
 // A linker call's totals (device memory, cleared before its kernels) and the

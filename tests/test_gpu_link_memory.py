@@ -5,11 +5,10 @@ import numpy as np
 import pytest
 import torch
 
+from full_device import MB, FullDevice
 from paper_2106_15789_gb300 import Context
 
 pytestmark = pytest.mark.gpu
-
-MB = 1 << 20
 
 
 def _boxes(shape, count, seed, gap):
@@ -20,32 +19,6 @@ def _boxes(shape, count, seed, gap):
         z, y, x = (int(rng.integers(0, n - 24)) for n in shape)
         m[z:z + rng.integers(1, 20), y:y + rng.integers(1, 20), x:x + rng.integers(1, 24):gap] = 1
     return torch.from_numpy(m).cuda()
-
-
-class _Full:
-    """Holds all of the device's free memory but `left` bytes."""
-
-    def __init__(self, left):
-        torch.cuda.synchronize()
-        torch.cuda.empty_cache()
-        self.held = []
-        for unit in (1 << 30, 64 * MB, 2 * MB):
-            while True:
-                free = torch.cuda.mem_get_info()[0]
-                if free - left < unit:
-                    break
-                try:
-                    self.held.append(torch.empty((free - left) // unit * unit, dtype=torch.uint8, device="cuda"))
-                except torch.OutOfMemoryError:
-                    break
-        self.free = torch.cuda.mem_get_info()[0]
-
-    def __enter__(self):
-        return self
-
-    def __exit__(self, *a):
-        self.held.clear()
-        torch.cuda.empty_cache()
 
 
 # few runs and detections (a few hundred KB); more than the first tight room
@@ -59,7 +32,7 @@ def test_link_beside_a_full_device(gap, r_xy, count):
         want, n, ext = ctx.link(mask, r_xy, 1, min_xy=2)
     with Context(0, 1 << 16) as ctx:
         ctx.link(mask[:3], r_xy, 1)  # (the kernels are loaded)
-        with _Full(24 * MB) as full:
+        with FullDevice(24 * MB) as full:
             assert full.free < 32 * MB
             _, n1, ext1 = ctx.link(mask, r_xy, 1, min_xy=2, labels=labels)
         assert n1 == n and np.array_equal(ext1, ext) and torch.equal(labels, want)
@@ -80,6 +53,6 @@ def test_room_of_a_dense_mask_is_given_up():
         want, n, ext = ctx.link(mask, 1, 1)
     with Context(0, 1 << 16) as ctx:
         assert ctx.link(dense, 2, 0)[1] == 64
-        with _Full(8 * MB):  # with the 39 MB that the context holds: not for 34 + 20 + 9
+        with FullDevice(8 * MB):  # with the 39 MB that the context holds: not for 34 + 20 + 9
             _, n1, ext1 = ctx.link(mask, 1, 1, labels=labels)
         assert n1 == n and np.array_equal(ext1, ext) and torch.equal(labels, want)
