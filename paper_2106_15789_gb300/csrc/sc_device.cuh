@@ -185,6 +185,25 @@ __device__ __forceinline__ float two_sum(float x, float y, float* err) {
   return s;
 }
 
+// *s + *c += x with Neumaier's compensation (the running error of the float
+// sum is kept in *c).
+__device__ __forceinline__ void neumaier_add(float* s, float* c, float x) {
+  const float t = __fadd_rn(*s, x);
+  const float e = fabsf(*s) >= fabsf(x) ? __fadd_rn(__fsub_rn(*s, t), x) : __fadd_rn(__fsub_rn(x, t), *s);
+  *c = __fadd_rn(*c, e);
+  *s = t;
+}
+
+// Keys whose order is that of the values: of any float, and of non-negative ones.
+struct KeyOfValue {
+  __device__ __forceinline__ unsigned operator()(float v) const { return fkey(v); }
+  __device__ __forceinline__ float value(unsigned k) const { return fkey_inv(k); }
+};
+struct KeyOfDev {
+  __device__ __forceinline__ unsigned operator()(float v) const { return __float_as_uint(v); }
+  __device__ __forceinline__ float value(unsigned k) const { return __uint_as_float(k); }
+};
+
 // Bit i: byte i of x is not 0.
 __device__ __forceinline__ unsigned nonzero_bits(unsigned x) {
   const unsigned b = ((((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | x) >> 7) & 0x01010101u;

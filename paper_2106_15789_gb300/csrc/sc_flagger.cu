@@ -90,13 +90,6 @@ __device__ __forceinline__ double block_sum_d(double v, double* part) {
   return r;
 }
 
-__device__ __forceinline__ void neumaier_add(float* s, float* c, float x) {
-  const float t = __fadd_rn(*s, x);
-  const float e = fabsf(*s) >= fabsf(x) ? __fadd_rn(__fsub_rn(*s, t), x) : __fadd_rn(__fsub_rn(x, t), *s);
-  *c = __fadd_rn(*c, e);
-  *s = t;
-}
-
 // |x - m| of the median m = (a + b) / 2 (a == b for an odd count), faithfully
 // rounded (correctly for an odd count): -m = h + l exactly (a TwoSum of the
 // halves; l is 0 for an odd count), then x + h as a sum and its error, to which
@@ -529,15 +522,6 @@ __device__ void plane_bracket(const float* __restrict__ src, long long n, Of of,
   *lo = fmaxf(a, a + (float)da * w);
   *hi = fminf(b, a + (float)(db + 1u) * w);
 }
-
-struct KeyOfValue {
-  __device__ __forceinline__ unsigned operator()(float v) const { return fkey(v); }
-  __device__ __forceinline__ float value(unsigned k) const { return fkey_inv(k); }
-};
-struct KeyOfDev {
-  __device__ __forceinline__ unsigned operator()(float v) const { return __float_as_uint(v); }
-  __device__ __forceinline__ float value(unsigned k) const { return __uint_as_float(k); }
-};
 
 // Order statistics r and (want_next) r + 1 among the n copies in list (all in
 // [lo, hi], more than r of them). False (uniformly) when the step of the rank

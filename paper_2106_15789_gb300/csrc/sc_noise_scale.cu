@@ -212,20 +212,14 @@ __device__ __forceinline__ void find_digits(Scratch* S, unsigned ra, unsigned rb
 // and then - b/2 are taken exactly as sums of two floats and added back, which
 // rounds the exact difference faithfully (within one unit in the last place)
 // in single precision, without the slow FP64 pipe.
-__device__ __forceinline__ float two_diff(float x, float b, float* err) {
-  const float s = __fsub_rn(x, b);
-  const float bb = __fsub_rn(s, x);
-  *err = __fadd_rn(__fsub_rn(x, __fsub_rn(s, bb)), __fsub_rn(-b, bb));
-  return s;
-}
 struct AbsDev {
   float a, b;
   bool even;
   __device__ __forceinline__ float operator()(float x) const {
     if (!even) return fabsf(__fsub_rn(x, a));
     float e1, e2;
-    const float t = two_diff(x, 0.5f * a, &e1);
-    const float u = two_diff(t, 0.5f * b, &e2);
+    const float t = two_sum(x, -0.5f * a, &e1);
+    const float u = two_sum(t, -0.5f * b, &e2);
     return fabsf(__fadd_rn(u, __fadd_rn(e1, e2)));
   }
 };
@@ -430,14 +424,6 @@ __device__ void sample_bracket(Scratch* S, int slots, Of of, Key key, unsigned n
   *hi = fminf(b, a + (float)(S->digit[1] + 1u) * step);
   __syncthreads();
 }
-struct KeyOfValue {
-  __device__ __forceinline__ unsigned operator()(float v) const { return fkey(v); }
-  __device__ __forceinline__ float value(unsigned k) const { return fkey_inv(k); }
-};
-struct KeyOfDev {
-  __device__ __forceinline__ unsigned operator()(float v) const { return __float_as_uint(v); }
-  __device__ __forceinline__ float value(unsigned k) const { return __uint_as_float(k); }
-};
 
 // Samples every 8th voxel (of rows over 4,096 voxels fewer) of every rstep-th
 // row, the offset moving with the row, into the threads' columns; returns the
@@ -486,15 +472,6 @@ __device__ __forceinline__ int take_sample(const Win& w, Scratch* S) {
   c = __reduce_add_sync(0xffffffffu, c);
   if (lane == 0 && c) atomicAdd(&S->n_sample, c);
   return slot;
-}
-
-// *s + *c += x with Neumaier's compensation (the running error of the float
-// sum is kept in *c).
-__device__ __forceinline__ void neumaier_add(float* s, float* c, float x) {
-  const float t = __fadd_rn(*s, x);
-  const float e = fabsf(*s) >= fabsf(x) ? __fadd_rn(__fsub_rn(*s, t), x) : __fadd_rn(__fsub_rn(x, t), *s);
-  *c = __fadd_rn(*c, e);
-  *s = t;
 }
 
 __device__ __forceinline__ double block_sum_d(double v, double* part) {
