@@ -500,7 +500,7 @@ int sc_link(sc_ctx *ctx, const uint8_t *mask_dev, const int64_t *dims, int r_xy,
  * Pixels mode needs nz <= 1536 (a tile of spectra in shared memory). The
  * library keeps 5 bytes per channel and per pixel in the context and, for
  * channel noises by MAD or Gaussian fit of planes of 32,768 pixels or more,
- * scratch of half a byte per voxel, at most 256 MiB (or one channel's), which
+ * scratch of half a byte per voxel, at most 1 GiB (or one channel's), which
  * larger cubes use for a group of channels at a time. Where the device has no
  * memory for that the groups are smaller, or a block each measures the
  * channels: slower, with the same noises. Synchronises when any host output

@@ -421,7 +421,7 @@ cudaError_t launch_autoflag(const float* cube, const long long dims[3], double k
 // measured at a time by two passes over their planes). 0: the planes are not
 // measured so; they are, as with chan_group 0, streamed by a block each.
 size_t chan_plane_bytes(const long long dims[3], int mode);
-constexpr size_t kChanScratchMax = (size_t)1 << 28;  // what a group may take (one channel at least)
+constexpr size_t kChanScratchMax = (size_t)1 << 30;  // what a group may take (one channel at least)
 constexpr int kChanLaunches = 5;                     // kernels of a group
 
 constexpr int kLinkMaxRadius = 32;  // merging radii in voxels
