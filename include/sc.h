@@ -72,8 +72,8 @@ extern "C" {
 
 /* ---- warning bits (sc_stats.warnings, set per run) -------------------- */
 #define SC_WARN_ZERO_SIGMA 0x1u     /* some pair had sigma == 0 and added nothing to the mask */
-#define SC_WARN_FULL_SELECT 0x2u    /* a selection needed full passes (candidate set above capacity) */
-#define SC_WARN_FULL_CLIP 0x4u      /* a clip needed a separate pass (ambiguous set above capacity) */
+#define SC_WARN_FULL_SELECT 0x2u    /* reserved (a selection that needs full passes is not reported) */
+#define SC_WARN_FULL_CLIP 0x4u      /* reserved (a clip that needs a pass of its own is not reported) */
 #define SC_WARN_RANGE 0x8u          /* max|X| / sigma_0 exceeds 2^20: smoothed values may lose exactness */
 #define SC_WARN_GAUSS_FALLBACK 0x10u /* SC_NOISE_GAUSS: a histogram without a Gaussian-fit root; the MAD noise stood */
 

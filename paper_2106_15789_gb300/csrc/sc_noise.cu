@@ -7,10 +7,12 @@
 // Data flow for one measurement over an array S of n values:
 //   k_hist      (or the smoothing kernel's epilogue): histogram of S over
 //               bins of the float bits (monotone in the value).
-//   k_plan      one block: ranks of the middle order statistics -> the bins
-//               holding the median; from the bin counts alone, thresholds
-//               T1 < MAD < T2 and the value windows that can hold the MAD's
-//               elements; bounds on t*sigma for the clip; capacity checks.
+//   k_plan      a cluster of eight blocks: ranks of the middle order
+//               statistics -> the bins holding the median; from the bin counts
+//               alone, thresholds T1 < MAD < T2 and the value windows that can
+//               hold the MAD's elements; bounds on t*sigma for the clip;
+//               capacity checks; the candidate pass's class table. It clears
+//               the histogram for the next measurement of the run.
 //   k_pass2     one read of S: collects median candidates (values in the
 //               median bins), MAD candidates (values not surely inside or
 //               outside the MAD band), counts values surely inside the band,
@@ -197,7 +199,7 @@ cudaError_t launch_maxabs(const float* x, long long n, DevState* st, int sms, cu
 }
 
 // ---------------------------------------------------------------------------
-// Plan: one block of 1024 threads.
+// Plan: what its searches read of the scanned histogram.
 struct PlanCtx {
   const unsigned long long* cum;  // exclusive prefix counts, kNumBins + 1 entries
   BinCfg cfg;
@@ -578,10 +580,10 @@ cudaError_t launch_plan(DevState* st, unsigned long long* hist, int win, const f
 // undecided voxels are staged per warp) and full columns. Columns and stages
 // are flushed with one atomic each.
 //
-// What bounds it: the shared-memory pipe (71 % busy, two of three wavefronts
-// bank conflicts of the lookups) and issue (60 %, 17 instructions a value). With
-// a vote per 32 values and the 20 % of the groups that hold a MAD candidate in
-// the listing path it was issue alone (22.7): 1200 x 1200 x 1024 values took
+// What bounds it: the shared-memory pipe (63 % busy, half of its wavefronts bank
+// conflicts of the lookups) and issue (64 %, 19.5 instructions a value). With a
+// vote per 32 values and the 20 % of the groups that hold a MAD candidate in the
+// listing path it was issue (72 %, 22.4): 1200 x 1200 x 1024 values took
 // 1.10 ms, now 1.06; the read alone is 0.88 at the measured HBM rate. More loads
 // in flight (a cp.async ring in shared memory) cost that pipe more than they
 // gave: 1.27. The columns take what two blocks an SM leave: 8 values a lane

@@ -43,7 +43,7 @@ KINDS = ["normal", "ties", "constant", "offset", "outliers", "nan", "two"]
 
 
 # window sizes around the lane groups (4, 8, 16, 32 voxels), the turns of a
-# plane's rows, windows copied whole (up to 22 voxels a thread) and sampled
+# plane's rows, windows copied whole (up to 20 voxels a thread) and sampled
 # ones, rows longer than 32 voxels, and the largest window
 @pytest.mark.parametrize("window", [(17, 19, 15), (31, 31, 31), (33, 17, 17), (31, 33, 9), (15, 35, 31), (5, 9, 121),
                                     (101, 21, 21), (1, 31, 601), (601, 31, 1)])
